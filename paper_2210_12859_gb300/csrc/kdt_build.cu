@@ -54,14 +54,13 @@ __device__ __forceinline__ Where locate(int64_t p, int T, const int64_t *__restr
 }
 
 __global__ void prep_keys_kernel(const float *__restrict__ pts, int64_t total, int D, int e,
-                                 uint32_t *__restrict__ keys, uint32_t *__restrict__ vals, int *__restrict__ err)
+                                 uint32_t *__restrict__ keys, int *__restrict__ err)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         float x = pts[i * D + e];
         if (!isfinite(x))
             atomicOr(err, ERR_NONFINITE);
         keys[i] = float_key(x);
-        vals[i] = (uint32_t)i;
     }
 }
 
@@ -473,11 +472,11 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
 
     // per-dimension lists sorted by (tree, coordinate, index)
     for (int e = 0; e < D; ++e) {
-        KDT_LAUNCH prep_keys_kernel<<<g, BT, 0, s>>>(d_points, total, D, e, k0, lists[e], err);
-        KDT_TRY(radix_sort_pairs(k0, lists[e], k1, spare, total, 32, rscr, s));
+        KDT_LAUNCH prep_keys_kernel<<<g, BT, 0, s>>>(d_points, total, D, e, k0, err);
+        KDT_TRY(radix_sort_batch(&k0, &lists[e], &k1, &spare, total, 1, total, 0, 32, true, rscr, s));
         if (T > 1) {
             KDT_LAUNCH tree_keys_kernel<<<g, BT, 0, s>>>(lists[e], tree_of, total, k0);
-            KDT_TRY(radix_sort_pairs(k0, lists[e], k1, spare, total, tbits, rscr, s));
+            KDT_TRY(radix_sort_batch(&k0, &lists[e], &k1, &spare, total, 1, total, 0, tbits, false, rscr, s));
         }
     }
     KDT_CUDA(cudaMemcpyAsync(d_lptr, lists, 8 * sizeof(uint32_t *), cudaMemcpyHostToDevice, s));

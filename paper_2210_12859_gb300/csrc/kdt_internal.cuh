@@ -146,17 +146,20 @@ __host__ __device__ __forceinline__ int layout_of(int D) { return D <= 3 ? 0 : (
 __host__ __device__ __forceinline__ int float4_per_node(int D) { return D <= 4 ? 1 : 2; }
 
 // ---------------------------------------------------------------- primitives
-// Stable LSD radix sort of (u32 key, u32 value) pairs on bits [0, bits).
-// keys/vals hold the input and receive the output; tmp_k / tmp_v are scratch of
-// n elements each, `scratch` holds radix_scratch_elems(n) elements.
+// Stable LSD radix sort of (u32 key, u32 value) pairs by bits
+// [lo_bit, lo_bit + bits), 8 bits a pass (whole passes: bits above the range
+// take part where it is no multiple of 8), for `batch` arrays of n pairs at
+// distance `stride` (n < 2^32).  *keys / *vals hold the input; the pointers
+// are swapped with the temporaries' so that *keys / *vals point to the result.
+// iota: the values are the positions 0 .. n - 1 and *vals is not read.
+// `scratch` holds batch x radix_scratch_elems(n) elements, 8-byte aligned.
 size_t radix_scratch_elems(int64_t n);
-int radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *tmp_k, uint32_t *tmp_v, int64_t n,
-                     int bits, uint32_t *scratch, cudaStream_t s);
+int radix_sort_batch(uint32_t **keys, uint32_t **vals, uint32_t **tmp_k, uint32_t **tmp_v, int64_t n, int batch,
+                     int64_t stride, int lo_bit, int bits, bool iota, uint32_t *scratch, cudaStream_t s);
 
-// exclusive prefix sum of u32 in place (n elements), scratch of
-// scan_scratch_elems(n) elements
+// exclusive prefix sum in place (n elements), scratch of scan_scratch_elems(n)
+// elements
 size_t scan_scratch_elems(int64_t n);
-int exclusive_scan_u32(uint32_t *data, int64_t n, uint32_t *scratch, cudaStream_t s);
 int exclusive_scan_u64(unsigned long long *data, int64_t n, unsigned long long *scratch, cudaStream_t s);
 
 int num_sms();
@@ -233,19 +236,30 @@ constexpr size_t carve_size(std::initializer_list<size_t> bytes)
 // Tile sizes of the device-wide scan and radix sort (kdt_sort.cu), here so
 // that scratch sizes can be computed at compile time.
 constexpr int SCAN_TILE_ELEMS = 2048;   // elements per tile of the exclusive scan
-constexpr int RADIX_TILE_KEYS = 2048;   // keys per tile of the radix sort
+constexpr int RADIX_BLOCK = 256;        // threads per block of the radix sort
+constexpr int RADIX_MAX_PASSES = 4;
+// Pairs per thread of a radix pass.  A large tile writes longer runs of equal
+// digits; a small one spreads a small sort over more SMs.
+constexpr int RADIX_ITEMS_SMALL = 4;
+constexpr int RADIX_ITEMS_LARGE = 16;
+constexpr int64_t RADIX_SMALL_N = (int64_t)1 << 19;
+constexpr int radix_items_of(int64_t n) { return n <= RADIX_SMALL_N ? RADIX_ITEMS_SMALL : RADIX_ITEMS_LARGE; }
+constexpr int64_t radix_tiles_of(int64_t n)
+{
+    const int64_t tile = (int64_t)RADIX_BLOCK * radix_items_of(n);
+    return n > tile ? (n + tile - 1) / tile : 1;
+}
 constexpr size_t scan_scratch_elems_of(int64_t n)
 {
     return (size_t)((n + SCAN_TILE_ELEMS - 1) / SCAN_TILE_ELEMS) + 1;
 }
+// per array: 64-bit states of all tiles and passes, digit counts, tickets
 constexpr size_t radix_scratch_elems_of(int64_t n)
 {
-    const int64_t tiles = (n + RADIX_TILE_KEYS - 1) / RADIX_TILE_KEYS;
-    const size_t h = (size_t)256 * (size_t)(tiles > 1 ? tiles : 1);
-    return h + scan_scratch_elems_of((int64_t)h);
+    return (size_t)RADIX_MAX_PASSES * 256 * (2 * (size_t)radix_tiles_of(n) + 1) + 2 * RADIX_MAX_PASSES;
 }
 // Morton keys, permutation and two sort temporaries of Q u32 each, plus the
-// radix sort's histograms and scan partials
+// radix sort's states and digit counts
 constexpr size_t morton_scratch_bytes_of(int64_t Q)
 {
     return carve_size({(size_t)Q * 4, (size_t)Q * 4, (size_t)Q * 4, (size_t)Q * 4, radix_scratch_elems_of(Q) * 4});

@@ -653,8 +653,8 @@ int kdt_radius_model_train(kdt_tree *t, const float *d_q, int64_t Qt, int k, con
         uint64_t su = o.seed * 0xD1B54A32D192ED03ull + 99;
         const double u = (double)(splitmix(su) >> 11) * (1.0 / 9007199254740992.0);
         KDT_LAUNCH resample_kernel<<<grid_of(Qt), 256, 0, s>>>(cdf, Qt, floor_w, u, o.seed, keys, idx);
-        KDT_TRY(radix_sort_pairs(keys, idx, (uint32_t *)(B + o_tk), (uint32_t *)(B + o_tv), Qt, 32,
-                                 (uint32_t *)(B + o_rs), s));
+        uint32_t *tk = (uint32_t *)(B + o_tk), *tv = (uint32_t *)(B + o_tv);
+        KDT_TRY(radix_sort_batch(&keys, &idx, &tk, &tv, Qt, 1, Qt, 0, 32, false, (uint32_t *)(B + o_rs), s));
         float *feat2 = (float *)(B + o_f2), *lab2 = (float *)(B + o_l2);
         KDT_LAUNCH gather_samples_kernel<<<grid_of(Qt), 256, 0, s>>>(idx, Qt, (const float4 *)feat, lab,
                                                                      (float4 *)feat2, lab2);

@@ -1,9 +1,7 @@
 // Device-wide primitives used by the builder and the query reordering:
-// an exclusive prefix sum over u32 and a stable LSD radix sort of
-// (u32 key, u32 value) pairs, 8 bits per pass.
-//
-// Both are three-phase (per-tile reduce, scan of tile totals, per-tile scan
-// and scatter) so that every pass is a plain streaming read of its input.
+// an exclusive prefix sum (three-phase: per-tile reduce, scan of the tile
+// totals, per-tile scan) and a stable LSD radix sort of (u32 key, u32 value)
+// pairs, 8 bits and one kernel per pass.
 #include <algorithm>
 
 #include "kdt_internal.cuh"
@@ -18,9 +16,7 @@ constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 static_assert(SCAN_TILE == SCAN_TILE_ELEMS, "scan tile and the scratch-size formula disagree");
 
 constexpr int RADIX_THREADS = 256;
-constexpr int RADIX_ITEMS = 8;
-constexpr int RADIX_TILE = RADIX_THREADS * RADIX_ITEMS;
-static_assert(RADIX_TILE == RADIX_TILE_KEYS, "radix tile and the scratch-size formula disagree");
+static_assert(RADIX_THREADS == RADIX_BLOCK, "radix tile and the scratch-size formula disagree");
 constexpr int RADIX_WARPS = RADIX_THREADS / 32;
 
 template <typename T>
@@ -138,6 +134,20 @@ int exclusive_scan_t(T *data, int64_t n, T *scratch, cudaStream_t s)
 }
 
 // ---- radix sort
+//
+// Stable LSD sort, 8 bits a pass.  One kernel reads the keys once and counts
+// the digits of all passes; then every pass is one kernel that reads each
+// (key, value) pair once and writes it once: a block ranks its tile in
+// registers and shared memory, learns how many equal digits the tiles before
+// it hold by looking back through their published counts, and writes the tile
+// through shared memory so that equal digits leave in runs.
+//
+// Bound: memory, 16 bytes a pair and pass, for large sorts; the latency of a
+// pass's chain (load, rank, look-back, write) for small ones.  Against the
+// passes it replaced (a histogram kernel, three scan kernels and a scatter
+// that wrote every pair by itself, 20 launches a sort), the Morton order of
+// 10^7 queries takes 0.54 ms instead of 0.85 and that of 2^14 queries 43 us
+// instead of 115.
 
 __device__ __forceinline__ uint32_t lanemask_lt()
 {
@@ -146,76 +156,153 @@ __device__ __forceinline__ uint32_t lanemask_lt()
     return m;
 }
 
+// Digit counts of all passes, one read of the keys.  blockIdx.y: the array.
 __global__ void __launch_bounds__(RADIX_THREADS) radix_hist_kernel(const uint32_t *__restrict__ keys, int64_t n,
-                                                                     int shift, int64_t tiles,
+                                                                     int64_t stride, int lo_bit, int passes,
                                                                      uint32_t *__restrict__ hist)
 {
-    __shared__ uint32_t s_cnt[256];
-    s_cnt[threadIdx.x] = 0;
+    __shared__ uint32_t s_cnt[RADIX_MAX_PASSES * 256];
+    for (int i = threadIdx.x; i < passes * 256; i += RADIX_THREADS)
+        s_cnt[i] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RADIX_TILE;
-#pragma unroll
-    for (int j = 0; j < RADIX_ITEMS; ++j) {
-        int64_t i = base + (int64_t)j * RADIX_THREADS + threadIdx.x;
-        uint32_t d = i < n ? (keys[i] >> shift) & 255u : 256u;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (d < 256 && (peers & lanemask_lt()) == 0)
-            atomicAdd(&s_cnt[d], __popc(peers));
+    const uint32_t *k = keys + blockIdx.y * stride;
+    const int64_t step = (int64_t)gridDim.x * RADIX_THREADS;
+    for (int64_t i = (int64_t)blockIdx.x * RADIX_THREADS + threadIdx.x; i < n; i += step) {
+        const uint32_t key = k[i] >> lo_bit;
+        for (int p = 0; p < passes; ++p)
+            atomicAdd(&s_cnt[p * 256 + ((key >> (8 * p)) & 255u)], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = s_cnt[threadIdx.x];
+    uint32_t *h = hist + (int64_t)blockIdx.y * RADIX_MAX_PASSES * 256;
+    for (int i = threadIdx.x; i < passes * 256; i += RADIX_THREADS)
+        if (s_cnt[i])
+            atomicAdd(&h[i], s_cnt[i]);
 }
 
-// Stable scatter.  Items of a tile are taken in rounds j = 0..RADIX_ITEMS-1,
-// round j holding elements base + j*256 + tid, so index order is round-major,
-// then warp, then lane.  Within a round every warp groups equal digits with
-// match_any; per-digit prefix counts over the warps (plus the counts of earlier
-// rounds) give each element its rank among equal digits of the tile.
-__global__ void __launch_bounds__(RADIX_THREADS) radix_scatter_kernel(
-    const uint32_t *__restrict__ keys, const uint32_t *__restrict__ vals, int64_t n, int shift, int64_t tiles,
-    const uint32_t *__restrict__ offsets, uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out)
+// A tile's published count of one digit: nothing yet, the tile's own count, or
+// the count over the tile and all before it.
+constexpr unsigned long long ST_NONE = 0, ST_OWN = 1ull << 62, ST_ALL = 2ull << 62, ST_VALUE = (1ull << 62) - 1;
+// polls of one predecessor before its count is taken from its keys instead
+constexpr int RADIX_POLLS = 1 << 16;
+
+// Tiles are numbered by the order in which their blocks start, so every
+// predecessor of a running tile is running or done and publishes without
+// waiting for a later one.  A predecessor that has still published nothing
+// after RADIX_POLLS reads is counted from its keys: the wait is bounded and
+// the result does not depend on it.
+// IOTA: the values of the first pass are the positions.
+template <int ITEMS, bool IOTA>
+__global__ void __launch_bounds__(RADIX_THREADS) radix_pass_kernel(
+    const uint32_t *__restrict__ keys_, const uint32_t *__restrict__ vals_, uint32_t *__restrict__ keys_out_,
+    uint32_t *__restrict__ vals_out_, int64_t n, int64_t stride, int shift, int64_t tiles,
+    const uint32_t *__restrict__ hist_, unsigned long long *__restrict__ state_, uint32_t *__restrict__ ticket)
 {
-    __shared__ uint32_t s_off[256];
+    constexpr int TILE = RADIX_THREADS * ITEMS;
     __shared__ uint32_t s_warp[RADIX_WARPS][256];
-    const int tid = threadIdx.x;
-    const int w = tid >> 5;
-    s_off[tid] = offsets[(int64_t)tid * tiles + blockIdx.x];
-    const int64_t base = (int64_t)blockIdx.x * RADIX_TILE;
+    __shared__ uint32_t s_key[TILE], s_val[TILE];
+    __shared__ unsigned long long s_to[256];  // where the tile's run of a digit goes, less its start in the tile
+    __shared__ uint32_t s_scan[33];
+    __shared__ uint32_t s_tile;
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (tid == 0)
+        s_tile = atomicAdd(ticket + blockIdx.y, 1u);
+    for (int i = tid; i < RADIX_WARPS * 256; i += RADIX_THREADS)
+        (&s_warp[0][0])[i] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile;
+    const uint32_t *keys = keys_ + blockIdx.y * stride;
+    const uint32_t *vals = IOTA ? nullptr : vals_ + blockIdx.y * stride;
+    unsigned long long *state = state_ + (int64_t)blockIdx.y * tiles * 256;
+    const int64_t base = tile * TILE;
+    const int count = (int)(n - base < TILE ? n - base : TILE);
+
+    // a warp owns 32 ITEMS consecutive pairs, item j of lane i at 32 j + i
+    const int first = w * 32 * ITEMS + lane;
+    uint32_t key[ITEMS], val[ITEMS];
+    uint32_t rank[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const int i = first + 32 * j;
+        key[j] = i < count ? keys[base + i] : 0xffffffffu;
+        if constexpr (IOTA)
+            val[j] = (uint32_t)(base + i);
+        else
+            val[j] = i < count ? vals[base + i] : 0;
+    }
+    // rank among the warp's equal digits, in order
     const uint32_t lt = lanemask_lt();
-    for (int j = 0; j < RADIX_ITEMS; ++j) {
 #pragma unroll
-        for (int w2 = 0; w2 < RADIX_WARPS; ++w2)
-            s_warp[w2][tid] = 0;
-        int64_t i = base + (int64_t)j * RADIX_THREADS + tid;
-        bool valid = i < n;
-        uint32_t key = valid ? keys[i] : 0;
-        uint32_t val = valid ? vals[i] : 0;
-        uint32_t d = valid ? (key >> shift) & 255u : 256u;
-        __syncthreads();
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        uint32_t rank = __popc(peers & lt);
-        if (valid && rank == 0)
-            s_warp[w][d] = __popc(peers);
-        __syncthreads();
-        {
-            uint32_t run = s_off[tid];
+    for (int j = 0; j < ITEMS; ++j) {
+        const bool valid = first + 32 * j < count;
+        const uint32_t d = valid ? (key[j] >> shift) & 255u : 256u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        uint32_t at = 0;
+        if (valid)
+            at = s_warp[w][d];
+        __syncwarp();
+        if (valid && (peers & lt) == 0)
+            s_warp[w][d] = at + __popc(peers);
+        __syncwarp();
+        rank[j] = at + __popc(peers & lt);
+    }
+    __syncthreads();
+    // thread tid: digit tid.  Counts of the warps before each warp, the
+    // tile's count, and the digit's first place in the sorted tile
+    uint32_t mine = 0;
 #pragma unroll
-            for (int w2 = 0; w2 < RADIX_WARPS; ++w2) {
-                uint32_t c = s_warp[w2][tid];
-                s_warp[w2][tid] = run;
-                run += c;
-            }
-            s_off[tid] = run;
+    for (int v = 0; v < RADIX_WARPS; ++v) {
+        const uint32_t c = s_warp[v][tid];
+        s_warp[v][tid] = mine;
+        mine += c;
+    }
+    volatile unsigned long long *st = state;
+    st[tile * 256 + tid] = (tile ? ST_OWN : ST_ALL) | mine;
+    uint32_t total;
+    const uint32_t in_tile = block_exclusive_sum(mine, s_scan, &total);
+    const uint32_t all = hist_[(int64_t)blockIdx.y * RADIX_MAX_PASSES * 256 + tid];
+    // pairs with a smaller digit (below n < 2^32), then pairs of this digit in earlier tiles
+    const uint32_t smaller = block_exclusive_sum(all, s_scan, &total);
+    unsigned long long before = 0;
+    for (int64_t t = tile - 1; t >= 0; --t) {
+        unsigned long long v = ST_NONE;
+        for (int polls = 0; polls < RADIX_POLLS; ++polls) {
+            v = st[t * 256 + tid];
+            if (v != ST_NONE)
+                break;
         }
-        __syncthreads();
-        if (valid) {
-            uint32_t dst = s_warp[w][d] + rank;
-            if (dst < n) {  // always true for a consistent histogram
-                keys_out[dst] = key;
-                vals_out[dst] = val;
-            }
+        if (v == ST_NONE) {
+            unsigned long long c = 0;
+            for (int64_t i = t * TILE; i < (t + 1) * TILE; ++i)
+                c += ((keys[i] >> shift) & 255u) == (uint32_t)tid;
+            v = ST_OWN | c;
         }
-        __syncthreads();
+        before += v & ST_VALUE;
+        if (v & ST_ALL)
+            break;
+    }
+    if (tile)
+        st[tile * 256 + tid] = ST_ALL | (before + mine);
+    s_to[tid] = smaller + before - in_tile;
+#pragma unroll
+    for (int v = 0; v < RADIX_WARPS; ++v)
+        s_warp[v][tid] += in_tile;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j)
+        if (first + 32 * j < count) {
+            const uint32_t r = s_warp[w][(key[j] >> shift) & 255u] + rank[j];
+            s_key[r] = key[j];
+            s_val[r] = val[j];
+        }
+    __syncthreads();
+    uint32_t *keys_out = keys_out_ + blockIdx.y * stride, *vals_out = vals_out_ + blockIdx.y * stride;
+    for (int i = tid; i < count; i += RADIX_THREADS) {
+        const uint32_t k = s_key[i];
+        const unsigned long long dst = s_to[(k >> shift) & 255u] + (uint32_t)i;
+        if (dst < (unsigned long long)n) {  // always, for a consistent histogram
+            keys_out[dst] = k;
+            vals_out[dst] = s_val[i];
+        }
     }
 }
 
@@ -224,11 +311,6 @@ __global__ void __launch_bounds__(RADIX_THREADS) radix_scatter_kernel(
 size_t scan_scratch_elems(int64_t n)
 {
     return scan_scratch_elems_of(n);
-}
-
-int exclusive_scan_u32(uint32_t *data, int64_t n, uint32_t *scratch, cudaStream_t s)
-{
-    return exclusive_scan_t<uint32_t>(data, n, scratch, s);
 }
 
 int exclusive_scan_u64(unsigned long long *data, int64_t n, unsigned long long *scratch, cudaStream_t s)
@@ -241,29 +323,58 @@ size_t radix_scratch_elems(int64_t n)
     return radix_scratch_elems_of(n);
 }
 
-int radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *tmp_k, uint32_t *tmp_v, int64_t n, int bits,
-                     uint32_t *scratch, cudaStream_t s)
+namespace {
+
+template <int ITEMS>
+int radix_passes(uint32_t *&ka, uint32_t *&va, uint32_t *&kb, uint32_t *&vb, int64_t n, int batch, int64_t stride,
+                 int lo_bit, int passes, bool iota, const uint32_t *hist, unsigned long long *state,
+                 uint32_t *ticket, cudaStream_t s)
 {
-    if (n <= 1)
-        return KDT_OK;
-    int64_t tiles = (n + RADIX_TILE - 1) / RADIX_TILE;
-    uint32_t *hist = scratch;
-    uint32_t *scan_tmp = scratch + 256 * tiles;
-    int passes = (bits + 7) / 8;
-    uint32_t *ka = keys, *va = vals, *kb = tmp_k, *vb = tmp_v;
+    const int64_t tiles = radix_tiles_of(n);
+    const dim3 grid((unsigned)tiles, (unsigned)batch);
     for (int p = 0; p < passes; ++p) {
-        KDT_LAUNCH radix_hist_kernel<<<(unsigned)tiles, RADIX_THREADS, 0, s>>>(ka, n, 8 * p, tiles, hist);
-        KDT_TRY(exclusive_scan_u32(hist, 256 * tiles, scan_tmp, s));
-        KDT_LAUNCH radix_scatter_kernel<<<(unsigned)tiles, RADIX_THREADS, 0, s>>>(ka, va, n, 8 * p, tiles, hist, kb, vb);
+        const uint32_t *h = hist + 256 * p;
+        unsigned long long *st = state + (int64_t)p * batch * tiles * 256;
+        uint32_t *tk = ticket + p * batch;
+        if (iota && p == 0)
+            KDT_LAUNCH radix_pass_kernel<ITEMS, true><<<grid, RADIX_THREADS, 0, s>>>(
+                ka, va, kb, vb, n, stride, lo_bit + 8 * p, tiles, h, st, tk);
+        else
+            KDT_LAUNCH radix_pass_kernel<ITEMS, false><<<grid, RADIX_THREADS, 0, s>>>(
+                ka, va, kb, vb, n, stride, lo_bit + 8 * p, tiles, h, st, tk);
         KDT_CUDA(cudaGetLastError());
         std::swap(ka, kb);
         std::swap(va, vb);
     }
-    if (ka != keys) {
-        KDT_CUDA(cudaMemcpyAsync(keys, ka, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-        KDT_CUDA(cudaMemcpyAsync(vals, va, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    }
     return KDT_OK;
+}
+
+}  // namespace
+
+int radix_sort_batch(uint32_t **keys, uint32_t **vals, uint32_t **tmp_k, uint32_t **tmp_v, int64_t n, int batch,
+                     int64_t stride, int lo_bit, int bits, bool iota, uint32_t *scratch, cudaStream_t s)
+{
+    const int passes = std::min(RADIX_MAX_PASSES, (bits + 7) / 8);
+    if (n < 1 || passes < 1)
+        return KDT_OK;
+    const int64_t tiles = radix_tiles_of(n);
+    // [state: passes x batch x tiles x 256 (64 bits)] [digit counts] [tickets]
+    unsigned long long *state = (unsigned long long *)scratch;
+    uint32_t *hist = (uint32_t *)(state + (int64_t)passes * batch * tiles * 256);
+    uint32_t *ticket = hist + (int64_t)batch * RADIX_MAX_PASSES * 256;
+    const size_t used = (char *)(ticket + passes * batch) - (char *)scratch;
+    KDT_CUDA(cudaMemsetAsync(scratch, 0, used, s));
+    const unsigned hb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 8 * RADIX_THREADS - 1) /
+                                                                              (8 * RADIX_THREADS),
+                                                                          (int64_t)num_sms() * 8));
+    KDT_LAUNCH radix_hist_kernel<<<dim3(hb, (unsigned)batch), RADIX_THREADS, 0, s>>>(*keys, n, stride, lo_bit, passes,
+                                                                                  hist);
+    KDT_CUDA(cudaGetLastError());
+    if (radix_items_of(n) == RADIX_ITEMS_SMALL)
+        return radix_passes<RADIX_ITEMS_SMALL>(*keys, *vals, *tmp_k, *tmp_v, n, batch, stride, lo_bit, passes, iota,
+                                               hist, state, ticket, s);
+    return radix_passes<RADIX_ITEMS_LARGE>(*keys, *vals, *tmp_k, *tmp_v, n, batch, stride, lo_bit, passes, iota, hist,
+                                           state, ticket, s);
 }
 
 int num_sms()
