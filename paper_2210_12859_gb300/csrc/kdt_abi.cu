@@ -10,6 +10,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "kdt_box.cuh"
 #include "kdt_learned.cuh"
 #include "kdt_query.cuh"
 #include "kdt_traverse.cuh"
@@ -288,6 +289,8 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
         a.inline_depth = 1;
     if (flags & (KDT_PLAIN_STEP | KDT_CLOSE_FIRST | KDT_STACK))
         KDT_TRY(launch_ablation(t->layout, a, flags, mode, s));
+    else if (box_query_serves(a, flags, mode))
+        KDT_TRY(launch_box_query(t, a, mode, s));
     else if (simple)
         KDT_TRY(launch_ablation(t->layout, a, KDT_PLAIN_STEP, mode, s));
     else
@@ -391,6 +394,8 @@ __attribute__((visibility("hidden"))) int kdt_tree_alloc_internal(int64_t N, int
     if (e == cudaSuccess && t->layout > 0)
         e = cudaMalloc(&t->ids, (size_t)N * sizeof(int32_t));
     if (e == cudaSuccess)
+        e = box_tree_alloc(t);
+    if (e == cudaSuccess)
         e = cudaMalloc(&t->bbox, 6 * sizeof(float));
     if (e == cudaSuccess)
         e = cudaMalloc(&t->err, sizeof(int));
@@ -445,6 +450,8 @@ int kdt_build_ex(const float *d_points, int64_t N, int D, int opts, void *stream
     int64_t off[2] = {0, N};
     int rc = build_forest(d_points, off, 1, D, t->nodes, t->ids, t->bbox, t->err, s, widest);
     if (rc == KDT_OK)
+        rc = build_box_tree(t, s);
+    if (rc == KDT_OK)
         rc = finish_build(t, opts, s);
     if (rc != KDT_OK) {
         kdt_free(t);
@@ -476,6 +483,7 @@ int kdt_rebuild(kdt_tree *t, const float *d_points, int opts, void *stream)
     }
     int64_t off[2] = {0, t->N};
     KDT_TRY(build_forest(d_points, off, 1, t->D, t->nodes, t->ids, t->bbox, t->err, s, t->layout == 3));
+    KDT_TRY(build_box_tree(t, s));
     return finish_build(t, opts, s);
 }
 
@@ -585,6 +593,7 @@ void kdt_free(kdt_tree *t)
     cudaDeviceSynchronize();
     cudaFree(t->nodes_alloc);
     cudaFree(t->ids);
+    cudaFree(t->box_rec);
     cudaFree(t->bbox);
     cudaFree(t->err);
     cudaFree(t->payload);

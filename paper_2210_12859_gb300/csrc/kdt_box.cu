@@ -1,0 +1,443 @@
+// Build of the box tree and the kNN kernels that walk it (layout in kdt_box.cuh).
+#include <algorithm>
+
+#include "kdt_box.cuh"
+
+namespace kdt {
+
+int grid_for_kernel(const void *fn, int threads, size_t smem);
+
+namespace {
+
+constexpr int BOX_BUILD_THREADS = 256;
+constexpr int BOX_THREADS = 128;
+
+template <int NC>
+struct Box {
+    float lo[NC], hi[NC];
+    __device__ __forceinline__ void none()
+    {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            lo[j] = __int_as_float(0x7f800000);
+            hi[j] = __int_as_float(0xff800000);
+        }
+    }
+    __device__ __forceinline__ void add(const float (&c)[NC])
+    {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            lo[j] = fminf(lo[j], c[j]);
+            hi[j] = fmaxf(hi[j], c[j]);
+        }
+    }
+};
+
+// box of node v into its record
+template <int NC>
+__device__ __forceinline__ void put_box(float4 *rec, uint32_t v, const Box<NC> &b)
+{
+    float *r = reinterpret_cast<float *>(rec + (size_t)(v >> 2) * BoxFormat<NC>::REC) + (v & 3u);
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        r[8 * j] = b.lo[j];
+        r[8 * j + 4] = b.hi[j];
+    }
+}
+
+// The block's boxes (thread i: node v0 + i of one level, `count` of them, a
+// power of two or a multiple of the block) into the records above, four
+// levels up the record tree as far as the block holds whole subtrees.
+template <int NC>
+__device__ __forceinline__ void reduce_boxes(float4 *rec, uint32_t v, int count, Box<NC> b)
+{
+    __shared__ float s_box[BOX_BUILD_THREADS][2 * NC + 1];
+    const int tid = threadIdx.x;
+    for (;;) {
+        if (tid < count && v > 1)
+            put_box<NC>(rec, v, b);
+        if (count < 4)
+            return;
+        __syncthreads();
+        if (tid < count) {
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                s_box[tid][j] = b.lo[j];
+                s_box[tid][NC + j] = b.hi[j];
+            }
+        }
+        __syncthreads();
+        count >>= 2;
+        // thread i takes nodes 4i .. 4i + 3 of the block; v of thread 0 is the first
+        v = (v - tid) / 4 + tid;
+        if (tid < count) {
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                b.lo[j] = fminf(fminf(s_box[4 * tid][j], s_box[4 * tid + 1][j]),
+                                fminf(s_box[4 * tid + 2][j], s_box[4 * tid + 3][j]));
+                b.hi[j] = fmaxf(fmaxf(s_box[4 * tid][NC + j], s_box[4 * tid + 1][NC + j]),
+                                fmaxf(s_box[4 * tid + 2][NC + j], s_box[4 * tid + 3][NC + j]));
+            }
+        }
+    }
+}
+
+// Thread i: bucket i.  Finds the node from above that the bucket holds by
+// walking down from the root, writes the bucket's groups and box, and the
+// block reduces its boxes.  Bound: the gathers of the tree's last four levels
+// (each row of a bucket is contiguous, and neighbouring threads read
+// neighbouring rows) and the latency of the walk, whose upper nodes are shared
+// by the block.
+template <int LAYOUT>
+__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(const float4 *__restrict__ nodes,
+                                                                      const int32_t *__restrict__ ids, int N, int D,
+                                                                      float4 *__restrict__ rec,
+                                                                      float4 *__restrict__ grp)
+{
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    const BoxShape sh(N);
+    const uint32_t first = blockIdx.x * BOX_BUILD_THREADS, i = first + threadIdx.x;
+    const int count = (int)min((int64_t)BOX_BUILD_THREADS, sh.buckets - (int64_t)first);
+    Box<NC> box;
+    box.none();
+    if ((int64_t)i < sh.buckets) {
+        const float nan = __int_as_float(0x7fffffff);
+        // the point handed down to this bucket
+        float hand[NC];
+        uint32_t hand_id = 0xffffffffu;
+        bool held = false;
+        int dim = 0;
+        for (int l = 0; l < sh.LB; ++l) {
+            const int t = (int)(((1u << sh.LB) + i) >> (sh.LB - l)) - 1;
+            const NodeVal<LAYOUT> nd = fetch<LAYOUT, false>(nodes, nullptr, 0, t);
+            const int sd = split_dim_of<LAYOUT>(nd, dim);
+            const bool right = i >> (sh.LB - l - 1) & 1u;
+            const bool to_right = held && select_dim<NC>(hand, sd) > select_dim<NC>(nd.c, sd);
+            if (!held || to_right != right) {
+                // the node's own point: to the other side than the one from
+                // above, or to the left
+                held = held || !right;
+                if (held) {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+                        hand[j] = nd.c[j];
+                    hand_id = LAYOUT == 0 ? nd.id : (LAYOUT == 3 ? nd.id & NODE_ID_MASK : (uint32_t)ids[t]);
+                }
+            }
+            dim = dim + 1 == D ? 0 : dim + 1;
+        }
+        const int root = (1 << sh.LB) - 1 + (int)i;
+        const int groups = (int64_t)i < sh.big ? 2 : 1;
+        float4 *g = grp + (size_t)(i + min((int64_t)i, sh.big)) * BoxFormat<NC>::GRP;
+        for (int k = 0; k < groups; ++k, g += BoxFormat<NC>::GRP) {
+            float c[NC][BOX_GROUP];
+            uint32_t id[BOX_GROUP];
+#pragma unroll
+            for (int m = 0; m < BOX_GROUP; ++m) {
+                // place m of the first group: node 0 .. 6 of the bucket's
+                // first three levels, then the one from above; of the second:
+                // the fourth level's nodes
+                const int up = k ? 3 : (m < 1 ? 0 : (m < 3 ? 1 : 2));
+                const int node = ((root + 1) << up) - 1 + (k ? m : m + 1 - (1 << up));
+                const bool above = k == 0 && m == 7;
+                const bool ok = above ? held : node < N;
+                if (!above && ok) {
+                    const NodeVal<LAYOUT> nd = fetch<LAYOUT, false>(nodes, nullptr, 0, node);
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+                        c[j][m] = nd.c[j];
+                    id[m] = LAYOUT == 0 ? nd.id : (LAYOUT == 3 ? nd.id & NODE_ID_MASK : (uint32_t)ids[node]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+                        c[j][m] = ok ? hand[j] : nan;
+                    id[m] = ok ? hand_id : 0xffffffffu;
+                }
+                // fminf / fmaxf pass over the NaN of an empty place
+#pragma unroll
+                for (int j = 0; j < NC; ++j) {
+                    box.lo[j] = fminf(box.lo[j], c[j][m]);
+                    box.hi[j] = fmaxf(box.hi[j], c[j][m]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                g[2 * j] = make_float4(c[j][0], c[j][1], c[j][2], c[j][3]);
+                g[2 * j + 1] = make_float4(c[j][4], c[j][5], c[j][6], c[j][7]);
+            }
+            uint4 *gi = reinterpret_cast<uint4 *>(g + 2 * NC);
+            gi[0] = make_uint4(id[0], id[1], id[2], id[3]);
+            gi[1] = make_uint4(id[4], id[5], id[6], id[7]);
+        }
+    }
+    if (sh.LB > 0)
+        reduce_boxes<NC>(rec, (uint32_t)sh.buckets + i, count, box);
+}
+
+// Thread i: node v0 + i of a level whose records are complete
+template <int NC>
+__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(float4 *__restrict__ rec, uint32_t v0)
+{
+    const uint32_t first = blockIdx.x * BOX_BUILD_THREADS, i = first + threadIdx.x;
+    const int count = (int)min((uint32_t)BOX_BUILD_THREADS, v0 - first);
+    Box<NC> box;
+    box.none();
+    if (i < v0) {
+        const float4 *r = rec + (size_t)(v0 + i) * BoxFormat<NC>::REC;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const float4 lo = r[2 * j], hi = r[2 * j + 1];
+            box.lo[j] = fminf(fminf(lo.x, lo.y), fminf(lo.z, lo.w));
+            box.hi[j] = fmaxf(fmaxf(hi.x, hi.y), fmaxf(hi.z, hi.w));
+        }
+    }
+    reduce_boxes<NC>(rec, v0 + i, count, box);
+}
+
+// ---- kNN
+//
+// Persistent lanes, a query each, as in the state machine's kernel; a warp
+// alternates between records (while more than BOX_RECORD_LANES of its lanes
+// are on one) and the buckets that its lanes have reached, and takes new
+// queries when BOX_FREE_LANES lanes are free.  Both are sweet spots of a sweep
+// on all kNN cases (records 0 / 4 / 8 / 16 / 24, free 1 / 4 / 8 / 16 / 24): a
+// bucket costs several records, so few lanes should be kept from it, and the
+// claim, the row's store and the new query's first bucket run best with most
+// lanes taking part (free 8 -> 24: surface k = 16 4.17 -> 3.78 ms, closest
+// point in 4-D 6.81 -> 6.58 ms).
+//
+// Bound: the arithmetic and selects of buckets and lists in 3-D with k >= 8
+// (issue slots 59 %, the ALU pipe 90 % busy), L1 wavefronts in 4-D and above
+// with incoherent queries (98 %).  Against the state machine's kernel: clustered
+// 2^24, k = 8 1040 -> 18.5 ms (13.3 k processed nodes a query -> 56 records and
+// 14 buckets), surface 2^22, k = 16 10.2 -> 3.8 ms, 8-D k = 10 23.3 -> 5.4 ms,
+// 10^7 closest points in 4-D 8.8 -> 6.6 ms, a scan of 5003 closest points
+// 45 -> 25 us.  The state machine is not faster on any of them.
+constexpr int BOX_RECORD_LANES = 4;
+constexpr int BOX_FREE_LANES = 24;
+
+template <int LAYOUT, int K, int MODE>
+__global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(const QueryArgs a, const BoxArgs b)
+{
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    using List = typename std::conditional<(K <= MAX_REG_K), RegList<K <= MAX_REG_K ? K : 1>, SmemList>::type;
+    extern __shared__ float4 s_dyn[];
+    const int64_t ngate = (MODE == MODE_BOUNDED && a.n_gate) ? (int64_t)*a.n_gate : INT64_MAX;
+    const uint32_t cap = a.step_cap ? a.step_cap : 3u * (uint32_t)a.N + 3u;
+    bool gated = false;
+    double ratio = 0.0;
+    float q[NC];
+    float r2 = 0.f;
+    List list;
+    float *const s_far = reinterpret_cast<float *>(s_dyn) + threadIdx.x;
+    const int stride = blockDim.x;
+    const f32x2 one = pair(b.one, b.one);
+    if constexpr (K > MAX_REG_K) {
+        if (a.heap) {
+            list.s = a.heap + ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * (size_t)a.k;
+            list.stride = 1;
+        } else {
+            list.s = reinterpret_cast<unsigned long long *>(s_dyn) + BoxWalk::MAX_RECORDS / 2 * stride + threadIdx.x;
+            list.stride = stride;
+        }
+    }
+    BoxWalk w;
+    w.v = 0;
+    uint32_t steps = 0;
+    // the first query of a lane is its place in the grid, the next ones are claimed
+    int64_t qi = -1;
+    bool busy = false, first = true, exhausted = false;
+    const int64_t lanes = (int64_t)gridDim.x * blockDim.x;
+    for (;;) {
+        const unsigned free_lanes = __ballot_sync(0xffffffffu, !busy && !exhausted);
+        const unsigned busy_lanes = __ballot_sync(0xffffffffu, busy);
+        if (!busy_lanes || __popc(free_lanes) >= BOX_FREE_LANES) {
+            // write the finished rows, take the next queries
+            if (!busy && qi >= 0) {
+                bool again = false;
+                if constexpr (MODE == MODE_BOUNDED) {
+                    const bool full = list.full(a.k);
+                    // exact when the list is full or the proposal did not
+                    // shrink the radius; else once more with the caller's
+                    again = steps <= cap && !(full || r2 == a.r2);
+                    if (again) {
+                        atomicAdd(a.fb_count, 1ull);
+                        gated = false;
+                        r2 = a.r2;
+                        list.init(a.k, r2);
+                        w.start(b.root, b.root_mask, s_far);
+                        steps = 0;
+                        busy = true;
+                    } else if (gated && full && list.cull() > 0.f && r2 < __int_as_float(0x7f800000)) {
+                        ratio += sqrt((double)r2 / (double)list.cull());
+                    }
+                }
+                if (!again) {
+                    if (steps > cap)
+                        atomicOr(a.err, ERR_TRAVERSAL);
+                    list.store(a.k, a.out_ids + qi * a.k, a.out_d2 + qi * a.k);
+                    qi = -1;
+                }
+            }
+            const bool need = !busy && !exhausted;
+            int64_t slot;
+            if (first)
+                slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+            else if (lanes >= a.Q)
+                slot = a.Q;
+            else
+                slot = claim_slot(need, a.counter);
+            if (need) {
+                if (!first && slot < a.Q)
+                    slot += lanes;
+                if (slot < a.Q) {
+                    qi = a.perm ? (int64_t)a.perm[slot] : slot;
+                    gated = MODE == MODE_BOUNDED && slot < ngate;
+                    r2 = gated ? a.r2q[qi] : a.r2;
+                    load_query<LAYOUT>(a.queries, qi, a.D, q);
+                    list.init(a.k, r2);
+                    w.start(b.root, b.root_mask, s_far);
+                    steps = 0;
+                    // no distance to a NaN query passes a test
+                    bool nan = false;
+#pragma unroll
+                    for (int j = 0; j < NC; ++j)
+                        nan = nan || q[j] != q[j];
+                    busy = !nan;
+                } else {
+                    exhausted = true;
+                }
+            }
+            first = false;
+            if (__all_sync(0xffffffffu, !busy && exhausted && qi < 0))
+                break;
+        }
+        // records, until few lanes are left on them
+        for (;;) {
+            if (busy && w.v < b.leaf) {
+                ++steps;
+                busy = w.template step<NC>(b.rec, q, one, list.cull(), stride);
+            }
+            if (__popc(__ballot_sync(0xffffffffu, busy && w.v < b.leaf)) <= BOX_RECORD_LANES)
+                break;
+        }
+        if (busy && w.v >= b.leaf) {
+            ++steps;
+            box_bucket<NC>(b, w.v - b.leaf, q, one, list);
+            busy = w.pop(list.cull(), stride);
+        }
+        if (steps > cap)
+            busy = false;
+    }
+    if (MODE == MODE_BOUNDED) {
+        for (int o = 16; o > 0; o >>= 1)
+            ratio += __shfl_down_sync(0xffffffffu, ratio, o);
+        if ((threadIdx.x & 31) == 0 && ratio != 0.0)
+            atomicAdd(a.ratio_sum, ratio);
+    }
+}
+
+template <int LAYOUT, int K, int MODE>
+int launch_box_one(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
+{
+    const void *fn = (const void *)box_knn_kernel<LAYOUT, K, MODE>;
+    // few queries: small blocks, so that they spread over the SMs
+    int threads = BOX_THREADS;
+    while (threads > 32 && a.Q < (int64_t)num_sms() * threads)
+        threads >>= 1;
+    const size_t smem = (size_t)threads * (4 * BoxWalk::MAX_RECORDS + (K > MAX_REG_K && !a.heap ? 8 * a.k : 0));
+    if (smem > 48 * 1024)
+        KDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int64_t grid = grid_for_kernel(fn, threads, smem);
+    if (a.heap)
+        grid = std::max<int64_t>(1, std::min<int64_t>(grid, a.heap_threads / threads));
+    grid = std::min<int64_t>(grid, (a.Q + threads - 1) / threads);
+    if (grid * threads < a.Q)
+        KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
+    KDT_LAUNCH box_knn_kernel<LAYOUT, K, MODE><<<(unsigned)grid, threads, smem, s>>>(a, b);
+    KDT_CUDA(cudaGetLastError());
+    return KDT_OK;
+}
+
+template <int LAYOUT, int MODE>
+int launch_box_k(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
+{
+    if (a.k <= 1)
+        return launch_box_one<LAYOUT, 1, MODE>(a, b, s);
+    if (a.k <= 2)
+        return launch_box_one<LAYOUT, 2, MODE>(a, b, s);
+    if (a.k <= 4)
+        return launch_box_one<LAYOUT, 4, MODE>(a, b, s);
+    if (a.k <= 8)
+        return launch_box_one<LAYOUT, 8, MODE>(a, b, s);
+    if (a.k <= 16)
+        return launch_box_one<LAYOUT, 16, MODE>(a, b, s);
+    return launch_box_one<LAYOUT, 64, MODE>(a, b, s);
+}
+
+template <int LAYOUT>
+int build_box_layout(const kdt_tree *t, cudaStream_t s)
+{
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    const BoxShape sh(t->N);
+    KDT_LAUNCH box_leaf_kernel<LAYOUT><<<(unsigned)((sh.buckets + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS),
+                                         BOX_BUILD_THREADS, 0, s>>>(t->nodes, t->ids, (int)t->N, t->D, t->box_rec,
+                                                                     t->box_grp);
+    KDT_CUDA(cudaGetLastError());
+    // a block writes the boxes of five levels of the record tree (256 nodes
+    // and their 64, 16, 4 and 1 ancestors), the next launch starts above them
+    for (int l = sh.LB - 10; l >= 1; l -= 10) {
+        const uint32_t v0 = 1u << l;
+        KDT_LAUNCH box_upper_kernel<NC><<<(v0 + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS, BOX_BUILD_THREADS, 0,
+                                          s>>>(t->box_rec, v0);
+        KDT_CUDA(cudaGetLastError());
+    }
+    return KDT_OK;
+}
+
+}  // namespace
+
+cudaError_t box_tree_alloc(kdt_tree *t)
+{
+    const BoxShape sh(t->N);
+    const size_t rec = (size_t)sh.records() * 2 * box_coords(t->D);
+    const size_t grp = (size_t)sh.groups() * 2 * (box_coords(t->D) + 1);
+    // a group starts on a 128-byte line where its size allows (records of 96
+    // bytes: rounded up to a line)
+    const size_t at = (rec + 7) & ~(size_t)7;
+    const cudaError_t e = cudaMalloc(&t->box_rec, (at + grp) * sizeof(float4));
+    t->box_grp = t->box_rec + at;
+    return e;
+}
+
+int build_box_tree(const kdt_tree *t, cudaStream_t s)
+{
+    switch (t->layout) {
+    case 0: return build_box_layout<0>(t, s);
+    case 1: return build_box_layout<1>(t, s);
+    case 3: return build_box_layout<3>(t, s);
+    default: return build_box_layout<2>(t, s);
+    }
+}
+
+int launch_box_query(const kdt_tree *t, const QueryArgs &a, int mode, cudaStream_t s)
+{
+    const BoxShape sh(t->N);
+    BoxArgs b;
+    b.rec = t->box_rec;
+    b.grp = t->box_grp;
+    b.leaf = (uint32_t)sh.buckets;
+    b.big = (uint32_t)sh.big;
+    b.root = sh.LB & 1 ? 0u : 1u;
+    b.root_mask = sh.LB & 1 ? 12u : 15u;
+    const bool bounded = mode == MODE_BOUNDED;
+    // the groups hold coordinates and ids alike for layouts 0 and 3
+    switch (t->layout) {
+    case 0:
+    case 3: return bounded ? launch_box_k<0, MODE_BOUNDED>(a, b, s) : launch_box_k<0, MODE_RESULTS>(a, b, s);
+    case 1: return launch_box_k<1, MODE_RESULTS>(a, b, s);
+    default: return launch_box_k<2, MODE_RESULTS>(a, b, s);
+    }
+}
+
+}  // namespace kdt

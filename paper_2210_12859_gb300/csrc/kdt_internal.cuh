@@ -296,6 +296,8 @@ struct kdt_tree {
     float4 *nodes_alloc = nullptr; // allocation; 16-byte nodes start one slot in, so that the siblings
                                    // 2c+1 and 2c+2 share one 32-byte sector
     int32_t *ids = nullptr;        // layout > 0
+    float4 *box_rec = nullptr;     // box tree of the result queries (kdt_box.cuh): records,
+    float4 *box_grp = nullptr;     // and point groups (in the records' allocation)
     float *bbox = nullptr;         // device [2][3]: lo, hi of the first min(D,3) dims
     int *err = nullptr;            // device error word
     kdt::Model model;

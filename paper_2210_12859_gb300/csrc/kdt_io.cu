@@ -12,6 +12,7 @@
 
 #include <vector>
 
+#include "kdt_box.cuh"
 #include "kdt_query.cuh"
 
 namespace kdt {
@@ -194,6 +195,8 @@ int kdt_tree_load(const char *path, void *stream, kdt_tree **out)
         unsigned g = (unsigned)std::min<int64_t>((N + 255) / 256, (int64_t)num_sms() * 16);
         KDT_LAUNCH import_kernel<<<g, 256, 0, s>>>(d_coords, d_ids, d_dims, N, D, t->nodes, t->ids);
         e = cudaGetLastError();
+        if (e == cudaSuccess && build_box_tree(t, s) != KDT_OK)
+            e = cudaErrorUnknown;
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(s);
     }

@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "kdt_box.cuh"
 #include "kdt_learned.cuh"
 #include "kdt_query.cuh"
 
@@ -375,8 +376,9 @@ int run_learned_query(kdt_tree *t, const float *d_q, int64_t Q, int k, float r2,
     a.fb_count = (unsigned long long *)t->stats;
     a.ratio_sum = (double *)(t->stats + 1);
     const bool ordered = !(flags & KDT_UNORDERED);
-    KDT_TRY(launch_query(t->layout, a, ordered, MODE_BOUNDED, false, s));
-    return KDT_OK;
+    if (box_query_serves(a, flags, MODE_BOUNDED))
+        return launch_box_query(t, a, MODE_BOUNDED, s);
+    return launch_query(t->layout, a, ordered, MODE_BOUNDED, false, s);
 }
 
 // The automatic gate, from the training queries: the processed nodes the

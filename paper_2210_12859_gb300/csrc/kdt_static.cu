@@ -14,6 +14,7 @@
 // work counter) and overwrites the rest before reading it.  Two calls whose
 // work overlaps on the GPU (different streams, or host threads racing) use
 // the same bytes and race; serialise them.
+#include "kdt_box.cuh"
 #include "kdt_query.cuh"
 
 namespace kdt {
@@ -98,5 +99,7 @@ extern "C" int kdt_knn_static(const kdt_tree *t, const float *d_q, int64_t Q, in
     a.light_run = light_run_for(t, k);
     a.step_cap = t->debug_step_cap;
     a.inline_depth = inline_depth_for(t, k) >= 2 ? inline_depth_for(t, k) : 1;  // depth 0 is plain-query only
+    if (box_query_serves(a, flags, MODE_RESULTS))
+        return launch_box_query(t, a, MODE_RESULTS, s);
     return launch_query(t->layout, a, !(flags & KDT_UNORDERED), MODE_RESULTS, false, s);
 }
