@@ -73,7 +73,7 @@ bool debug_alloc_fails()
     return false;
 }
 
-// ---------------------------------------------------------------- Morton order
+// ---------------------------------------------------------------- query order
 
 __device__ __forceinline__ uint32_t spread3(uint32_t x)
 {
@@ -85,30 +85,82 @@ __device__ __forceinline__ uint32_t spread3(uint32_t x)
     return x;
 }
 
-// 30-bit Morton code of the first min(D,3) coordinates quantised to 10 bits
-// inside the bounding box of the query's tree.  With `nodes` (a single tree
-// of D <= 3), the key is a 5-bit cost class above a 27-bit Morton code (9 bits
-// per coordinate), most expensive class first: a query whose greedy descent
-// ends far from its leaf point, relative to the tree's mean point spacing,
-// lies outside the data and processes many nodes, more the farther it ends.
-// With r = d2(leaf) / spacing^2, queries with r > 64 are classed by
-// floor(log2 r) (larger first), the others in three classes (r > 8, r > 1,
-// the rest).  Starting the longest queries first keeps them out of the end of
-// the launch, where too few lanes are left to hide their latency.
-// With T > 1 trees the key is the tree's index (tbits bits) above the code's
-// high 32 - tbits bits, so one sort orders by tree and by code within a tree.
+// Forests: the tree's index (tbits bits) above the high 32 - tbits bits of the
+// query's 30-bit Morton code (its first min(D, 3) coordinates, 10 bits each
+// inside the bounding box of the query's tree), so that one sort orders by
+// tree and along the curve within a tree.
 __global__ void morton_kernel(const float *__restrict__ qs, int64_t Q, int D, const float *__restrict__ bbox, int T,
-                              int tbits, const int64_t *__restrict__ q_off, const float4 *__restrict__ nodes,
-                              int64_t N, bool stored, uint32_t *__restrict__ keys,
-                              unsigned long long *__restrict__ n_far)
+                              int tbits, const int64_t *__restrict__ q_off, uint32_t *__restrict__ keys)
 {
-    float spacing2 = 0.f;
-    if (nodes) {
-        float vol = 1.f;
-        for (int j = 0; j < D; ++j)
-            vol *= fmaxf(bbox[3 + j] - bbox[j], 1e-30f);
-        spacing2 = powf(vol / (float)N, 2.f / (float)D);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x) {
+        int t = 0;
+        int lo = 0, hi = T - 1;
+        while (lo < hi) {
+            int mid = (lo + hi + 1) >> 1;
+            if (q_off[mid] <= i)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        t = lo;
+        const float *bb = bbox + 6 * t;
+        uint32_t code = 0;
+        for (int j = 0; j < 3 && j < D; ++j) {
+            float ext = bb[3 + j] - bb[j];
+            float x = ext > 0.f ? (qs[i * D + j] - bb[j]) / ext : 0.f;
+            x = fminf(fmaxf(x, 0.f), 1.f);
+            uint32_t c = (uint32_t)fminf(x * 1024.f, 1023.f);
+            code |= spread3(c) << (2 - j);
+        }
+        keys[i] = (uint32_t)((((uint64_t)t << 32) | ((uint64_t)code << 2)) >> tbits);
     }
+}
+
+// Single trees: the path of the query's descent from the root, a bit a level,
+// over `levels` full levels.  Queries in this order share the nodes of their
+// walks for as many levels as the order resolves, whatever the points'
+// density and dimensions: a Morton code cuts the space on planes of its own
+// and sees three coordinates.  One dependent 4-byte load a level, the upper
+// levels from L1.
+// LAYOUT as in kdt_internal.cuh.
+template <int LAYOUT>
+__global__ void path_kernel(const float *__restrict__ qs, int64_t Q, int D, const float4 *__restrict__ nodes,
+                            int levels, uint32_t *__restrict__ keys)
+{
+    constexpr int STRIDE = LAYOUT == 2 ? 8 : 4;
+    const float *c = reinterpret_cast<const float *>(nodes);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t v = 1;  // node + 1
+        int dim = 0;
+        for (int l = 0; l < levels; ++l) {
+            const size_t at = (size_t)(v - 1) * STRIDE;
+            if (LAYOUT == 3)
+                dim = (int)(__float_as_uint(__ldg(c + at + 3)) >> NODE_DIM_SHIFT);
+            const bool right = __ldg(qs + i * D + dim) > __ldg(c + at + dim);
+            v = 2 * v + right;
+            if (LAYOUT != 3)
+                dim = dim + 1 == D ? 0 : dim + 1;
+        }
+        keys[i] = v - (1u << levels);
+    }
+}
+
+// KDT_COST_ORDER (D <= 3): a 5-bit cost class above 27 bits of the path, most
+// expensive class first: a query whose greedy descent ends far from its leaf
+// point, relative to the tree's mean point spacing, lies outside the data and
+// processes many nodes, more the farther it ends.  With r = d2(leaf) /
+// spacing^2, queries with r > 64 are classed by floor(log2 r) (larger first),
+// the others in three classes (r > 8, r > 1, the rest).  Starting the longest
+// queries first keeps them out of the end of the launch, where too few lanes
+// are left to hide their latency.
+__global__ void cost_path_kernel(const float *__restrict__ qs, int64_t Q, int D, const float *__restrict__ bbox,
+                                 const float4 *__restrict__ nodes, int64_t N, bool stored,
+                                 uint32_t *__restrict__ keys, unsigned long long *__restrict__ n_far)
+{
+    float vol = 1.f;
+    for (int j = 0; j < D; ++j)
+        vol *= fmaxf(bbox[3 + j] - bbox[j], 1e-30f);
+    const float spacing2 = powf(vol / (float)N, 2.f / (float)D);
     // every thread of the grid runs the same number of iterations, so the
     // warp vote that counts far queries sees full warps
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -117,43 +169,22 @@ __global__ void morton_kernel(const float *__restrict__ qs, int64_t Q, int D, co
         const int64_t i = it * stride + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
         bool far = false;
         if (i < Q) {
-            int t = 0;
-            if (T > 1) {
-                int lo = 0, hi = T - 1;
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (q_off[mid] <= i)
-                        lo = mid;
-                    else
-                        hi = mid - 1;
-                }
-                t = lo;
+            float q[3];
+            load_query<0>(qs, i, D, q);
+            uint32_t leaf;
+            const float r = descent_leaf_d2(nodes, nullptr, 0, (int)N, D, q, stored, &leaf) / spacing2;
+            uint32_t cls;
+            if (r > 64.f) {  // floor(log2 r) >= 6: classes 28 (r < 128) down to 0
+                const int e = ilogbf(r);
+                cls = (uint32_t)(28 - min(e - 6, 28));
+                far = true;
+            } else {
+                cls = r > 8.f ? 29u : (r > 1.f ? 30u : 31u);  // NaN: 31
             }
-            const float *bb = bbox + 6 * t;
-            uint32_t code = 0;
-            const float cells = nodes ? 512.f : 1024.f;
-            for (int j = 0; j < 3 && j < D; ++j) {
-                float ext = bb[3 + j] - bb[j];
-                float x = ext > 0.f ? (qs[i * D + j] - bb[j]) / ext : 0.f;
-                x = fminf(fmaxf(x, 0.f), 1.f);
-                uint32_t c = (uint32_t)fminf(x * cells, cells - 1.f);
-                code |= spread3(c) << (2 - j);
-            }
-            if (nodes) {
-                float q[3];
-                load_query<0>(qs, i, D, q);
-                const float r = descent_leaf_d2(nodes, nullptr, 0, (int)N, D, q, stored) / spacing2;
-                uint32_t cls;
-                if (r > 64.f) {  // floor(log2 r) >= 6: classes 28 (r < 128) down to 0
-                    const int e = ilogbf(r);
-                    cls = (uint32_t)(28 - min(e - 6, 28));
-                    far = true;
-                } else {
-                    cls = r > 8.f ? 29u : (r > 1.f ? 30u : 31u);  // NaN: 31
-                }
-                code |= cls << 27;
-            }
-            keys[i] = T > 1 ? (uint32_t)((((uint64_t)t << 32) | ((uint64_t)code << 2)) >> tbits) : code;
+            // leaf + 1 in binary is a 1 and the path; the path's first bit to bit 26
+            const int l = 31 - __clz(leaf + 1);
+            const uint32_t path = leaf + 1 - (1u << l);
+            keys[i] = cls << 27 | (l <= 27 ? path << (27 - l) : path >> (l - 27));
         }
         if (n_far) {
             const unsigned m = __ballot_sync(0xffffffffu, far);
@@ -174,41 +205,75 @@ size_t morton_scratch_bytes(int64_t Q)
     return morton_scratch_bytes_of(Q);
 }
 
-// Bits of the key that the order needs, from the top: past sixteen Morton
-// cells a query, further bits only split cells that hold one query or none
-// (the order changes nothing but the speed).  The head bits (tree, cost
-// class) count in full; with fewer than three coordinates the code has fewer
-// bits that vary.  Each pass saved of a small sort is about 8 us (2^14
-// queries: 24 bits, three passes, 43 us for the whole order).
-static int order_bits(int64_t Q, int D, int head, int total)
-{
-    const int dims = std::min(D, 3);
-    const int code = ((floor_log2((uint64_t)Q) + 4) * 3 + dims - 1) / dims;
-    return std::min(total, (head + code + 7) / 8 * 8);
-}
+// Bits below the head (tree, cost class) that an order of Q queries needs:
+// with a cell for every four queries, further bits hardly move a warp's work
+// (measured from 1/4 to 32 cells a query: within 1 %; the order changes nothing
+// but the speed), while each pass of 8 bits
+// saved of a small sort is about 8 us (photon gather of 2^18 167 -> 152 us).
+static int path_bits(int64_t Q) { return std::max(floor_log2((uint64_t)std::max<int64_t>(Q, 1)) - 2, 1); }
 
-// permutation of the queries along the Morton curve (stable: equal codes keep
-// their index order); perm receives traversal order -> query index
-int morton_order(const float *d_q, int64_t Q, int D, const float *bbox, int T, const int64_t *d_qoff, int tbits,
-                 const float4 *nodes, int64_t N, bool stored, void *scratch, uint32_t **perm_out, cudaStream_t s,
-                 unsigned long long *n_far)
+struct OrderArrays {
+    uint32_t *keys, *perm, *tk, *tv, *rs;
+    OrderArrays(void *scratch, int64_t Q)
+    {
+        Carve c{(char *)scratch};
+        keys = c.take<uint32_t>(Q);
+        perm = c.take<uint32_t>(Q);
+        tk = c.take<uint32_t>(Q);
+        tv = c.take<uint32_t>(Q);
+        rs = c.take<uint32_t>(radix_scratch_elems(Q));
+    }
+};
+
+// permutation of the queries by their paths in the tree (stable: equal paths
+// keep their index order); perm receives traversal order -> query index
+int query_order(const kdt_tree *t, const float *d_q, int64_t Q, bool cost, void *scratch, uint32_t **perm_out,
+                cudaStream_t s, unsigned long long *n_far)
 {
-    Carve c{(char *)scratch};
-    uint32_t *keys = c.take<uint32_t>(Q);
-    uint32_t *perm = c.take<uint32_t>(Q);
-    uint32_t *tk = c.take<uint32_t>(Q);
-    uint32_t *tv = c.take<uint32_t>(Q);
-    uint32_t *rs = c.take<uint32_t>(radix_scratch_elems(Q));
-    const bool cost = nodes && D <= 3 && T == 1;
+    OrderArrays o(scratch, Q);
+    cost = cost && t->D <= 3;
     if (n_far)
         KDT_CUDA(cudaMemsetAsync(n_far, 0, sizeof(unsigned long long), s));
-    KDT_LAUNCH morton_kernel<<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, bbox, T, tbits, d_qoff, cost ? nodes : nullptr, N,
-                                                        stored, keys, cost ? n_far : nullptr);
+    int lo, bits;
+    if (cost) {
+        KDT_LAUNCH cost_path_kernel<<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->bbox, t->nodes, t->N, t->layout == 3,
+                                                               o.keys, n_far);
+        bits = std::min(32, (5 + path_bits(Q) + 7) / 8 * 8);
+        lo = 32 - bits;
+    } else {
+        // the levels above the last are full
+        const int levels = std::min(floor_log2((uint64_t)t->N), path_bits(Q));
+        switch (t->layout) {
+        case 0: KDT_LAUNCH path_kernel<0><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
+        case 1: KDT_LAUNCH path_kernel<1><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
+        case 3: KDT_LAUNCH path_kernel<3><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
+        default: KDT_LAUNCH path_kernel<2><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys);
+        }
+        bits = std::max(levels, 1);
+        lo = 0;
+    }
     KDT_CUDA(cudaGetLastError());
-    const int total = cost || T > 1 ? 32 : 30;
-    const int bits = order_bits(T > 1 ? std::max<int64_t>(Q / T, 1) : Q, D, T > 1 ? tbits : (cost ? 5 : 0), total);
-    KDT_TRY(radix_sort_batch(&keys, &perm, &tk, &tv, Q, 1, Q, total - bits, bits, true, rs, s));
-    *perm_out = perm;
+    KDT_TRY(radix_sort_batch(&o.keys, &o.perm, &o.tk, &o.tv, Q, 1, Q, lo, bits, true, o.rs, s));
+    *perm_out = o.perm;
+    return KDT_OK;
+}
+
+// the same for a forest's queries: by tree, along the Morton curve within one
+static int forest_order(const kdt_forest *f, const float *d_q, int64_t Q, const int64_t *d_qoff, void *scratch,
+                        uint32_t **perm_out, cudaStream_t s)
+{
+    OrderArrays o(scratch, Q);
+    const int T = f->f.T, D = f->f.D;
+    const int tbits = T > 1 ? floor_log2((uint64_t)(T - 1)) + 1 : 0;
+    KDT_LAUNCH morton_kernel<<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, f->bbox, T, tbits, d_qoff, o.keys);
+    KDT_CUDA(cudaGetLastError());
+    // a Morton code wastes bits on empty space and, with fewer than three
+    // coordinates, on those missing
+    const int dims = std::min(D, 3);
+    const int code = ((path_bits(Q / T) + 2) * 3 + dims - 1) / dims;
+    const int bits = std::min(32, (tbits + code + 7) / 8 * 8);
+    KDT_TRY(radix_sort_batch(&o.keys, &o.perm, &o.tk, &o.tv, Q, 1, Q, 32 - bits, bits, true, o.rs, s));
+    *perm_out = o.perm;
     return KDT_OK;
 }
 
@@ -259,9 +324,7 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
     }
     a.group = list_group_for(t, k);
     if (morton)
-        KDT_TRY(morton_order(d_q, Q, t->D, t->bbox, 1, nullptr, 0, (flags & KDT_COST_ORDER) ? t->nodes : nullptr,
-                             t->N, t->layout == 3, c.base + c.off, const_cast<uint32_t **>(&a.perm),
-                             s));
+        KDT_TRY(query_order(t, d_q, Q, flags & KDT_COST_ORDER, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
     a.nodes = t->nodes;
     a.ids = t->ids;
     a.N = (int)t->N;
@@ -796,11 +859,8 @@ static int forest_enqueue(kdt_forest *f, ForestGraph *g, const float *d_q, int64
     unsigned long long *counter = c.take<unsigned long long>(8);
     c.take<int64_t>(T + 1);  // query offsets (filled before)
     QueryArgs a;
-    if (flags & KDT_MORTON) {
-        int tbits = T > 1 ? floor_log2((uint64_t)(T - 1)) + 1 : 0;
-        KDT_TRY(morton_order(d_q, Q, f->f.D, f->bbox, T, d_qoff, tbits, nullptr, 0, false, c.base + c.off,
-                             const_cast<uint32_t **>(&a.perm), s));
-    }
+    if (flags & KDT_MORTON)
+        KDT_TRY(forest_order(f, d_q, Q, d_qoff, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
     a.nodes = f->nodes;
     a.ids = f->ids;
     a.D = f->f.D;

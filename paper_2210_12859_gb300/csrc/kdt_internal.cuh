@@ -164,12 +164,6 @@ int exclusive_scan_u64(unsigned long long *data, int64_t n, unsigned long long *
 
 int num_sms();
 
-// permutation of queries along the Morton curve (traversal order -> query index);
-// with cost classes (nodes given), n_far (device, may be NULL) receives the
-// number of queries in the far classes, which come first in the permutation
-int morton_order(const float *d_q, int64_t Q, int D, const float *bbox, int T, const int64_t *d_qoff, int tbits,
-                 const float4 *nodes, int64_t N, bool stored, void *scratch, uint32_t **perm_out, cudaStream_t s,
-                 unsigned long long *n_far = nullptr);
 size_t morton_scratch_bytes(int64_t Q);
 
 // ---------------------------------------------------------------- scratch
@@ -258,7 +252,7 @@ constexpr size_t radix_scratch_elems_of(int64_t n)
 {
     return (size_t)RADIX_MAX_PASSES * 256 * (2 * (size_t)radix_tiles_of(n) + 1) + 2 * RADIX_MAX_PASSES;
 }
-// Morton keys, permutation and two sort temporaries of Q u32 each, plus the
+// Order keys, permutation and two sort temporaries of Q u32 each, plus the
 // radix sort's states and digit counts
 constexpr size_t morton_scratch_bytes_of(int64_t Q)
 {
@@ -348,6 +342,12 @@ struct kdt_forest {
 extern "C" int kdt_tree_alloc_internal(int64_t N, int D, kdt_tree **out);
 
 namespace kdt {
+// permutation of a tree's queries by the path of their descent (traversal
+// order -> query index); with cost, by cost class first (D <= 3), and n_far
+// (device, may be NULL) then receives the number of queries in the far
+// classes, which come first in the permutation.  scratch: morton_scratch_bytes(Q)
+int query_order(const kdt_tree *t, const float *d_q, int64_t Q, bool cost, void *scratch, uint32_t **perm_out,
+                cudaStream_t s, unsigned long long *n_far = nullptr);
 // staging depth (levels) for a query on tree t with k neighbours: the tree's
 // own setting, else the tuned value for its shape, else the default
 int stage_levels_for(const kdt_tree *t, int k);

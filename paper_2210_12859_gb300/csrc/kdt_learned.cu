@@ -340,8 +340,7 @@ int run_learned_query(kdt_tree *t, const float *d_q, int64_t Q, int k, float r2,
     float *r2q = (float *)(B + off_r2);
     uint32_t *perm = nullptr;
     if (morton)
-        KDT_TRY(morton_order(d_q, Q, t->D, t->bbox, 1, nullptr, 0, (flags & KDT_COST_ORDER) ? t->nodes : nullptr,
-                             t->N, t->layout == 3, B + off_m, &perm, s, n_far));
+        KDT_TRY(query_order(t, d_q, Q, flags & KDT_COST_ORDER, B + off_m, &perm, s, n_far));
     KDT_LAUNCH round_params_kernel<<<(P + 255) / 256, 256, 0, s>>>(t->model.d_params, wts);
     KDT_TRY(tc_radius(t, wts, d_q, Q, perm, r2, r2q, s, n_far));
     if (n_far)

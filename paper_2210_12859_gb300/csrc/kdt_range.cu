@@ -411,8 +411,7 @@ int run_range(const kdt_tree *t, int kind, int act, int flags, RangeArgs a, cuda
     a.err = t->err;
     a.perm = nullptr;
     if (morton)
-        KDT_TRY(morton_order(a.a, a.Q, t->D, t->bbox, 1, nullptr, 0, nullptr, t->N, t->layout == 3, c.base + c.off,
-                             const_cast<uint32_t **>(&a.perm), s));
+        KDT_TRY(query_order(t, a.a, a.Q, false, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
     KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
     switch (t->layout) {
     case 0: return launch_range_layout<0>(kind, act, a, s);

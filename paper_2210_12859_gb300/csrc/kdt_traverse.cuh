@@ -662,9 +662,10 @@ __device__ __forceinline__ void stage_nodes(const float4 *__restrict__ nodes, fl
 // Greedy close-child descent from the root (Sec. 3.2's closeSide rule at every
 // node) until that child does not exist; returns the FP32 squared distance to
 // the last node reached (layout 0 / 3 trees, D <= 3; stored: split dimension
-// stored in the node).
+// stored in the node), and that node.
 __device__ __forceinline__ float descent_leaf_d2(const float4 *__restrict__ nodes, const float4 *s_nodes, int staged,
-                                                 int N, int D, const float (&q)[3], bool stored = false)
+                                                 int N, int D, const float (&q)[3], bool stored = false,
+                                                 uint32_t *leaf = nullptr)
 {
     int node = 0, dim = 0;
     NodeVal<0> nd = fetch<0>(nodes, s_nodes, staged, 0);
@@ -678,6 +679,8 @@ __device__ __forceinline__ float descent_leaf_d2(const float4 *__restrict__ node
         dim = dim + 1 == D ? 0 : dim + 1;
         nd = fetch<0>(nodes, s_nodes, staged, node);
     }
+    if (leaf)
+        *leaf = (uint32_t)node;
     return dist2<3>(nd.c, q);
 }
 
