@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(co
         }
         if (busy && w.v >= b.leaf) {
             ++steps;
-            box_bucket<NC>(b, w.v - b.leaf, q, one, list);
+            box_bucket<NC, K>(b, w.v - b.leaf, q, one, list);
             busy = w.pop(list.cull(), stride);
         }
         if (steps > cap)
