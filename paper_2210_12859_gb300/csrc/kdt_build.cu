@@ -20,10 +20,12 @@
 //   * every other list still needed later is stably partitioned inside each
 //     segment into [left | node | right] with a segmented scan of the side
 //     flags, which keeps each part sorted by its own key.
-// All of it is streaming passes over arrays of N elements plus gathers of a
-// 1-byte side array (N bytes, resident in L2).  T > 1 trees are built in the
-// same passes: lists are first sorted by (tree, coordinate, index) and every
-// position knows its tree.
+// These passes run over arrays of N elements only for the levels whose subtrees
+// are larger than SUB_N points; then one block a subtree builds all the levels
+// that are left in shared memory (sub_kernel).  With them the build of 2^24
+// points is 12 passes over the lists instead of 24, and that of 20 k points 16
+// launches instead of 160.  T > 1 trees are built in the same passes: lists are
+// first sorted by (tree, coordinate, index) and every position knows its tree.
 #include <algorithm>
 #include <vector>
 
@@ -37,6 +39,25 @@ constexpr int PITEMS = 4;        // items per thread, partition scan
 constexpr int PTILE = BT * PITEMS;
 
 enum : uint8_t { SIDE_LEFT = 0, SIDE_NODE = 1, SIDE_RIGHT = 2 };
+
+// Largest subtree that one block builds in shared memory.  Large builds take
+// the largest that leaves two blocks on an SM, since every level above costs a
+// pass over all lists (2^24 points: 0.42 ms a level); small ones, which fill few
+// SMs either way and whose blocks are bound by instruction issue, a smaller one.
+constexpr int SUB_LOG2_LARGE = 12, SUB_LOG2_SMALL = 10;
+constexpr int64_t SUB_SMALL_TOTAL = (int64_t)1 << 18;
+inline int sub_log2_of(int64_t total) { return total <= SUB_SMALL_TOTAL ? SUB_LOG2_SMALL : SUB_LOG2_LARGE; }
+
+// levels of a tree of n points whose subtrees are larger than 2^sub_log2: the
+// subtrees of level l hold at most 2^(H-l) - 1 points above the last level and
+// min(M, 2^(H-l)) on it
+__host__ __device__ __forceinline__ int top_levels(int64_t n, int sub_log2)
+{
+    const Topo tp(n);
+    const int l = tp.H > sub_log2 ? tp.H - sub_log2 : 0;
+    const int64_t w = (int64_t)1 << (tp.H - l);
+    return w - 1 + (tp.M < w ? tp.M : w) <= (int64_t)1 << sub_log2 ? l : l + 1;
+}
 
 struct Where {
     int64_t base;   // first position of the position's tree
@@ -53,15 +74,17 @@ __device__ __forceinline__ Where locate(int64_t p, int T, const int64_t *__restr
     return {b, off[i + 1] - b};
 }
 
-__global__ void prep_keys_kernel(const float *__restrict__ pts, int64_t total, int D, int e,
+// sort keys of dimensions e0 .. e0 + ne - 1, `total` apart
+__global__ void prep_keys_kernel(const float *__restrict__ pts, int64_t total, int D, int e0, int ne,
                                  uint32_t *__restrict__ keys, int *__restrict__ err)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        float x = pts[i * D + e];
-        if (!isfinite(x))
-            atomicOr(err, ERR_NONFINITE);
-        keys[i] = float_key(x);
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
+        for (int e = 0; e < ne; ++e) {
+            float x = pts[i * D + e0 + e];
+            if (!isfinite(x))
+                atomicOr(err, ERR_NONFINITE);
+            keys[e * total + i] = float_key(x);
+        }
 }
 
 __global__ void tree_keys_kernel(const uint32_t *__restrict__ vals, const int32_t *__restrict__ tree_of, int64_t total,
@@ -87,28 +110,56 @@ __global__ void tree_of_kernel(const int64_t *__restrict__ off, int T, int64_t t
     }
 }
 
+struct ListPtrs {
+    const uint32_t *p[8];
+};
+
 // bounding box of the first min(D,3) dims of each tree: the extremes of the
 // per-dimension sorted lists
-__global__ void bbox_kernel(const float *__restrict__ pts, int D, const uint32_t *const *lists,
-                            const int64_t *__restrict__ off, int T, float *__restrict__ bbox)
+__global__ void bbox_kernel(const float *__restrict__ pts, int D, ListPtrs lists, const int64_t *__restrict__ off,
+                            int T, int64_t total, float *__restrict__ bbox)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= T)
         return;
-    int64_t a = off[i], b = off[i + 1];
+    int64_t a = T == 1 ? 0 : off[i], b = T == 1 ? total : off[i + 1];
     for (int e = 0; e < 3; ++e) {
         float lo = 0.f, hi = 0.f;
         if (e < D && b > a) {
-            lo = pts[(int64_t)lists[e][a] * D + e];
-            hi = pts[(int64_t)lists[e][b - 1] * D + e];
+            lo = pts[(int64_t)lists.p[e][a] * D + e];
+            hi = pts[(int64_t)lists.p[e][b - 1] * D + e];
         }
         bbox[i * 6 + e] = lo;
         bbox[i * 6 + 3 + e] = hi;
     }
 }
 
+// a node of the tree whose first point is at `base`: the point pid as node u
+__device__ __forceinline__ void emit_node(const float *__restrict__ pts, int D, int64_t base, int64_t u, uint32_t pid,
+                                          uint32_t dim_bits, float4 *__restrict__ nodes, int32_t *__restrict__ ids)
+{
+    const float *c = pts + (int64_t)pid * D;
+    const int32_t local = (int32_t)(pid - (uint32_t)base);
+    const int64_t node = base + u;
+    if (D <= 3) {
+        nodes[node] = make_float4(c[0], D > 1 ? c[1] : 0.f, D > 2 ? c[2] : 0.f,
+                                  __uint_as_float((uint32_t)local | dim_bits));
+    } else if (D == 4) {
+        nodes[node] = make_float4(c[0], c[1], c[2], c[3]);
+        ids[node] = local;
+    } else {
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            v[j] = j < D ? c[j] : 0.f;
+        nodes[2 * node] = make_float4(v[0], v[1], v[2], v[3]);
+        nodes[2 * node + 1] = make_float4(v[4], v[5], v[6], v[7]);
+        ids[node] = local;
+    }
+}
+
 // Level l, split list: record each point's side and emit the level's nodes.
-__global__ void assign_kernel(const uint32_t *__restrict__ list, int64_t total, int l, int T,
+__global__ void assign_kernel(const uint32_t *__restrict__ list, int64_t total, int l, int sub_log2, int T,
                               const int64_t *__restrict__ off, const int32_t *__restrict__ tree_of,
                               const float *__restrict__ pts, int D, uint8_t *__restrict__ side,
                               float4 *__restrict__ nodes, int32_t *__restrict__ ids)
@@ -116,7 +167,7 @@ __global__ void assign_kernel(const uint32_t *__restrict__ list, int64_t total, 
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total; p += (int64_t)gridDim.x * blockDim.x) {
         Where w = locate(p, T, off, tree_of, total);
         Topo tp(w.n);
-        if (l > tp.H)
+        if (l >= top_levels(w.n, sub_log2))
             continue;
         int64_t u = tp.node_at(p - w.base);
         int lu = Topo::level(u);
@@ -125,24 +176,7 @@ __global__ void assign_kernel(const uint32_t *__restrict__ list, int64_t total, 
         uint32_t pid = list[p];
         if (lu == l) {
             side[pid] = SIDE_NODE;
-            const float *c = pts + (int64_t)pid * D;
-            int32_t local = (int32_t)(pid - (uint32_t)w.base);
-            int64_t node = w.base + u;
-            if (D <= 3) {
-                float4 v = make_float4(c[0], D > 1 ? c[1] : 0.f, D > 2 ? c[2] : 0.f, __int_as_float(local));
-                nodes[node] = v;
-            } else if (D == 4) {
-                nodes[node] = make_float4(c[0], c[1], c[2], c[3]);
-                ids[node] = local;
-            } else {
-                float v[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    v[j] = j < D ? c[j] : 0.f;
-                nodes[2 * node] = make_float4(v[0], v[1], v[2], v[3]);
-                nodes[2 * node + 1] = make_float4(v[4], v[5], v[6], v[7]);
-                ids[node] = local;
-            }
+            emit_node(pts, D, w.base, u, pid, 0u, nodes, ids);
         } else {
             int bit = (int)(((u + 1) >> (lu - l - 1)) & 1);
             side[pid] = bit ? SIDE_RIGHT : SIDE_LEFT;
@@ -151,10 +185,6 @@ __global__ void assign_kernel(const uint32_t *__restrict__ list, int64_t total, 
 }
 
 // ---- stored split dimension (widest extent of the node's points)
-
-struct ListPtrs {
-    const uint32_t *p[8];
-};
 
 // split dimension of every node of level l: within the node's segment each
 // list is sorted by its coordinate, so its first and last elements give the
@@ -203,9 +233,7 @@ __global__ void assign_widest_kernel(ListPtrs lists, int64_t n, int l, const uin
         const uint32_t pid = lists.p[e][p];
         if (lu == l) {
             side[pid] = SIDE_NODE;
-            const float *c = pts + (int64_t)pid * D;
-            const uint32_t word = pid | ((uint32_t)e << NODE_DIM_SHIFT);
-            nodes[u] = make_float4(c[0], D > 1 ? c[1] : 0.f, D > 2 ? c[2] : 0.f, __uint_as_float(word));
+            emit_node(pts, D, 0, u, pid, (uint32_t)e << NODE_DIM_SHIFT, nodes, nullptr);
         } else {
             const int bit = (int)(((u + 1) >> (lu - l - 1)) & 1);
             side[pid] = bit ? SIDE_RIGHT : SIDE_LEFT;
@@ -237,7 +265,7 @@ struct Item {
     int64_t base, n;
 };
 
-__device__ __forceinline__ void load_item(const uint32_t *__restrict__ in, int64_t p, int64_t total, int l, int T,
+__device__ __forceinline__ void load_item(const uint32_t *__restrict__ in, int64_t p, int64_t total, int l, int sub_log2, int T,
                                           const int64_t *__restrict__ off, const int32_t *__restrict__ tree_of,
                                           const uint8_t *__restrict__ side, Item &it)
 {
@@ -249,7 +277,7 @@ __device__ __forceinline__ void load_item(const uint32_t *__restrict__ in, int64
     it.pid = in[p];
     Where w = locate(p, T, off, tree_of, total);
     Topo tp(w.n);
-    if (l > tp.H)
+    if (l >= top_levels(w.n, sub_log2))
         return;
     int64_t lp = p - w.base;
     int64_t u = tp.node_at(lp);
@@ -316,7 +344,8 @@ __device__ __forceinline__ Seg block_exclusive_seg(Seg x, Seg *s_warp, Seg *agg)
     return r;
 }
 
-__global__ void __launch_bounds__(BT) part_reduce_kernel(const uint32_t *__restrict__ in, int64_t total, int l, int T,
+__global__ void __launch_bounds__(BT) part_reduce_kernel(const uint32_t *__restrict__ in, int64_t total, int l,
+                                                         int sub_log2, int T,
                                                          const int64_t *__restrict__ off,
                                                          const int32_t *__restrict__ tree_of,
                                                          const uint8_t *__restrict__ side, Seg *__restrict__ tiles)
@@ -327,7 +356,7 @@ __global__ void __launch_bounds__(BT) part_reduce_kernel(const uint32_t *__restr
 #pragma unroll
     for (int j = 0; j < PITEMS; ++j) {
         Item it;
-        load_item(in, base + j, total, l, T, off, tree_of, side, it);
+        load_item(in, base + j, total, l, sub_log2, T, off, tree_of, side, it);
         acc = seg_op(acc, it.s);
     }
     Seg agg;
@@ -351,7 +380,8 @@ __global__ void __launch_bounds__(1024) part_tiles_kernel(Seg *__restrict__ tile
     }
 }
 
-__global__ void __launch_bounds__(BT) part_scatter_kernel(const uint32_t *__restrict__ in, int64_t total, int l, int T,
+__global__ void __launch_bounds__(BT) part_scatter_kernel(const uint32_t *__restrict__ in, int64_t total, int l,
+                                                          int sub_log2, int T,
                                                           const int64_t *__restrict__ off,
                                                           const int32_t *__restrict__ tree_of,
                                                           const uint8_t *__restrict__ side,
@@ -363,7 +393,7 @@ __global__ void __launch_bounds__(BT) part_scatter_kernel(const uint32_t *__rest
     Seg acc{0, 0};
 #pragma unroll
     for (int j = 0; j < PITEMS; ++j) {
-        load_item(in, base + j, total, l, T, off, tree_of, side, it[j]);
+        load_item(in, base + j, total, l, sub_log2, T, off, tree_of, side, it[j]);
         acc = seg_op(acc, it[j].s);
     }
     Seg agg;
@@ -395,6 +425,448 @@ __global__ void __launch_bounds__(BT) part_scatter_kernel(const uint32_t *__rest
     }
 }
 
+// ---- single trees: one pass a list and level
+
+// The in-order layout of a complete tree of n < 2^30 points in 32 bits.
+struct Layout32 {
+    int n, H, M;
+    __device__ __forceinline__ explicit Layout32(int n_) : n(n_)
+    {
+        H = 31 - __clz(n_);
+        M = n_ - ((1 << H) - 1);
+    }
+    __device__ __forceinline__ static int level(int u) { return 31 - __clz(u + 1); }
+    __device__ __forceinline__ int node_at(int p) const
+    {
+        const int P = p < 2 * M ? p : 2 * (p - M) + 1;
+        const int tz = __ffs(P + 1) - 1;
+        return (1 << (H - tz)) - 1 + ((P + 1) >> (tz + 1));
+    }
+    __device__ __forceinline__ int inorder(int u) const
+    {
+        const int l = level(u);
+        const int P = ((2 * (u - ((1 << l) - 1)) + 1) << (H - l)) - 1;
+        const int missing = min((P + 1) >> 1, 1 << H) - M;
+        return P - max(missing, 0);
+    }
+    // the j-th subtree of level l: w = 2^(H-l) places on the last level
+    __device__ __forceinline__ int start(int l, int j) const { return (j << (H - l)) + min(M, j << (H - l)); }
+    __device__ __forceinline__ int size(int l, int j) const
+    {
+        const int w = 1 << (H - l);
+        return w - 1 + min(max(M - j * w, 0), w);
+    }
+    // points of its left subtree
+    __device__ __forceinline__ int left(int l, int j) const
+    {
+        const int w = 1 << (H - l), h = w >> 1;
+        return h - 1 + min(max(M - j * w, 0), h);
+    }
+    // points of the left subtrees of the subtrees before it on the level
+    __device__ __forceinline__ int lefts_before(int l, int j) const
+    {
+        const int w = 1 << (H - l), h = w >> 1;
+        const int full = M >= h ? min(j, ((M - h) >> (H - l)) + 1) : 0;
+        return j * (h - 1) + full * h + (full < j ? min(max(M - full * w, 0), h) : 0);
+    }
+};
+
+// Where the element at place p of a level's list goes: `lefts` and `ones` are
+// the left elements and the level's nodes at places before p.
+__device__ __forceinline__ int part_dest(const Layout32 &t, int l, int u, int lu, int p, int side, int lefts, int ones)
+{
+    const int j = ((u + 1) >> (lu - l)) - (1 << l);
+    const int s = t.start(l, j), in = s + t.left(l, j);
+    if (side == SIDE_NODE)
+        return in;
+    const int lb = lefts - t.lefts_before(l, j);
+    if (side == SIDE_LEFT)
+        return s + lb;
+    return in + 1 + (p - s) - lb - (ones - j);
+}
+
+constexpr int TOP_ITEMS = 8;
+constexpr int TOP_TILE = BT * TOP_ITEMS;
+constexpr int TOP_LISTS = 3;  // lists of one launch
+constexpr unsigned long long TOP_OWN = 1ull << 62, TOP_ALL = 2ull << 62, TOP_VALUE = (1ull << 62) - 1;
+constexpr int TOP_POLLS = 1 << 16;
+
+struct PartArgs {
+    const uint32_t *in[TOP_LISTS];
+    uint32_t *out[TOP_LISTS];
+    const uint8_t *side;
+    unsigned long long *state;  // [list][tiles]
+    uint32_t *ticket;           // [list]
+    int n, l, tiles;
+    // the list that splits the next level also records that level's sides and
+    // emits its nodes (-1: none does)
+    int next;
+    uint8_t *side_next;
+    const float *pts;
+    int D;
+    float4 *nodes;
+    int32_t *ids;
+};
+
+// Stable partition of up to three lists by the level's sides in one pass each.
+// A plain count of the left elements suffices, no segmented one: how many the
+// earlier subtrees of the level hold is a closed form of the layout.  The count
+// of the tiles before comes from a bounded look-back as in the radix sort (a
+// silent predecessor is counted from its elements).
+//
+// Bound: the random bytes, a gather an element and list and a store an element
+// for the next level's sides (L1-to-L2 requests 56 % busy), and the wait for the
+// look-back.  It replaced a count, a single-block scan and a scatter with 64-bit
+// segmented scans a list, and a pass that assigned the next level's sides: a
+// level of 2^24 points takes 0.42 ms instead of 0.71.  Tiles of 4 / 8 / 16 elements
+// a thread: the build of 2^24 points 11.4 / 11.0 / 12.9 ms.
+__global__ void __launch_bounds__(BT, 4) part_kernel(const PartArgs a)
+{
+    __shared__ uint32_t s_cnt[BT / 32];
+    __shared__ unsigned long long s_before;
+    __shared__ uint32_t s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, y = blockIdx.y;
+    if (tid == 0)
+        s_tile = atomicAdd(a.ticket + y, 1u);
+    __syncthreads();
+    const int tile = (int)s_tile;
+    const uint32_t *in = y == 0 ? a.in[0] : (y == 1 ? a.in[1] : a.in[2]);
+    uint32_t *out = y == 0 ? a.out[0] : (y == 1 ? a.out[1] : a.out[2]);
+    const Layout32 t(a.n);
+    const int first = tile * TOP_TILE + w * 32 * TOP_ITEMS + lane;
+    uint32_t pid[TOP_ITEMS], before[TOP_ITEMS], sides = 0;  // before: nodes << 16 | lefts, of the warp's earlier places
+    uint32_t run = 0;
+    const uint32_t lt = (1u << lane) - 1;
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j) {
+        const int p = first + 32 * j;
+        pid[j] = p < a.n ? in[p] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j) {
+        const int p = first + 32 * j;
+        uint32_t s = 3;  // not in a subtree of the level
+        if (p < a.n && Layout32::level(t.node_at(p)) >= a.l)
+            s = a.side[pid[j]];
+        sides |= s << (2 * j);
+        const uint32_t bl = __ballot_sync(0xffffffffu, s == SIDE_LEFT), bn = __ballot_sync(0xffffffffu, s == SIDE_NODE);
+        before[j] = run + (__popc(bl & lt) | __popc(bn & lt) << 16);
+        run += __popc(bl) | __popc(bn) << 16;
+    }
+    if (lane == 0)
+        s_cnt[w] = run;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t own = lane < BT / 32 ? s_cnt[lane] : 0;
+        own = __reduce_add_sync(0xffffffffu, own);  // at most 4096 of each
+        const unsigned long long mine = (unsigned long long)(own >> 16) << 32 | (own & 0xffffu);
+        volatile unsigned long long *st = a.state + (size_t)y * a.tiles;
+        if (lane == 0)
+            st[tile] = (tile ? TOP_OWN : TOP_ALL) | mine;
+        unsigned long long sum = 0;
+        for (int back = tile - 1; back >= 0; back -= 32) {
+            const int q = back - lane;
+            unsigned long long v = q < 0 ? TOP_ALL : 0;
+            for (int polls = 0; v == 0 && polls < TOP_POLLS; ++polls)
+                v = st[q];
+            if (v == 0) {
+                unsigned long long c = 0;
+                for (int p = q * TOP_TILE; p < (q + 1) * TOP_TILE; ++p)
+                    if (Layout32::level(t.node_at(p)) >= a.l) {
+                        const int s = a.side[in[p]];
+                        c += s == SIDE_LEFT ? 1ull : (s == SIDE_NODE ? 1ull << 32 : 0ull);
+                    }
+                v = TOP_OWN | c;
+            }
+            __syncwarp();
+            const uint32_t all = __ballot_sync(0xffffffffu, (v & TOP_ALL) != 0);
+            const int stop = all ? __ffs(all) - 1 : 31;
+            unsigned long long x = lane <= stop ? v & TOP_VALUE : 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                x += __shfl_xor_sync(0xffffffffu, x, o);
+            sum += x;
+            if (all)
+                break;
+        }
+        if (lane == 0) {
+            if (tile)
+                st[tile] = TOP_ALL | (sum + mine);
+            s_before = sum;
+        }
+    }
+    __syncthreads();
+    uint32_t warps = lane < w ? s_cnt[lane] : 0;
+    warps = __reduce_add_sync(0xffffffffu, warps);
+    const int lefts0 = (int)(s_before & 0xffffffffu) + (int)(warps & 0xffffu);
+    const int ones0 = (int)(s_before >> 32) + (int)(warps >> 16);
+    const bool next = y == a.next;
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j) {
+        const int s = sides >> (2 * j) & 3u;
+        if (s == 3)
+            continue;
+        const int p = first + 32 * j;
+        const int u = t.node_at(p), lu = Layout32::level(u);
+        const int d = part_dest(t, a.l, u, lu, p, s, lefts0 + (int)(before[j] & 0xffffu), ones0 + (int)(before[j] >> 16));
+        if (d < 0 || d >= a.n)  // never, for consistent sides
+            continue;
+        out[d] = pid[j];
+        if (next && s != SIDE_NODE) {
+            const int v = t.node_at(d), lv = Layout32::level(v);
+            if (lv == a.l + 1) {
+                a.side_next[pid[j]] = SIDE_NODE;
+                emit_node(a.pts, a.D, 0, v, pid[j], 0u, a.nodes, a.ids);
+            } else {
+                a.side_next[pid[j]] = (v + 1) >> (lv - a.l - 2) & 1 ? SIDE_RIGHT : SIDE_LEFT;
+            }
+        }
+    }
+}
+
+// ---- the levels whose subtrees fit one block
+
+// places a thread looks after; places and counts of a subtree fit 13 bits
+constexpr int SUB_ITEMS = 4;
+static_assert(SUB_LOG2_LARGE <= 12, "places and counts of a subtree are packed");
+
+struct SubArgs {
+    ListPtrs lists;
+    const int64_t *off;       // T > 1: first point of every tree, [T + 1]
+    const int32_t *first_job; // T > 1: first block of every tree, [T + 1]
+    int64_t total;
+    int T, D;
+    bool widest;
+    const float *pts;
+    uint16_t *place;          // [total] scratch: a point's place in its block
+    float4 *nodes;
+    int32_t *ids;
+};
+
+// bytes of sub_kernel's arrays: pid, warp counts, then 16-bit places, lists and bytes
+inline size_t sub_smem(int D, int sub_log2)
+{
+    const size_t n = (size_t)1 << sub_log2;
+    return n * (4 + 2 * (D + 1) + 2) + 2 * 32 * 4;
+}
+
+// Block b: one subtree of the first level whose subtrees fit, all its levels.
+// The points are renumbered 0 .. n - 1, so the lists are 16-bit and lie in
+// shared memory with the side bytes; a level is one look at the split list and
+// one stable partition of the others by a block-wide count, both with the
+// closed forms of the subtree's own layout, two lists at a time so that a
+// place's closed forms are worked out once for both.  A node's point is noted
+// by in-order place and all nodes are written at the end, a level's nodes side
+// by side.
+//
+// Bound: instruction issue (the places' closed forms, some 60 instructions a
+// place and level) between the block's barriers.  Threads with 4 / 8 / 16 places
+// each: a build of 2^24 points 11.0 / 11.2 / 12.8 ms, a rebuild of 20 k 196 / 210 /
+// 233 us; subtrees of 2^11 instead of 2^12 cost the large build 0.2 ms, of 2^9 or
+// 2^11 instead of 2^10 the small one 2 to 6 us.
+template <int SUB_LOG2>
+__global__ void __launch_bounds__((1 << SUB_LOG2) / SUB_ITEMS, SUB_LOG2 == 12 ? 1 : 4) sub_kernel(const SubArgs a)
+{
+    constexpr int SUB_N = 1 << SUB_LOG2;
+    constexpr int THREADS = SUB_N / SUB_ITEMS;
+    constexpr int WARPS = THREADS / 32;
+    static_assert(WARPS <= 32, "the warp counts of two lists are summed by one warp");
+    extern __shared__ uint32_t s_mem[];
+    uint32_t *s_pid = s_mem;                                          // [SUB_N]
+    uint32_t *s_cnt = s_pid + SUB_N;                                  // [2][32]: two lists, a warp each
+    uint16_t *s_fin = reinterpret_cast<uint16_t *>(s_cnt + 64);       // [SUB_N] by in-order place
+    uint16_t *s_list = s_fin + SUB_N;                                 // [D][SUB_N]
+    uint8_t *s_side = reinterpret_cast<uint8_t *>(s_list + (size_t)a.D * SUB_N);  // [SUB_N]
+    uint8_t *s_dim = s_side + SUB_N;                                  // [SUB_N] split dimension of a node (widest)
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, D = a.D;
+
+    int64_t base = 0, tn = a.total;
+    int job = blockIdx.x;
+    if (a.T > 1) {
+        int lo = 0, hi = a.T - 1;  // last tree that starts at or before the block (empty trees have no block)
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.first_job[mid] <= job)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        base = a.off[lo];
+        tn = a.off[lo + 1] - base;
+        job -= a.first_job[lo];
+    }
+    const Layout32 whole((int)tn);
+    const int top = top_levels(tn, SUB_LOG2);
+    const int n = whole.size(top, job);
+    const int64_t seg = base + whole.start(top, job);
+    const Layout32 t(n);
+
+    const uint32_t *l0 = a.lists.p[0] + seg;
+    for (int i = tid; i < n; i += THREADS) {
+        const uint32_t pid = l0[i];
+        s_pid[i] = pid;
+        s_list[i] = (uint16_t)i;
+        a.place[pid] = (uint16_t)i;
+    }
+    __syncthreads();
+    for (int e = 1; e < D; ++e) {
+        const uint32_t *le = a.lists.p[e] + seg;
+        for (int i = tid; i < n; i += THREADS)
+            s_list[e * SUB_N + i] = a.place[le[i]];
+    }
+    __syncthreads();
+
+    // the node of a thread's places: index + 1, 0 past the end
+    const int first = w * 32 * SUB_ITEMS + lane;
+    uint16_t node[SUB_ITEMS];
+#pragma unroll
+    for (int k = 0; k < SUB_ITEMS; ++k)
+        node[k] = first + 32 * k < n ? (uint16_t)(t.node_at(first + 32 * k) + 1) : (uint16_t)0;
+    const uint32_t lt = (1u << lane) - 1;
+    for (int l = 0; l <= t.H; ++l) {
+        const int d = (top + l) % D;
+        const uint32_t level = 1u << l;  // node + 1 of the level's first node
+        if (a.widest) {
+            const int count = min(1 << l, n - ((1 << l) - 1));
+            for (int j = tid; j < count; j += THREADS) {
+                const int s = t.start(l, j), z = s + t.size(l, j) - 1;
+                int best = 0;
+                float best_ext = -1.f;
+                for (int e = 0; e < D; ++e) {
+                    const float lo = a.pts[(int64_t)s_pid[s_list[e * SUB_N + s]] * D + e];
+                    const float hi = a.pts[(int64_t)s_pid[s_list[e * SUB_N + z]] * D + e];
+                    const float ext = __fsub_rn(hi, lo);
+                    if (ext > best_ext) {
+                        best_ext = ext;
+                        best = e;
+                    }
+                }
+                s_dim[(1 << l) - 1 + j] = (uint8_t)best;
+            }
+            __syncthreads();
+        }
+        // the split list: sides, and the level's nodes
+#pragma unroll
+        for (int k = 0; k < SUB_ITEMS; ++k) {
+            const uint32_t u = node[k];
+            if (u < level)
+                continue;
+            const int p = first + 32 * k;
+            const int below = 31 - __clz(u) - l;
+            const int e = a.widest ? s_dim[(u >> below) - 1] : d;
+            const int id = s_list[e * SUB_N + p];
+            if (below == 0) {
+                s_side[id] = SIDE_NODE;
+                s_fin[p] = (uint16_t)id;
+            } else {
+                s_side[id] = u >> (below - 1) & 1 ? SIDE_RIGHT : SIDE_LEFT;
+            }
+        }
+        if (l == t.H)
+            break;
+        __syncthreads();
+        // the other lists, two at a time; e1 < 0: one
+        for (int e0 = !a.widest && d == 0 ? 1 : 0; e0 < D;) {
+            int e1 = e0 + 1;
+            if (e1 == d && !a.widest)
+                ++e1;
+            int e_next = e1 + 1;
+            if (e_next == d && !a.widest)
+                ++e_next;
+            const bool two = e1 < D;
+            uint16_t *la = s_list + e0 * SUB_N, *lb = s_list + (two ? e1 : e0) * SUB_N;
+            // ids and sides (12 + 2 bits) of both lists; lefts and nodes at the warp's earlier places
+            uint32_t item[SUB_ITEMS], before_a[SUB_ITEMS], before_b[SUB_ITEMS];
+            uint32_t run_a = 0, run_b = 0;
+#pragma unroll
+            for (int k = 0; k < SUB_ITEMS; ++k) {
+                uint32_t ia = 0, ib = 0, sa = 3, sb = 3;
+                if (node[k] >= level) {
+                    ia = la[first + 32 * k];
+                    ib = lb[first + 32 * k];
+                    sa = s_side[ia];
+                    sb = s_side[ib];
+                }
+                item[k] = ia | sa << 14 | ib << 16 | sb << 30;
+                const uint32_t al = __ballot_sync(0xffffffffu, sa == SIDE_LEFT);
+                const uint32_t an = __ballot_sync(0xffffffffu, sa == SIDE_NODE);
+                const uint32_t bl = __ballot_sync(0xffffffffu, sb == SIDE_LEFT);
+                const uint32_t bn = __ballot_sync(0xffffffffu, sb == SIDE_NODE);
+                before_a[k] = run_a + (__popc(al & lt) | __popc(an & lt) << 16);
+                before_b[k] = run_b + (__popc(bl & lt) | __popc(bn & lt) << 16);
+                run_a += __popc(al) | __popc(an) << 16;
+                run_b += __popc(bl) | __popc(bn) << 16;
+            }
+            if (lane == 0) {
+                s_cnt[w] = run_a;
+                s_cnt[32 + w] = run_b;
+            }
+            __syncthreads();
+            const uint32_t warps_a = __reduce_add_sync(0xffffffffu, lane < w ? s_cnt[lane] : 0);
+            const uint32_t warps_b = __reduce_add_sync(0xffffffffu, lane < w ? s_cnt[32 + lane] : 0);
+#pragma unroll
+            for (int k = 0; k < SUB_ITEMS; ++k) {
+                const uint32_t u = node[k];
+                if (u < level)
+                    continue;
+                // as part_dest, once for both lists
+                const int p = first + 32 * k;
+                const int j = (int)(u >> (31 - __clz(u) - l)) - (1 << l);
+                const int s = t.start(l, j), in = s + t.left(l, j), lefts = t.lefts_before(l, j);
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    if (x == 1 && !two)
+                        continue;
+                    const uint32_t c = x ? warps_b + before_b[k] : warps_a + before_a[k];
+                    const uint32_t it = x ? item[k] >> 16 : item[k] & 0xffffu;
+                    const int side = it >> 14;
+                    const int lbf = (int)(c & 0xffffu) - lefts;
+                    const int to = side == SIDE_NODE ? in
+                                   : (side == SIDE_LEFT ? s + lbf : in + 1 + (p - s) - lbf - ((int)(c >> 16) - j));
+                    if (to >= 0 && to < n)  // always, for consistent sides
+                        (x ? lb : la)[to] = (uint16_t)(it & 0xfffu);
+                }
+            }
+            __syncthreads();
+            e0 = e_next;
+        }
+    }
+    __syncthreads();
+    for (int u = tid; u < n; u += THREADS) {
+        const int l = Layout32::level(u), j = u - ((1 << l) - 1);
+        // the subtree's root is node job of level `top`
+        const int64_t at = ((int64_t)1 << (top + l)) - 1 + ((int64_t)job << l) + j;
+        emit_node(a.pts, D, base, at, s_pid[s_fin[t.inorder(u)]],
+                  a.widest ? (uint32_t)s_dim[u] << NODE_DIM_SHIFT : 0u, a.nodes, a.ids);
+    }
+}
+
+template <int SUB_LOG2>
+int launch_sub(const SubArgs &a, int64_t jobs, cudaStream_t s)
+{
+    const size_t smem = sub_smem(a.D, SUB_LOG2);
+    KDT_CUDA(cudaFuncSetAttribute((const void *)sub_kernel<SUB_LOG2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem));
+    KDT_LAUNCH sub_kernel<SUB_LOG2><<<(unsigned)jobs, (1 << SUB_LOG2) / SUB_ITEMS, smem, s>>>(a);
+    KDT_CUDA(cudaGetLastError());
+    return KDT_OK;
+}
+
+// level 0 of a single tree: sides and the root from its split list
+__global__ void __launch_bounds__(BT) root_kernel(const uint32_t *__restrict__ list, int n,
+                                                  const float *__restrict__ pts, int D, uint8_t *__restrict__ side,
+                                                  float4 *__restrict__ nodes, int32_t *__restrict__ ids)
+{
+    const Layout32 t(n);
+    const int in = t.left(0, 0);
+    for (int p = blockIdx.x * BT + threadIdx.x; p < n; p += gridDim.x * BT) {
+        const uint32_t pid = list[p];
+        side[pid] = p < in ? SIDE_LEFT : (p == in ? SIDE_NODE : SIDE_RIGHT);
+        if (p == in)
+            emit_node(pts, D, 0, 0, pid, 0u, nodes, ids);
+    }
+}
+
 inline unsigned grid_for(int64_t n)
 {
     int64_t b = (n + BT - 1) / BT;
@@ -418,113 +890,194 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
                  int *err, cudaStream_t s, bool widest)
 {
     const int64_t total = h_off[T];
-    int maxH = 0;
-    for (int i = 0; i < T; ++i) {
-        int64_t n = h_off[i + 1] - h_off[i];
-        if (n > 0)
-            maxH = std::max(maxH, floor_log2((uint64_t)n));
-    }
     if (total == 0)
         return KDT_OK;
+    // levels built by passes over the whole lists, and the blocks of sub_kernel
+    const int sub_log2 = sub_log2_of(total);
+    int levels = 0;
+    std::vector<int32_t> first_job(T + 1, 0);
+    int64_t jobs = 0;
+    for (int i = 0; i < T; ++i) {
+        const int64_t n = h_off[i + 1] - h_off[i];
+        first_job[i] = (int32_t)jobs;
+        if (n > 0) {
+            levels = std::max(levels, top_levels(n, sub_log2));
+            jobs += (int64_t)1 << top_levels(n, sub_log2);
+        }
+    }
+    first_job[T] = (int32_t)jobs;
 
-    // scratch: D lists + spare + 2 key arrays (u32), side (u8), tree_of (i32),
-    // offsets (i64), tiles (Seg), radix scratch
-    const int64_t ptiles = (total + PTILE - 1) / PTILE;
-    const size_t rs = radix_scratch_elems(total);
+    // Arrays of `total` u32: lists, keys and their temporaries.  Small builds,
+    // whose time is their launches, sort all dimensions at once (1.05 M points
+    // of 3 dimensions: below the launch's cost from there); large ones one
+    // after the other with one temporary.
+    const bool together = (int64_t)total * D <= ((int64_t)1 << 21);
+    const int at_once = together ? D : 1;
+    const int64_t ptiles = (total + PTILE - 1) / PTILE;         // T > 1
+    const int top_tiles = (int)((total + TOP_TILE - 1) / TOP_TILE);  // T == 1
+    const size_t rs = radix_scratch_elems(total) * at_once;
     size_t bytes = 0;
     auto take = [&](size_t b) {
         size_t o = bytes;
         bytes += (b + 255) & ~(size_t)255;
         return o;
     };
-    size_t o_lists = take((size_t)(D + 1) * total * 4);
-    size_t o_keys = take((size_t)2 * total * 4);
-    size_t o_side = take((size_t)total);
+    // lists [D], list temporaries [at_once], keys and their temporaries
+    // [2 at_once]: all but the lists serve the partitions as targets
+    const int spares = 3 * at_once;
+    size_t o_lists = take((size_t)(D + spares) * total * 4);
+    size_t o_side = take((size_t)total * 2);
+    size_t o_place = take((size_t)total * 2);
     size_t o_tree = take(T > 1 ? (size_t)total * 4 : 0);
-    size_t o_off = take((size_t)(T + 1) * 8);
-    size_t o_tiles = take((size_t)ptiles * sizeof(Seg));
+    size_t o_off = take(T > 1 ? (size_t)(T + 1) * 8 : 0);
+    size_t o_job = take(T > 1 ? (size_t)(T + 1) * 4 : 0);
+    size_t o_tiles = take(T > 1 ? (size_t)ptiles * sizeof(Seg) : 0);
     size_t o_rs = take(rs * 4);
-    size_t o_lptr = take((size_t)8 * sizeof(uint32_t *));
+    // look-back states and tickets of every partition
+    const int parts = T == 1 ? levels * D : 0;
+    const size_t state_bytes = (size_t)parts * top_tiles * 8 + (size_t)parts * 4;
+    size_t o_state = take(state_bytes);
     size_t o_dim = take(widest ? (size_t)total : 0);
     DevBuf buf;
     buf.s = s;
     KDT_CUDA(cudaMallocAsync(&buf.p, bytes, s));
     char *B = (char *)buf.p;
-    uint32_t *lists[9];
-    for (int e = 0; e <= D; ++e)
-        lists[e] = (uint32_t *)(B + o_lists) + (size_t)e * total;
-    uint32_t *spare = lists[D];
-    uint32_t *k0 = (uint32_t *)(B + o_keys);
-    uint32_t *k1 = k0 + total;
-    uint8_t *side = (uint8_t *)(B + o_side);
+    uint32_t *arrays = (uint32_t *)(B + o_lists);
+    uint32_t *lists[8], *spare[24];
+    for (int e = 0; e < D; ++e)
+        lists[e] = arrays + (size_t)e * total;
+    for (int i = 0; i < spares; ++i)
+        spare[i] = arrays + (size_t)(D + i) * total;
+    uint8_t *side = (uint8_t *)(B + o_side), *side_next = side + total;
     int32_t *tree_of = T > 1 ? (int32_t *)(B + o_tree) : nullptr;
-    int64_t *d_off = (int64_t *)(B + o_off);
+    int64_t *d_off = T > 1 ? (int64_t *)(B + o_off) : nullptr;
+    int32_t *d_job = T > 1 ? (int32_t *)(B + o_job) : nullptr;
     Seg *tiles = (Seg *)(B + o_tiles);
     uint32_t *rscr = (uint32_t *)(B + o_rs);
-    uint32_t **d_lptr = (uint32_t **)(B + o_lptr);
     uint8_t *node_dim = (uint8_t *)(B + o_dim);
 
-    KDT_CUDA(cudaMemcpyAsync(d_off, h_off, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
     const unsigned g = grid_for(total);
-    if (T > 1)
+    if (T > 1) {
+        KDT_CUDA(cudaMemcpyAsync(d_off, h_off, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        KDT_CUDA(cudaMemcpyAsync(d_job, first_job.data(), (T + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         KDT_LAUNCH tree_of_kernel<<<g, BT, 0, s>>>(d_off, T, total, tree_of);
+    }
     int tbits = T > 1 ? floor_log2((uint64_t)(T - 1)) + 1 : 0;
 
     // per-dimension lists sorted by (tree, coordinate, index)
-    for (int e = 0; e < D; ++e) {
-        KDT_LAUNCH prep_keys_kernel<<<g, BT, 0, s>>>(d_points, total, D, e, k0, err);
-        KDT_TRY(radix_sort_batch(&k0, &lists[e], &k1, &spare, total, 1, total, 0, 32, true, rscr, s));
+    for (int e = 0; e < D; e += at_once) {
+        uint32_t *k0 = spare[at_once], *k1 = spare[2 * at_once], *v0 = lists[e], *v1 = spare[0];
+        KDT_LAUNCH prep_keys_kernel<<<g, BT, 0, s>>>(d_points, total, D, e, at_once, k0, err);
+        KDT_TRY(radix_sort_batch(&k0, &v0, &k1, &v1, total, at_once, total, 0, 32, true, rscr, s));
         if (T > 1) {
-            KDT_LAUNCH tree_keys_kernel<<<g, BT, 0, s>>>(lists[e], tree_of, total, k0);
-            KDT_TRY(radix_sort_batch(&k0, &lists[e], &k1, &spare, total, 1, total, 0, tbits, false, rscr, s));
+            for (int i = 0; i < at_once; ++i)
+                KDT_LAUNCH tree_keys_kernel<<<g, BT, 0, s>>>(v0 + (size_t)i * total, tree_of, total,
+                                                             k0 + (size_t)i * total);
+            KDT_TRY(radix_sort_batch(&k0, &v0, &k1, &v1, total, at_once, total, 0, tbits, false, rscr, s));
         }
+        // an odd number of passes leaves the result in the temporaries
+        if (v0 != lists[e])
+            for (int i = 0; i < at_once; ++i)
+                std::swap(lists[e + i], spare[i]);
     }
-    KDT_CUDA(cudaMemcpyAsync(d_lptr, lists, 8 * sizeof(uint32_t *), cudaMemcpyHostToDevice, s));
-    KDT_LAUNCH bbox_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_points, D, d_lptr, d_off, T, bbox);
+    ListPtrs lp;
+    auto list_ptrs = [&]() {
+        for (int e = 0; e < 8; ++e)
+            lp.p[e] = e < D ? lists[e] : nullptr;
+    };
+    list_ptrs();
+    KDT_LAUNCH bbox_kernel<<<(T + 127) / 128, 128, 0, s>>>(d_points, D, lp, d_off, T, total, bbox);
 
-    if (widest) {
-        // per-node split dimensions: every list may be a node's split list,
-        // so every list is partitioned at every level that has a successor
-        for (int l = 0; l <= maxH; ++l) {
-            ListPtrs lp;
-            for (int e = 0; e < 8; ++e)
-                lp.p[e] = e < D ? lists[e] : nullptr;
-            const int64_t level_nodes = std::min<int64_t>((int64_t)1 << l, total - (((int64_t)1 << l) - 1));
-            KDT_LAUNCH widest_kernel<<<grid_for(level_nodes), BT, 0, s>>>(lp, total, l, d_points, D, node_dim);
-            KDT_LAUNCH assign_widest_kernel<<<g, BT, 0, s>>>(lp, total, l, node_dim, d_points, D, side, nodes);
-            if (l < maxH) {
-                for (int e = 0; e < D; ++e) {
-                    KDT_LAUNCH part_reduce_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, T, d_off, tree_of,
-                                                                                  side, tiles);
-                    KDT_LAUNCH part_tiles_kernel<<<1, 1024, 0, s>>>(tiles, ptiles);
-                    KDT_LAUNCH part_scatter_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, T, d_off,
-                                                                                   tree_of, side, tiles, spare);
-                    std::swap(lists[e], spare);
+    if (T == 1) {
+        const int n = (int)total;
+        unsigned long long *state = (unsigned long long *)(B + o_state);
+        uint32_t *ticket = (uint32_t *)(state + (size_t)parts * top_tiles);
+        if (parts)
+            KDT_CUDA(cudaMemsetAsync(state, 0, state_bytes, s));
+        if (levels && !widest)
+            KDT_LAUNCH root_kernel<<<g, BT, 0, s>>>(lists[0], n, d_points, D, side, nodes, ids);
+        for (int l = 0; l < levels; ++l) {
+            const int d = l % D;
+            if (widest) {
+                list_ptrs();
+                KDT_LAUNCH widest_kernel<<<grid_for((int64_t)1 << l), BT, 0, s>>>(lp, total, l, d_points, D, node_dim);
+                KDT_LAUNCH assign_widest_kernel<<<g, BT, 0, s>>>(lp, total, l, node_dim, d_points, D, side, nodes);
+            } else if (D == 1 && l > 0) {
+                // no list is partitioned that could note the next level's sides
+                KDT_LAUNCH assign_kernel<<<g, BT, 0, s>>>(lists[0], total, l, sub_log2, 1, nullptr, nullptr, d_points, D, side,
+                                                          nodes, ids);
+            }
+            // the lists to partition, TOP_LISTS or as many as there are spares at a time
+            int todo[8], count = 0;
+            for (int e = 0; e < D; ++e)
+                if (widest || e != d)
+                    todo[count++] = e;
+            const int step = std::min(TOP_LISTS, spares);
+            for (int c = 0; c < count; c += step) {
+                const int ny = std::min(step, count - c);
+                PartArgs pa;
+                pa.next = -1;
+                for (int i = 0; i < ny; ++i) {
+                    pa.in[i] = lists[todo[c + i]];
+                    pa.out[i] = spare[i];
+                    if (!widest && l + 1 < levels && todo[c + i] == (l + 1) % D)
+                        pa.next = i;
                 }
+                pa.side = side;
+                pa.state = state;
+                pa.ticket = ticket;
+                state += (size_t)ny * top_tiles;
+                ticket += ny;
+                pa.n = n;
+                pa.l = l;
+                pa.tiles = top_tiles;
+                pa.side_next = side_next;
+                pa.pts = d_points;
+                pa.D = D;
+                pa.nodes = nodes;
+                pa.ids = ids;
+                KDT_LAUNCH part_kernel<<<dim3((unsigned)top_tiles, (unsigned)ny), BT, 0, s>>>(pa);
+                for (int i = 0; i < ny; ++i)
+                    std::swap(lists[todo[c + i]], spare[i]);
+            }
+            if (!widest && D > 1)
+                std::swap(side, side_next);
+            KDT_CUDA(cudaGetLastError());
+        }
+    } else {
+        for (int l = 0; l < levels; ++l) {
+            const int d = l % D;
+            KDT_LAUNCH assign_kernel<<<g, BT, 0, s>>>(lists[d], total, l, sub_log2, T, d_off, tree_of, d_points, D, side, nodes,
+                                                      ids);
+            for (int e = 0; e < D; ++e) {
+                if (e == d)
+                    continue;
+                KDT_LAUNCH part_reduce_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, sub_log2, T, d_off, tree_of,
+                                                                              side, tiles);
+                KDT_LAUNCH part_tiles_kernel<<<1, 1024, 0, s>>>(tiles, ptiles);
+                KDT_LAUNCH part_scatter_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, sub_log2, T, d_off, tree_of,
+                                                                               side, tiles, spare[0]);
+                std::swap(lists[e], spare[0]);
             }
             KDT_CUDA(cudaGetLastError());
         }
-        return KDT_OK;
     }
-    for (int l = 0; l <= maxH; ++l) {
-        const int d = l % D;
-        KDT_LAUNCH assign_kernel<<<g, BT, 0, s>>>(lists[d], total, l, T, d_off, tree_of, d_points, D, side, nodes, ids);
-        for (int e = 0; e < D; ++e) {
-            if (e == d)
-                continue;
-            // next level that splits on e
-            int nl = l + ((e - d + D) % D);
-            if (nl > maxH)
-                continue;
-            KDT_LAUNCH part_reduce_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, T, d_off, tree_of, side, tiles);
-            KDT_LAUNCH part_tiles_kernel<<<1, 1024, 0, s>>>(tiles, ptiles);
-            KDT_LAUNCH part_scatter_kernel<<<(unsigned)ptiles, BT, 0, s>>>(lists[e], total, l, T, d_off, tree_of, side, tiles,
-                                                                spare);
-            std::swap(lists[e], spare);
-        }
-        KDT_CUDA(cudaGetLastError());
-    }
-    return KDT_OK;
+
+    SubArgs sa;
+    list_ptrs();
+    sa.lists = lp;
+    sa.off = d_off;
+    sa.first_job = d_job;
+    sa.total = total;
+    sa.T = T;
+    sa.D = D;
+    sa.widest = widest;
+    sa.pts = d_points;
+    sa.place = (uint16_t *)(B + o_place);
+    sa.nodes = nodes;
+    sa.ids = ids;
+    return sub_log2 == SUB_LOG2_SMALL ? launch_sub<SUB_LOG2_SMALL>(sa, jobs, s)
+                                      : launch_sub<SUB_LOG2_LARGE>(sa, jobs, s);
 }
 
 }  // namespace kdt
