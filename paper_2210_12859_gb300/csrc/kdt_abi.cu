@@ -75,73 +75,63 @@ bool debug_alloc_fails()
 
 // ---------------------------------------------------------------- query order
 
-__device__ __forceinline__ uint32_t spread3(uint32_t x)
+// The path of a query's descent from the root, a bit a level, over the first
+// `levels` levels: the bits of the node reached (a tree of fewer levels is
+// walked to its last full one and the path padded).  Queries in this order
+// share the nodes of their walks for as many levels as the order resolves,
+// whatever the points' density and dimensions: a Morton code cuts the space on
+// planes of its own and sees three coordinates.  One dependent 4-byte load a
+// level, the upper levels from L1.
+// LAYOUT as in kdt_internal.cuh; nodes, n: the tree's.
+template <int LAYOUT>
+__device__ __forceinline__ uint32_t descent_path(const float *__restrict__ q, int D, const float4 *__restrict__ nodes,
+                                                 int64_t n, int levels)
 {
-    x &= 0x3ffu;
-    x = (x | (x << 16)) & 0x030000ffu;
-    x = (x | (x << 8)) & 0x0300f00fu;
-    x = (x | (x << 4)) & 0x030c30c3u;
-    x = (x | (x << 2)) & 0x09249249u;
-    return x;
+    constexpr int STRIDE = LAYOUT == 2 ? 8 : 4;
+    const float *c = reinterpret_cast<const float *>(nodes);
+    const int full = min(levels, floor_log2((uint64_t)n));  // the levels above the last are full
+    uint32_t v = 1;  // node + 1
+    int dim = 0;
+    for (int l = 0; l < full; ++l) {
+        const size_t at = (size_t)(v - 1) * STRIDE;
+        if (LAYOUT == 3)
+            dim = (int)(__float_as_uint(__ldg(c + at + 3)) >> NODE_DIM_SHIFT);
+        const bool right = __ldg(q + dim) > __ldg(c + at + dim);
+        v = 2 * v + right;
+        if (LAYOUT != 3)
+            dim = dim + 1 == D ? 0 : dim + 1;
+    }
+    return (v - (1u << full)) << (levels - full);
 }
 
-// Forests: the tree's index (tbits bits) above the high 32 - tbits bits of the
-// query's 30-bit Morton code (its first min(D, 3) coordinates, 10 bits each
-// inside the bounding box of the query's tree), so that one sort orders by
-// tree and along the curve within a tree.
-__global__ void morton_kernel(const float *__restrict__ qs, int64_t Q, int D, const float *__restrict__ bbox, int T,
-                              int tbits, const int64_t *__restrict__ q_off, uint32_t *__restrict__ keys)
+template <int LAYOUT>
+__global__ void path_kernel(const float *__restrict__ qs, int64_t Q, int D, const float4 *__restrict__ nodes,
+                            int64_t n, int levels, uint32_t *__restrict__ keys)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x)
+        keys[i] = descent_path<LAYOUT>(qs + i * D, D, nodes, n, levels);
+}
+
+// Forests: the tree's index above the path in its tree, so that one sort
+// orders by tree and within it.
+template <int LAYOUT>
+__global__ void forest_path_kernel(const float *__restrict__ qs, int64_t Q, int D, const float4 *__restrict__ nodes,
+                                   int T, const int64_t *__restrict__ node_off, const int64_t *__restrict__ q_off,
+                                   int levels, uint32_t *__restrict__ keys)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x) {
-        int t = 0;
         int lo = 0, hi = T - 1;
         while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
+            const int mid = (lo + hi + 1) >> 1;
             if (q_off[mid] <= i)
                 lo = mid;
             else
                 hi = mid - 1;
         }
-        t = lo;
-        const float *bb = bbox + 6 * t;
-        uint32_t code = 0;
-        for (int j = 0; j < 3 && j < D; ++j) {
-            float ext = bb[3 + j] - bb[j];
-            float x = ext > 0.f ? (qs[i * D + j] - bb[j]) / ext : 0.f;
-            x = fminf(fmaxf(x, 0.f), 1.f);
-            uint32_t c = (uint32_t)fminf(x * 1024.f, 1023.f);
-            code |= spread3(c) << (2 - j);
-        }
-        keys[i] = (uint32_t)((((uint64_t)t << 32) | ((uint64_t)code << 2)) >> tbits);
-    }
-}
-
-// Single trees: the path of the query's descent from the root, a bit a level,
-// over `levels` full levels.  Queries in this order share the nodes of their
-// walks for as many levels as the order resolves, whatever the points'
-// density and dimensions: a Morton code cuts the space on planes of its own
-// and sees three coordinates.  One dependent 4-byte load a level, the upper
-// levels from L1.
-// LAYOUT as in kdt_internal.cuh.
-template <int LAYOUT>
-__global__ void path_kernel(const float *__restrict__ qs, int64_t Q, int D, const float4 *__restrict__ nodes,
-                            int levels, uint32_t *__restrict__ keys)
-{
-    constexpr int STRIDE = LAYOUT == 2 ? 8 : 4;
-    const float *c = reinterpret_cast<const float *>(nodes);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t v = 1;  // node + 1
-        int dim = 0;
-        for (int l = 0; l < levels; ++l) {
-            const size_t at = (size_t)(v - 1) * STRIDE;
-            if (LAYOUT == 3)
-                dim = (int)(__float_as_uint(__ldg(c + at + 3)) >> NODE_DIM_SHIFT);
-            const bool right = __ldg(qs + i * D + dim) > __ldg(c + at + dim);
-            v = 2 * v + right;
-            if (LAYOUT != 3)
-                dim = dim + 1 == D ? 0 : dim + 1;
-        }
-        keys[i] = v - (1u << levels);
+        const int64_t base = node_off[lo], n = node_off[lo + 1] - base;
+        const uint32_t path =
+            n > 0 ? descent_path<LAYOUT>(qs + i * D, D, nodes + base * LayoutTraits<LAYOUT>::NF, n, levels) : 0u;
+        keys[i] = ((uint32_t)lo << levels) | path;
     }
 }
 
@@ -244,10 +234,10 @@ int query_order(const kdt_tree *t, const float *d_q, int64_t Q, bool cost, void 
         // the levels above the last are full
         const int levels = std::min(floor_log2((uint64_t)t->N), path_bits(Q));
         switch (t->layout) {
-        case 0: KDT_LAUNCH path_kernel<0><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
-        case 1: KDT_LAUNCH path_kernel<1><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
-        case 3: KDT_LAUNCH path_kernel<3><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys); break;
-        default: KDT_LAUNCH path_kernel<2><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, levels, o.keys);
+        case 0: KDT_LAUNCH path_kernel<0><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, t->N, levels, o.keys); break;
+        case 1: KDT_LAUNCH path_kernel<1><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, t->N, levels, o.keys); break;
+        case 3: KDT_LAUNCH path_kernel<3><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, t->N, levels, o.keys); break;
+        default: KDT_LAUNCH path_kernel<2><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, t->D, t->nodes, t->N, levels, o.keys);
         }
         bits = std::max(levels, 1);
         lo = 0;
@@ -258,21 +248,25 @@ int query_order(const kdt_tree *t, const float *d_q, int64_t Q, bool cost, void 
     return KDT_OK;
 }
 
-// the same for a forest's queries: by tree, along the Morton curve within one
-static int forest_order(const kdt_forest *f, const float *d_q, int64_t Q, const int64_t *d_qoff, void *scratch,
-                        uint32_t **perm_out, cudaStream_t s)
+// the same for a forest's queries: by tree, then by path; max_q: the most
+// queries of one tree
+static int forest_order(const kdt_forest *f, const float *d_q, int64_t Q, int64_t max_q, const int64_t *d_qoff,
+                        void *scratch, uint32_t **perm_out, cudaStream_t s)
 {
     OrderArrays o(scratch, Q);
     const int T = f->f.T, D = f->f.D;
     const int tbits = T > 1 ? floor_log2((uint64_t)(T - 1)) + 1 : 0;
-    KDT_LAUNCH morton_kernel<<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, f->bbox, T, tbits, d_qoff, o.keys);
+    // whole passes, rounded to the nearest; the bits that one has left go to the path
+    const int passes = std::min(4, std::max((tbits + path_bits(max_q) + 4) / 8, (tbits + 7) / 8));
+    const int levels = std::max(std::min(8 * passes, 31) - tbits, 0);
+    const int64_t *no = f->f.d_offsets;
+    switch (layout_of(D)) {
+    case 0: KDT_LAUNCH forest_path_kernel<0><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, f->nodes, T, no, d_qoff, levels, o.keys); break;
+    case 1: KDT_LAUNCH forest_path_kernel<1><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, f->nodes, T, no, d_qoff, levels, o.keys); break;
+    default: KDT_LAUNCH forest_path_kernel<2><<<grid_1d(Q), 256, 0, s>>>(d_q, Q, D, f->nodes, T, no, d_qoff, levels, o.keys);
+    }
     KDT_CUDA(cudaGetLastError());
-    // a Morton code wastes bits on empty space and, with fewer than three
-    // coordinates, on those missing
-    const int dims = std::min(D, 3);
-    const int code = ((path_bits(Q / T) + 2) * 3 + dims - 1) / dims;
-    const int bits = std::min(32, (tbits + code + 7) / 8 * 8);
-    KDT_TRY(radix_sort_batch(&o.keys, &o.perm, &o.tk, &o.tv, Q, 1, Q, 32 - bits, bits, true, o.rs, s));
+    KDT_TRY(radix_sort_batch(&o.keys, &o.perm, &o.tk, &o.tv, Q, 1, Q, 0, std::max(levels + tbits, 1), true, o.rs, s));
     *perm_out = o.perm;
     return KDT_OK;
 }
@@ -782,6 +776,7 @@ struct ForestGraph {
     float r2 = 0;
     int flags = 0;
     std::vector<int64_t> qoff;
+    int64_t max_q = 0;         // most queries of one tree
     void *scratch = nullptr;   // persistent scratch referenced by the graph
     size_t scratch_bytes = 0;
     int threads = 0;           // launch parameters the graph was captured with
@@ -833,6 +828,8 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
     int rc = e == cudaSuccess ? KDT_OK : cuda_error(e, "forest allocation", __FILE__, __LINE__);
     if (rc == KDT_OK)
         rc = build_forest(d_points, h_off, T, D, f->nodes, f->ids, f->bbox, f->err, s);
+    if (rc == KDT_OK)
+        rc = build_box_forest(f, s);
     if (rc == KDT_OK) {
         int h = 0;
         e = cudaMemcpyAsync(&h, f->err, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -860,7 +857,7 @@ static int forest_enqueue(kdt_forest *f, ForestGraph *g, const float *d_q, int64
     c.take<int64_t>(T + 1);  // query offsets (filled before)
     QueryArgs a;
     if (flags & KDT_MORTON)
-        KDT_TRY(forest_order(f, d_q, Q, d_qoff, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
+        KDT_TRY(forest_order(f, d_q, Q, g->max_q, d_qoff, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
     a.nodes = f->nodes;
     a.ids = f->ids;
     a.D = f->f.D;
@@ -879,6 +876,8 @@ static int forest_enqueue(kdt_forest *f, ForestGraph *g, const float *d_q, int64
     a.claim_steps = f->claim_steps > 0 ? f->claim_steps : default_claim_steps_k(k);
     a.inline_depth = f->inline_depth == 1 ? 1 : 2;
     a.light_run = f->light_run > 0 ? f->light_run : 1;
+    if (box_query_serves(a, flags, MODE_RESULTS))
+        return launch_box_forest(f, a, s);
     return launch_query(layout_of(f->f.D), a, !(flags & KDT_UNORDERED), 0, true, s);
 }
 
@@ -996,7 +995,10 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
             a.counter = counter;
             a.staged = (flags & KDT_NO_STAGE) ? 0 : staged_for_levels(n, 6);
             a.claim_steps = default_claim_steps_k(k);
-            KDT_TRY(launch_query(layout, a, !(flags & KDT_UNORDERED), 0, false, s));
+            if (box_query_serves(a, flags, MODE_RESULTS))
+                KDT_TRY(launch_box_query(layout, ((const BoxRef *)f->box_host)[i], a, MODE_RESULTS, s));
+            else
+                KDT_TRY(launch_query(layout, a, !(flags & KDT_UNORDERED), 0, false, s));
         }
         return KDT_OK;
     }
@@ -1006,7 +1008,7 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         g = new ForestGraph();
         f->graph = g;
     }
-    const bool same = g->exec && g->q == d_q && g->ids == d_ids && g->d2 == d_d2 && g->k == k && g->r2 == r2 &&
+    const bool same = g->q == d_q && g->ids == d_ids && g->d2 == d_d2 && g->k == k && g->r2 == r2 &&
                       g->flags == flags && g->threads == f->threads && g->claim_steps == f->claim_steps &&
                       g->inline_depth == f->inline_depth && g->light_run == f->light_run &&
                       g->qoff.size() == (size_t)T + 1 &&
@@ -1025,7 +1027,7 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
             KDT_CUDA(cudaMalloc(&g->scratch, need));
             g->scratch_bytes = need;
         }
-        g->q = d_q;
+        g->q = nullptr;  // set once the offsets are on their way
         g->ids = d_ids;
         g->d2 = d_d2;
         g->k = k;
@@ -1036,16 +1038,25 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         g->inline_depth = f->inline_depth;
         g->light_run = f->light_run;
         g->qoff.assign(h_qoff, h_qoff + T + 1);
+        g->max_q = 1;
+        for (int i = 0; i < T; ++i)
+            g->max_q = std::max(g->max_q, h_qoff[i + 1] - h_qoff[i]);
     }
     Carve c{(char *)g->scratch};
     c.take<unsigned long long>(8);
     int64_t *d_qoff = c.take<int64_t>(T + 1);
-    if (!same)
-        KDT_CUDA(cudaMemcpyAsync(d_qoff, h_qoff, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     KDT_CUDA(cudaStreamIsCapturing(s, &cs));
-    if (cs != cudaStreamCaptureStatusNone || s == nullptr)
+    if (!same) {
+        KDT_CUDA(cudaMemcpyAsync(d_qoff, h_qoff, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        // a captured copy has not run: the next call makes its own
+        if (cs == cudaStreamCaptureStatusNone)
+            g->q = d_q;
+    }
+    // arguments seen for the first time are enqueued as they are; a graph is
+    // captured when they come again (capture and instantiation cost more than
+    // the launches that one replay saves)
+    if (!same || cs != cudaStreamCaptureStatusNone || s == nullptr)
         return forest_enqueue(f, g, d_q, Q, d_qoff, k, r2, flags, d_ids, d_d2, s);
     if (!g->exec) {
         cudaGraph_t graph = nullptr;
@@ -1192,9 +1203,11 @@ void kdt_forest_free(kdt_forest *f)
     }
     cudaFree(f->nodes);
     cudaFree(f->ids);
+    cudaFree(f->box_data);
     cudaFree(f->bbox);
     cudaFree(f->f.d_offsets);
     cudaFree(f->err);
+    delete[] (BoxRef *)f->box_host;
     delete[] f->h_offsets;
     delete f;
 }

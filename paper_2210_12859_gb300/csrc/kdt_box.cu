@@ -1,5 +1,6 @@
 // Build of the box tree and the kNN kernels that walk it (layout in kdt_box.cuh).
 #include <algorithm>
+#include <vector>
 
 #include "kdt_box.cuh"
 
@@ -88,15 +89,53 @@ __device__ __forceinline__ void reduce_boxes(float4 *rec, uint32_t v, int count,
 // (each row of a bucket is contiguous, and neighbouring threads read
 // neighbouring rows) and the latency of the walk, whose upper nodes are shared
 // by the block.
+struct BoxBuild {
+    const float4 *nodes;
+    const int32_t *ids;
+    int64_t N;
+    int D;
+    float4 *rec, *grp;
+    // forests: the trees, their first nodes and their first blocks
+    int T;
+    const BoxRef *trees;
+    const int64_t *off;
+    const int32_t *first_block;
+};
+
+// the block's tree in `a` (nodes, ids, N, rec, grp) and its number within the tree
 template <int LAYOUT>
-__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(const float4 *__restrict__ nodes,
-                                                                      const int32_t *__restrict__ ids, int N, int D,
-                                                                      float4 *__restrict__ rec,
-                                                                      float4 *__restrict__ grp)
+__device__ __forceinline__ uint32_t box_build_tree(BoxBuild &a)
+{
+    if (a.T == 1)
+        return blockIdx.x;
+    int lo = 0, hi = a.T - 1;  // last tree that starts at or before the block
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (a.first_block[mid] <= (int)blockIdx.x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    const int64_t base = a.off[lo];
+    a.N = a.off[lo + 1] - base;
+    a.nodes += base * LayoutTraits<LAYOUT>::NF;
+    a.ids = a.ids ? a.ids + base : nullptr;
+    a.rec = const_cast<float4 *>(a.trees[lo].rec);
+    a.grp = const_cast<float4 *>(a.trees[lo].grp);
+    return blockIdx.x - a.first_block[lo];
+}
+
+template <int LAYOUT>
+__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(BoxBuild a)
 {
     constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    const uint32_t block = box_build_tree<LAYOUT>(a);
+    const float4 *__restrict__ nodes = a.nodes;
+    const int32_t *__restrict__ ids = a.ids;
+    float4 *rec = a.rec, *grp = a.grp;
+    const int N = (int)a.N, D = a.D;
     const BoxShape sh(N);
-    const uint32_t first = blockIdx.x * BOX_BUILD_THREADS, i = first + threadIdx.x;
+    const uint32_t first = block * BOX_BUILD_THREADS, i = first + threadIdx.x;
     const int count = (int)min((int64_t)BOX_BUILD_THREADS, sh.buckets - (int64_t)first);
     Box<NC> box;
     box.none();
@@ -174,11 +213,16 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(const float
         reduce_boxes<NC>(rec, (uint32_t)sh.buckets + i, count, box);
 }
 
-// Thread i: node v0 + i of a level whose records are complete
-template <int NC>
-__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(float4 *__restrict__ rec, uint32_t v0)
+// Thread i: node i of the level `up` levels above the buckets, whose records
+// are complete
+template <int LAYOUT>
+__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(BoxBuild a, int up)
 {
-    const uint32_t first = blockIdx.x * BOX_BUILD_THREADS, i = first + threadIdx.x;
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    const uint32_t block = box_build_tree<LAYOUT>(a);
+    float4 *rec = a.rec;
+    const uint32_t v0 = 1u << (BoxShape(a.N).LB - up);
+    const uint32_t first = block * BOX_BUILD_THREADS, i = first + threadIdx.x;
     const int count = (int)min((uint32_t)BOX_BUILD_THREADS, v0 - first);
     Box<NC> box;
     box.none();
@@ -216,14 +260,16 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(float4 *__
 constexpr int BOX_RECORD_LANES = 4;
 constexpr int BOX_FREE_LANES = 24;
 
-template <int LAYOUT, int K, int MODE>
+// FOREST: a lane's query finds its tree by its place in the query offsets.
+template <int LAYOUT, int K, int MODE, bool FOREST>
 __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(const QueryArgs a, const BoxArgs b)
 {
     constexpr int NC = LayoutTraits<LAYOUT>::NC;
     using List = typename std::conditional<(K <= MAX_REG_K), RegList<K <= MAX_REG_K ? K : 1>, SmemList>::type;
     extern __shared__ float4 s_dyn[];
     const int64_t ngate = (MODE == MODE_BOUNDED && a.n_gate) ? (int64_t)*a.n_gate : INT64_MAX;
-    const uint32_t cap = a.step_cap ? a.step_cap : 3u * (uint32_t)a.N + 3u;
+    uint32_t cap = a.step_cap ? a.step_cap : 3u * (uint32_t)a.N + 3u;
+    BoxRef tree = b.tree;
     bool gated = false;
     double ratio = 0.0;
     float q[NC];
@@ -265,7 +311,7 @@ __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(co
                         gated = false;
                         r2 = a.r2;
                         list.init(a.k, r2);
-                        w.start(b.root, b.root_mask, s_far);
+                        w.start(tree.leaf, s_far);
                         steps = 0;
                         busy = true;
                     } else if (gated && full && list.cull() > 0.f && r2 < __int_as_float(0x7f800000)) {
@@ -294,16 +340,28 @@ __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(co
                     qi = a.perm ? (int64_t)a.perm[slot] : slot;
                     gated = MODE == MODE_BOUNDED && slot < ngate;
                     r2 = gated ? a.r2q[qi] : a.r2;
+                    if constexpr (FOREST) {
+                        int lo = 0, hi = a.T - 1;  // last tree whose queries start at or before qi
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (a.q_off[mid] <= qi)
+                                lo = mid;
+                            else
+                                hi = mid - 1;
+                        }
+                        tree = b.trees[lo];
+                        cap = 3u * (uint32_t)(a.node_off[lo + 1] - a.node_off[lo]) + 3u;
+                    }
                     load_query<LAYOUT>(a.queries, qi, a.D, q);
                     list.init(a.k, r2);
-                    w.start(b.root, b.root_mask, s_far);
+                    w.start(tree.leaf, s_far);
                     steps = 0;
                     // no distance to a NaN query passes a test
                     bool nan = false;
 #pragma unroll
                     for (int j = 0; j < NC; ++j)
                         nan = nan || q[j] != q[j];
-                    busy = !nan;
+                    busy = !nan && (!FOREST || tree.leaf > 0);
                 } else {
                     exhausted = true;
                 }
@@ -314,16 +372,16 @@ __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(co
         }
         // records, until few lanes are left on them
         for (;;) {
-            if (busy && w.v < b.leaf) {
+            if (busy && w.v < tree.leaf) {
                 ++steps;
-                busy = w.template step<NC>(b.rec, q, one, list.cull(), stride);
+                busy = w.template step<NC>(tree.rec, q, one, list.cull(), stride);
             }
-            if (__popc(__ballot_sync(0xffffffffu, busy && w.v < b.leaf)) <= BOX_RECORD_LANES)
+            if (__popc(__ballot_sync(0xffffffffu, busy && w.v < tree.leaf)) <= BOX_RECORD_LANES)
                 break;
         }
-        if (busy && w.v >= b.leaf) {
+        if (busy && w.v >= tree.leaf) {
             ++steps;
-            box_bucket<NC, K>(b, w.v - b.leaf, q, one, list);
+            box_bucket<NC, K>(tree, w.v - tree.leaf, q, one, list);
             busy = w.pop(list.cull(), stride);
         }
         if (steps > cap)
@@ -337,10 +395,10 @@ __global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(co
     }
 }
 
-template <int LAYOUT, int K, int MODE>
+template <int LAYOUT, int K, int MODE, bool FOREST>
 int launch_box_one(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
 {
-    const void *fn = (const void *)box_knn_kernel<LAYOUT, K, MODE>;
+    const void *fn = (const void *)box_knn_kernel<LAYOUT, K, MODE, FOREST>;
     // few queries: small blocks, so that they spread over the SMs
     int threads = BOX_THREADS;
     while (threads > 32 && a.Q < (int64_t)num_sms() * threads)
@@ -354,89 +412,160 @@ int launch_box_one(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
     grid = std::min<int64_t>(grid, (a.Q + threads - 1) / threads);
     if (grid * threads < a.Q)
         KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
-    KDT_LAUNCH box_knn_kernel<LAYOUT, K, MODE><<<(unsigned)grid, threads, smem, s>>>(a, b);
+    KDT_LAUNCH box_knn_kernel<LAYOUT, K, MODE, FOREST><<<(unsigned)grid, threads, smem, s>>>(a, b);
     KDT_CUDA(cudaGetLastError());
     return KDT_OK;
 }
 
-template <int LAYOUT, int MODE>
+template <int LAYOUT, int MODE, bool FOREST>
 int launch_box_k(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
 {
     if (a.k <= 1)
-        return launch_box_one<LAYOUT, 1, MODE>(a, b, s);
+        return launch_box_one<LAYOUT, 1, MODE, FOREST>(a, b, s);
     if (a.k <= 2)
-        return launch_box_one<LAYOUT, 2, MODE>(a, b, s);
+        return launch_box_one<LAYOUT, 2, MODE, FOREST>(a, b, s);
     if (a.k <= 4)
-        return launch_box_one<LAYOUT, 4, MODE>(a, b, s);
+        return launch_box_one<LAYOUT, 4, MODE, FOREST>(a, b, s);
     if (a.k <= 8)
-        return launch_box_one<LAYOUT, 8, MODE>(a, b, s);
+        return launch_box_one<LAYOUT, 8, MODE, FOREST>(a, b, s);
     if (a.k <= 16)
-        return launch_box_one<LAYOUT, 16, MODE>(a, b, s);
-    return launch_box_one<LAYOUT, 64, MODE>(a, b, s);
+        return launch_box_one<LAYOUT, 16, MODE, FOREST>(a, b, s);
+    return launch_box_one<LAYOUT, 64, MODE, FOREST>(a, b, s);
 }
 
-template <int LAYOUT>
-int build_box_layout(const kdt_tree *t, cudaStream_t s)
+// blocks of the launch `up` levels above the buckets of a tree of n points
+int64_t box_blocks(int64_t n, int up)
 {
-    constexpr int NC = LayoutTraits<LAYOUT>::NC;
-    const BoxShape sh(t->N);
-    KDT_LAUNCH box_leaf_kernel<LAYOUT><<<(unsigned)((sh.buckets + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS),
-                                         BOX_BUILD_THREADS, 0, s>>>(t->nodes, t->ids, (int)t->N, t->D, t->box_rec,
-                                                                     t->box_grp);
-    KDT_CUDA(cudaGetLastError());
-    // a block writes the boxes of five levels of the record tree (256 nodes
-    // and their 64, 16, 4 and 1 ancestors), the next launch starts above them
-    for (int l = sh.LB - 10; l >= 1; l -= 10) {
-        const uint32_t v0 = 1u << l;
-        KDT_LAUNCH box_upper_kernel<NC><<<(v0 + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS, BOX_BUILD_THREADS, 0,
-                                          s>>>(t->box_rec, v0);
+    const BoxShape sh(n);
+    if (n < 1 || sh.LB - up < (up ? 1 : 0))
+        return 0;
+    return (((int64_t)1 << (sh.LB - up)) + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS;
+}
+
+// A block writes the boxes of five levels of the record tree (256 nodes and
+// their 64, 16, 4 and 1 ancestors), the next launch starts above them; `blocks`
+// and `first` (device, T > 1) of each launch, none after one without blocks.
+constexpr int BOX_LAUNCHES = 3;  // LB <= 26
+constexpr int BOX_LAUNCH_LEVELS = 10;
+
+template <int LAYOUT>
+int build_box_layout(BoxBuild a, const int64_t *blocks, const int32_t *const *first, cudaStream_t s)
+{
+    for (int r = 0; r < BOX_LAUNCHES && blocks[r] > 0; ++r) {
+        a.first_block = first[r];
+        if (r == 0)
+            KDT_LAUNCH box_leaf_kernel<LAYOUT><<<(unsigned)blocks[r], BOX_BUILD_THREADS, 0, s>>>(a);
+        else
+            KDT_LAUNCH box_upper_kernel<LAYOUT><<<(unsigned)blocks[r], BOX_BUILD_THREADS, 0, s>>>(
+                a, BOX_LAUNCH_LEVELS * r);
         KDT_CUDA(cudaGetLastError());
     }
     return KDT_OK;
 }
 
+int build_boxes(int layout, const BoxBuild &a, const int64_t *blocks, const int32_t *const *first, cudaStream_t s)
+{
+    switch (layout) {
+    case 0: return build_box_layout<0>(a, blocks, first, s);
+    case 1: return build_box_layout<1>(a, blocks, first, s);
+    case 3: return build_box_layout<3>(a, blocks, first, s);
+    default: return build_box_layout<2>(a, blocks, first, s);
+    }
+}
+
+// float4s of a tree's records, rounded up to a 128-byte line, and of its groups
+size_t box_rec_size(int64_t n, int D) { return ((size_t)BoxShape(n).records() * 2 * box_coords(D) + 7) & ~(size_t)7; }
+size_t box_grp_size(int64_t n, int D) { return (size_t)BoxShape(n).groups() * 2 * (box_coords(D) + 1); }
+
 }  // namespace
 
 cudaError_t box_tree_alloc(kdt_tree *t)
 {
-    const BoxShape sh(t->N);
-    const size_t rec = (size_t)sh.records() * 2 * box_coords(t->D);
-    const size_t grp = (size_t)sh.groups() * 2 * (box_coords(t->D) + 1);
-    // a group starts on a 128-byte line where its size allows (records of 96
-    // bytes: rounded up to a line)
-    const size_t at = (rec + 7) & ~(size_t)7;
-    const cudaError_t e = cudaMalloc(&t->box_rec, (at + grp) * sizeof(float4));
-    t->box_grp = t->box_rec + at;
+    const size_t rec = box_rec_size(t->N, t->D);
+    const cudaError_t e = cudaMalloc(&t->box_rec, (rec + box_grp_size(t->N, t->D)) * sizeof(float4));
+    t->box_grp = t->box_rec + rec;
     return e;
 }
 
 int build_box_tree(const kdt_tree *t, cudaStream_t s)
 {
-    switch (t->layout) {
-    case 0: return build_box_layout<0>(t, s);
-    case 1: return build_box_layout<1>(t, s);
-    case 3: return build_box_layout<3>(t, s);
-    default: return build_box_layout<2>(t, s);
+    BoxBuild a = {t->nodes, t->ids, t->N, t->D, t->box_rec, t->box_grp, 1, nullptr, nullptr, nullptr};
+    int64_t blocks[BOX_LAUNCHES];
+    const int32_t *first[BOX_LAUNCHES] = {nullptr, nullptr, nullptr};
+    for (int r = 0; r < BOX_LAUNCHES; ++r)
+        blocks[r] = box_blocks(t->N, BOX_LAUNCH_LEVELS * r);
+    return build_boxes(t->layout, a, blocks, first, s);
+}
+
+int build_box_forest(kdt_forest *f, cudaStream_t s)
+{
+    const int T = f->f.T, D = f->f.D;
+    // [records and groups of every tree][BoxRef of every tree][first blocks of every launch]
+    size_t at = 0;
+    std::vector<size_t> rec(T), grp(T);
+    std::vector<int32_t> first((size_t)BOX_LAUNCHES * (T + 1), 0);
+    int64_t blocks[BOX_LAUNCHES] = {0, 0, 0};
+    for (int i = 0; i < T; ++i) {
+        const int64_t n = f->h_offsets[i + 1] - f->h_offsets[i];
+        for (int r = 0; r < BOX_LAUNCHES; ++r) {
+            first[(size_t)r * (T + 1) + i] = (int32_t)blocks[r];
+            blocks[r] += box_blocks(n, BOX_LAUNCH_LEVELS * r);
+        }
+        rec[i] = at;
+        at += n ? box_rec_size(n, D) : 0;
+        grp[i] = at;
+        at += n ? (box_grp_size(n, D) + 7) & ~(size_t)7 : 0;
+    }
+    for (int r = 0; r < BOX_LAUNCHES; ++r)
+        first[(size_t)r * (T + 1) + T] = (int32_t)blocks[r];
+    const size_t data = at * sizeof(float4), refs = (size_t)T * sizeof(BoxRef);
+    char *p = nullptr;
+    KDT_CUDA(cudaMalloc(&p, data + refs + first.size() * sizeof(int32_t)));
+    f->box_data = (float4 *)p;
+    f->box_refs = p + data;
+    BoxRef *ref = new BoxRef[T];
+    f->box_host = ref;
+    for (int i = 0; i < T; ++i) {
+        const int64_t n = f->h_offsets[i + 1] - f->h_offsets[i];
+        ref[i] = n ? box_ref(n, f->box_data + rec[i], f->box_data + grp[i]) : BoxRef{nullptr, nullptr, 0, 0};
+    }
+    KDT_CUDA(cudaMemcpyAsync(p + data, ref, refs, cudaMemcpyHostToDevice, s));
+    KDT_CUDA(cudaMemcpyAsync(p + data + refs, first.data(), first.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    BoxBuild a = {f->nodes, f->ids, f->f.total, D, nullptr, nullptr, T, (const BoxRef *)f->box_refs, f->f.d_offsets,
+                  nullptr};
+    if (T == 1 && f->f.total) {
+        a.rec = f->box_data + rec[0];
+        a.grp = f->box_data + grp[0];
+    }
+    const int32_t *d_first[BOX_LAUNCHES];
+    for (int r = 0; r < BOX_LAUNCHES; ++r)
+        d_first[r] = (const int32_t *)(p + data + refs) + (size_t)r * (T + 1);
+    return build_boxes(layout_of(D), a, blocks, d_first, s);
+}
+
+int launch_box_query(int layout, const BoxRef &tree, const QueryArgs &a, int mode, cudaStream_t s)
+{
+    BoxArgs b;
+    b.tree = tree;
+    const bool bounded = mode == MODE_BOUNDED;
+    // the groups hold coordinates and ids alike for layouts 0 and 3
+    switch (layout) {
+    case 0:
+    case 3:
+        return bounded ? launch_box_k<0, MODE_BOUNDED, false>(a, b, s) : launch_box_k<0, MODE_RESULTS, false>(a, b, s);
+    case 1: return launch_box_k<1, MODE_RESULTS, false>(a, b, s);
+    default: return launch_box_k<2, MODE_RESULTS, false>(a, b, s);
     }
 }
 
-int launch_box_query(const kdt_tree *t, const QueryArgs &a, int mode, cudaStream_t s)
+int launch_box_forest(const kdt_forest *f, const QueryArgs &a, cudaStream_t s)
 {
-    const BoxShape sh(t->N);
     BoxArgs b;
-    b.rec = t->box_rec;
-    b.grp = t->box_grp;
-    b.leaf = (uint32_t)sh.buckets;
-    b.big = (uint32_t)sh.big;
-    b.root = sh.LB & 1 ? 0u : 1u;
-    b.root_mask = sh.LB & 1 ? 12u : 15u;
-    const bool bounded = mode == MODE_BOUNDED;
-    // the groups hold coordinates and ids alike for layouts 0 and 3
-    switch (t->layout) {
-    case 0:
-    case 3: return bounded ? launch_box_k<0, MODE_BOUNDED>(a, b, s) : launch_box_k<0, MODE_RESULTS>(a, b, s);
-    case 1: return launch_box_k<1, MODE_RESULTS>(a, b, s);
-    default: return launch_box_k<2, MODE_RESULTS>(a, b, s);
+    b.trees = (const BoxRef *)f->box_refs;
+    switch (layout_of(f->f.D)) {
+    case 0: return launch_box_k<0, MODE_RESULTS, true>(a, b, s);
+    case 1: return launch_box_k<1, MODE_RESULTS, true>(a, b, s);
+    default: return launch_box_k<2, MODE_RESULTS, true>(a, b, s);
     }
 }
 

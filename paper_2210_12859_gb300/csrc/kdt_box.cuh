@@ -167,10 +167,12 @@ struct BoxWalk {
     uint32_t mask;  // children of v to look at, while v has a record
     unsigned long long trail;
     float *far;     // of the next record down; `stride` floats to the next
-    __device__ __forceinline__ void start(uint32_t root, uint32_t root_mask, float *far_)
+    __device__ __forceinline__ void start(uint32_t leaf, float *far_)
     {
-        v = root;
-        mask = root_mask;
+        // leaf = 2^LB: an odd LB has the root record 0 with children 2 and 3
+        const bool odd = (leaf & 0xaaaaaaaau) != 0;
+        v = odd ? 0u : 1u;
+        mask = odd ? 12u : 15u;
         trail = 0;
         far = far_;
     }
@@ -221,14 +223,24 @@ struct BoxWalk {
     }
 };
 
-struct BoxArgs {
-    const float4 *rec = nullptr;
-    const float4 *grp = nullptr;
-    uint32_t leaf = 1;       // 2^LB
-    uint32_t big = 0;
-    uint32_t root = 1, root_mask = 15;
-    float one = 1.f;         // of the packed sums (add2)
+// A box tree in memory.
+struct BoxRef {
+    const float4 *rec, *grp;
+    uint32_t leaf;  // 2^LB
+    uint32_t big;
 };
+
+struct BoxArgs {
+    BoxRef tree = {nullptr, nullptr, 1, 0};
+    const BoxRef *trees = nullptr;  // forests: one a tree (leaf = 0: no points)
+    float one = 1.f;                // of the packed sums (add2)
+};
+
+inline BoxRef box_ref(int64_t n, const float4 *rec, const float4 *grp)
+{
+    const BoxShape sh(n);
+    return {rec, grp, (uint32_t)sh.buckets, (uint32_t)sh.big};
+}
 
 __device__ __forceinline__ void order_keys(unsigned long long &a, unsigned long long &b)
 {
@@ -275,7 +287,7 @@ constexpr int BOX_MERGE_FROM = 4;
 // warp runs the insertion as often as its busiest lane needs it and not once
 // for every place in which any lane has a taker.
 template <int NC, int K, class List>
-__device__ __forceinline__ void box_bucket(const BoxArgs &b, uint32_t i, const float (&q)[NC], f32x2 one, List &list)
+__device__ __forceinline__ void box_bucket(const BoxRef &b, uint32_t i, const float (&q)[NC], f32x2 one, List &list)
 {
     const float4 *g = b.grp + (size_t)(i + min(i, b.big)) * BoxFormat<NC>::GRP;
     const int groups = i < b.big ? 2 : 1;
@@ -317,9 +329,10 @@ __device__ __forceinline__ void box_bucket(const BoxArgs &b, uint32_t i, const f
 }
 
 // The tree's box arrays (t->N and t->D set), and their contents from its
-// level-order nodes.
+// level-order nodes; the same for all trees of a forest.
 cudaError_t box_tree_alloc(kdt_tree *t);
 int build_box_tree(const kdt_tree *t, cudaStream_t s);
+int build_box_forest(kdt_forest *f, cudaStream_t s);
 // Calls that the box tree serves: ordered queries for results, the learned
 // radius among them.  Counts of processed nodes are counts of the state
 // machine; the unordered machine, the ablations and lists spread over groups
@@ -329,6 +342,12 @@ inline bool box_query_serves(const QueryArgs &a, int flags, int mode)
     return (mode == MODE_RESULTS || (mode == MODE_BOUNDED && !a.visits)) && a.out_ids && a.group == 1 &&
            !(flags & (KDT_UNORDERED | KDT_PLAIN_STEP | KDT_CLOSE_FIRST | KDT_STACK));
 }
-int launch_box_query(const kdt_tree *t, const QueryArgs &a, int mode, cudaStream_t s);
+// kNN of one tree, and of a forest's queries (a.T, a.node_off and a.q_off set)
+int launch_box_query(int layout, const BoxRef &tree, const QueryArgs &a, int mode, cudaStream_t s);
+inline int launch_box_query(const kdt_tree *t, const QueryArgs &a, int mode, cudaStream_t s)
+{
+    return launch_box_query(t->layout, box_ref(t->N, t->box_rec, t->box_grp), a, mode, s);
+}
+int launch_box_forest(const kdt_forest *f, const QueryArgs &a, cudaStream_t s);
 
 }  // namespace kdt

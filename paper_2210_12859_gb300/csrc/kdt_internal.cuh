@@ -328,6 +328,9 @@ struct kdt_forest {
     kdt::ForestDesc f;
     float4 *nodes = nullptr;
     int32_t *ids = nullptr;
+    float4 *box_data = nullptr;    // box trees (kdt_box.cuh) of all trees, and where each is
+    void *box_refs = nullptr;      // (BoxRef [T], in box_data's allocation; a host copy in box_host)
+    void *box_host = nullptr;
     float *bbox = nullptr;         // [T][2][3]
     int64_t *h_offsets = nullptr;  // host copy [T+1]
     int *err = nullptr;

@@ -245,19 +245,15 @@ inline int launch_mode(const QueryArgs &a, bool ordered, int mode, int threads, 
             return set_error(KDT_EINVAL, "the learned radius path needs D <= 3");
         }
     default:
+        if (ordered)
+            return set_error(KDT_EINVAL, "ordered result queries are served by the box tree");
         // light runs (tuned for short queries) have their own instantiation
         // so that the default kernel keeps its single-step code
         if constexpr (!STAGE) {
-            if (a.light_run > 1) {
-                if (ordered)
-                    return launch_kernel(knn_kernel<LAYOUT, K, true, MODE_RESULTS, false, INLINE, true>, threads,
-                                         smem, a, s);
+            if (a.light_run > 1)
                 return launch_kernel(knn_kernel<LAYOUT, K, false, MODE_RESULTS, false, INLINE, true>, threads, smem,
                                      a, s);
-            }
         }
-        if (ordered)
-            return launch_kernel(knn_kernel<LAYOUT, K, true, MODE_RESULTS, STAGE, INLINE>, threads, smem, a, s);
         return launch_kernel(knn_kernel<LAYOUT, K, false, MODE_RESULTS, STAGE, INLINE>, threads, smem, a, s);
     }
 }
@@ -271,19 +267,14 @@ inline int launch_k(const QueryArgs &a, bool ordered, int mode, bool batched, cu
     if (batched) {
         if constexpr (LAYOUT == 3)
             return set_error(KDT_EINVAL, "forests store no per-node split dimensions");
+        if (ordered)
+            return set_error(KDT_EINVAL, "ordered forest queries are served by the box trees");
         const bool runs = a.light_run > 1;
-        if (a.inline_depth == 1) {
-            if (runs)
-                return ordered ? launch_kernel(knn_forest_kernel<LAYOUT, K, true, 1, true>, threads, list_bytes, a, s)
-                               : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 1, true>, threads, list_bytes, a, s);
-            return ordered ? launch_kernel(knn_forest_kernel<LAYOUT, K, true, 1>, threads, list_bytes, a, s)
-                           : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 1>, threads, list_bytes, a, s);
-        }
-        if (runs)
-            return ordered ? launch_kernel(knn_forest_kernel<LAYOUT, K, true, 2, true>, threads, list_bytes, a, s)
-                           : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 2, true>, threads, list_bytes, a, s);
-        return ordered ? launch_kernel(knn_forest_kernel<LAYOUT, K, true, 2>, threads, list_bytes, a, s)
-                       : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 2>, threads, list_bytes, a, s);
+        if (a.inline_depth == 1)
+            return runs ? launch_kernel(knn_forest_kernel<LAYOUT, K, false, 1, true>, threads, list_bytes, a, s)
+                        : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 1>, threads, list_bytes, a, s);
+        return runs ? launch_kernel(knn_forest_kernel<LAYOUT, K, false, 2, true>, threads, list_bytes, a, s)
+                    : launch_kernel(knn_forest_kernel<LAYOUT, K, false, 2>, threads, list_bytes, a, s);
     }
     if constexpr (K > MAX_REG_K) {
         // k-best lists spread over groups of lanes: plain results and visit counts

@@ -96,3 +96,23 @@ def test_rebuilt_and_loaded_trees(kdt, tmp_path):
     back = kdt.kdt_tree_load(path)
     both(kdt, back, dq, 8)
     assert same(kdt.kdt_knn(back, dq, 8), kdt.kdt_knn(kdt.kdt_build(b), dq, 8))
+
+
+@pytest.mark.parametrize("D", [1, 3, 4, 6])
+def test_forests(kdt, D):
+    """Trees on both sides of the box build's limits (empty, one bucket, 256
+    buckets, a second launch of the records) in one call, by path order and
+    as given, in one launch and one a tree."""
+    sizes = [0, 1, 7, 8, 40, 0, 2047, 2048, 4100, 16384, 33000, 5, 0]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    qs_n = [3, 5, 100, 0, 33, 7, 200, 1, 300, 1000, 2000, 9, 4]
+    qoff = np.concatenate([[0], np.cumsum(qs_n)]).astype(np.int64)
+    g = np.random.default_rng(D)
+    pts = torch.from_numpy(np.floor(g.random((int(off[-1]), D)) * 64).astype(np.float32) / 64).cuda()
+    dq = torch.from_numpy((g.random((int(qoff[-1]), D)) * 1.2 - 0.1).astype(np.float32)).cuda()
+    forest = kdt.kdt_build_batched(pts, off)
+    for k in (1, 8, 10, 24):
+        for r in (math.inf, 0.1):
+            want = kdt.kdt_knn_batched(forest, dq, qoff, k, r, kdt.KDT_UNORDERED)
+            for flags in (0, kdt.KDT_MORTON, kdt.KDT_PER_TREE):
+                assert same(kdt.kdt_knn_batched(forest, dq, qoff, k, r, flags), want), (k, r, flags)
