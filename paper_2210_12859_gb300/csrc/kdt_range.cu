@@ -4,24 +4,29 @@
 // inside an axis-aligned box.  Sec. 3 notes that other query primitives only
 // change the in-range test and what processNode does, and that a non-ordered
 // traversal is a simplification of the ordered one; both queries use the
-// unordered stack-free machine (left child first, a child is entered iff it
-// can hold a point in range) with a fixed range instead of a shrinking one.
-// The kernel is templated over the processNode action:
-//   ACT_COUNT   count the hits;
-//   ACT_FILL    write the hits to the query's slice [offsets[q], offsets[q+1])
-//               in traversal order (count and fill walk the same nodes in the
-//               same order, so no atomics are needed); hits from the first
-//               16-byte boundary of the slice on are collected four at a time
-//               in registers and written as 16-byte stores, the slice's
-//               unaligned head and its last partial group one word at a time;
-//   ACT_REDUCE  sum a per-point payload over the hits in traversal order (the
-//               point types with payload, e.g. photon power, that Sec. 3 names;
-//               the fixed-radius photon-map density estimate on top).
-// A payload is attached to the tree in node order, so that its loads follow
-// the node loads of the traversal; kNN reductions gather it through the
-// inverse permutation after an ordinary kNN query.
+// unordered machine's order (a node, its left subtree, its right subtree) with a
+// fixed range instead of a shrinking one.  Two kernels:
+//   box_range_kernel   walks the box tree (kdt_box.cuh) and finds the same hits
+//                      in the same order as the machine; templated over the
+//                      processNode action:
+//     ACT_COUNT   count the hits;
+//     ACT_FILL    write the hits to the query's slice [offsets[q], offsets[q+1])
+//                 in traversal order (count and fill walk the same nodes in
+//                 the same order, so no atomics are needed); hits from the
+//                 first 16-byte boundary of the slice on are collected four at
+//                 a time in registers and written as 16-byte stores, the
+//                 slice's unaligned head and its last partial group one word
+//                 at a time;
+//     ACT_REDUCE  sum a per-point payload over the hits in traversal order
+//                 (the point types with payload, e.g. photon power, that Sec. 3
+//                 names; the fixed-radius photon-map density estimate on top);
+//   range_visits_kernel  the machine itself, for the count of the nodes that it
+//                 processes (KDT_RANGE_VISITS).
+// A payload is attached to the tree in node order; kNN reductions gather it
+// through the inverse permutation after an ordinary kNN query.
 #include <string.h>
 
+#include "kdt_box.cuh"
 #include "kdt_learned.cuh"
 #include "kdt_query.cuh"
 
@@ -31,17 +36,6 @@ namespace {
 constexpr int RANGE_THREADS = 128;
 // traversal steps between two claim rounds of a warp (as for kNN, 64 beats 16)
 constexpr int RANGE_CLAIM_STEPS = 64;
-// levels below a bottom node that one traversal step walks with it, per
-// processNode action.  Measured on the clustered 2^24 set (2^22 ball queries):
-// one level takes the count pass from 103 to 74 ms at r = 0.004 (3852 nodes
-// per query) and leaves it unchanged at r = 0.001 (172 nodes); two levels gain
-// more on long queries (59 ms) but cost registers, and so resident warps, on
-// short ones (+9 %).  The fill, whose hit staging already holds more
-// registers, is fastest without inlining at r = 0.001 and within 6 % of the
-// best at r = 0.004.
-constexpr int RANGE_COUNT_LEVELS = 1;
-constexpr int RANGE_FILL_LEVELS = 0;
-constexpr int RANGE_REDUCE_LEVELS = 1;
 enum : int { ACT_COUNT = 0, ACT_FILL = 1, ACT_REDUCE = 2 };
 // binary32 rounding of pi
 constexpr float PI_F = 3.14159265358979323846f;
@@ -63,7 +57,6 @@ struct RangeArgs {
     int C;
     int mode;              // KDT_REDUCE_*
     float *out;            // [Q][C] (ACT_REDUCE)
-    bool count_visits;     // ACT_COUNT: count processed nodes instead of hits
     bool vec_fill;         // ACT_FILL: outputs 16-byte aligned, groups of four hits stored at once
     int *err;
     unsigned long long *counter;
@@ -93,11 +86,9 @@ __device__ __forceinline__ float finish_reduce(float s, int64_t n, int mode, flo
 }
 
 // One lane's range query: the query box / ball and the processNode action's
-// state.  node() is processNode for a node entered from its parent; cull()
-// gives which children can hold a point in range (their existence is the
-// caller's test).  The fill's pending group of up to three hits waits in
-// registers (a staging buffer in shared memory measured slower: the carve-out
-// it takes shrinks the L1 that neighbouring lanes share nodes through).
+// state.  The fill's pending group of up to three hits waits in registers (a
+// staging buffer in shared memory measured slower: the carve-out it takes
+// shrinks the L1 that neighbouring lanes share nodes through).
 // fill: the last `ns` hits (ns < 4) not yet written, newest in the last slot
 template <bool FILL>
 struct FillStage {
@@ -116,15 +107,23 @@ struct RangeLane : FillStage<ACT == ACT_FILL> {
     static constexpr int NC = LayoutTraits<LAYOUT>::NC;
     float lo[NC], hi[KIND == 1 ? NC : 1];
     float acc[ACT == ACT_REDUCE ? KDT_PAYLOAD_MAX_C : 1];
-    int32_t count, visits;  // hits and nodes of one query are below N < 2^30
+    int32_t count;  // hits of one query are below N < 2^30
 
-    __device__ __forceinline__ void start(const RangeArgs &a, int64_t qi)
+    // false: no point is in range of a query that is not a number
+    __device__ __forceinline__ bool start(const RangeArgs &a, int64_t qi)
     {
         load_query<LAYOUT>(a.a, qi, a.D, lo);
-        if constexpr (KIND == 1)
+        bool nan = false;
+#pragma unroll
+        for (int j = 0; j < NC; ++j)
+            nan = nan || lo[j] != lo[j];
+        if constexpr (KIND == 1) {
             load_query<LAYOUT>(a.b, qi, a.D, hi);
+#pragma unroll
+            for (int j = 0; j < NC; ++j)
+                nan = nan || hi[j] != hi[j];
+        }
         count = 0;
-        visits = 0;
         if constexpr (ACT == ACT_FILL) {
             this->base = a.offsets[qi];
             // saturated: a slice longer than any hit count, or negative, still
@@ -138,36 +137,36 @@ struct RangeLane : FillStage<ACT == ACT_FILL> {
             for (int c = 0; c < KDT_PAYLOAD_MAX_C; ++c)
                 acc[c] = 0.f;
         }
+        return !nan;
     }
 
-    __device__ __forceinline__ void node(const RangeArgs &a, const NodeVal<LAYOUT> &nd, int n)
+    __device__ __forceinline__ bool test(const RangeArgs &a, const NodeVal<LAYOUT> &nd, float &d2) const
     {
-        if constexpr (ACT == ACT_COUNT)
-            ++visits;
-        bool hit;
-        float d2 = 0.f;
         if constexpr (KIND == 0) {
             d2 = dist2<NC>(nd.c, lo);
-            hit = d2 <= a.r2;
+            return d2 <= a.r2;
         } else {
-            hit = true;
+            bool hit = true;
 #pragma unroll
             for (int j = 0; j < NC; ++j)
                 hit = hit && lo[j] <= nd.c[j] && nd.c[j] <= hi[j];
+            return hit;
         }
-        if (!hit)
-            return;
+    }
+
+    // processNode of a hit: node n, the point id
+    __device__ __forceinline__ void hit(const RangeArgs &a, int n, uint32_t id, float d2)
+    {
         if constexpr (ACT == ACT_FILL) {
             if (count < this->limit) {
-                const int32_t id = (int32_t)node_id<LAYOUT>(nd, a.ids, n);
                 const int64_t pos = this->base + count;
                 if (!a.vec_fill || (this->ns == 0 && (pos & 3) != 0)) {
                     // before the slice's first 16-byte boundary (or unaligned outputs)
-                    a.out_ids[pos] = id;
+                    a.out_ids[pos] = (int32_t)id;
                     if (KIND == 0 && a.out_d2)
                         a.out_d2[pos] = d2;
                 } else {
-                    this->sid0 = this->sid1; this->sid1 = this->sid2; this->sid2 = this->sid3; this->sid3 = id;
+                    this->sid0 = this->sid1; this->sid1 = this->sid2; this->sid2 = this->sid3; this->sid3 = (int32_t)id;
                     this->sd20 = this->sd21; this->sd21 = this->sd22; this->sd22 = this->sd23; this->sd23 = d2;
                     if (++this->ns == 4) {  // positions pos - 3 .. pos, pos - 3 on a 16-byte boundary
                         *reinterpret_cast<int4 *>(a.out_ids + pos - 3) =
@@ -190,20 +189,52 @@ struct RangeLane : FillStage<ACT == ACT_FILL> {
         ++count;
     }
 
-    __device__ __forceinline__ void cull(const RangeArgs &a, const NodeVal<LAYOUT> &nd, int sdim, bool &left_ok,
-                                         bool &right_ok) const
+    // boxes of a record that can hold a point in range, a bit each
+    __device__ __forceinline__ uint32_t boxes(const RangeArgs &a, const float4 *__restrict__ rec, f32x2 one) const
     {
-        const float split = select_dim<NC>(nd.c, sdim);
+        uint32_t in = 0;
         if constexpr (KIND == 0) {
-            const float sd = __fsub_rn(select_dim<NC>(lo, sdim), split);
-            const float sd2 = __fmul_rn(sd, sd);
-            left_ok = sd <= 0.f || sd2 <= a.r2;
-            right_ok = sd > 0.f || sd2 <= a.r2;
+            float d[4];
+            box_dist4<NC>(rec, lo, one, d);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                in |= d[c] <= a.r2 ? 1u << c : 0u;
         } else {
-            // left subtree coordinates are <= split, right ones >= split
-            left_ok = select_dim<NC>(lo, sdim) <= split;
-            right_ok = select_dim<NC>(hi, sdim) >= split;
+            in = 15u;
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const float4 l = __ldg(rec + 2 * j), h = __ldg(rec + 2 * j + 1);
+                in &= (l.x <= hi[j] && lo[j] <= h.x ? 1u : 0u) | (l.y <= hi[j] && lo[j] <= h.y ? 2u : 0u) |
+                      (l.z <= hi[j] && lo[j] <= h.z ? 4u : 0u) | (l.w <= hi[j] && lo[j] <= h.w ? 8u : 0u);
+            }
         }
+        return in;
+    }
+
+    // points of a group in range, a bit each
+    __device__ __forceinline__ uint32_t points(const RangeArgs &a, const float4 *__restrict__ g, f32x2 one,
+                                               float (&d)[8]) const
+    {
+        uint32_t in = 0;
+        if constexpr (KIND == 0) {
+            group_dist8<NC>(g, lo, one, d);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                in |= d[c] <= a.r2 ? 1u << c : 0u;
+        } else {
+            in = 255u;
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const float4 u = __ldg(g + 2 * j), v = __ldg(g + 2 * j + 1);
+                const float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+                uint32_t m = 0;
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    m |= lo[j] <= x[c] && x[c] <= hi[j] ? 1u << c : 0u;
+                in &= m;
+            }
+        }
+        return in;
     }
 
     // the query's end: the last partial group of the fill, the count or the
@@ -233,7 +264,7 @@ struct RangeLane : FillStage<ACT == ACT_FILL> {
                 atomicOr(a.err, ERR_RANGE);
         } else {
             if (a.counts)
-                a.counts[qi] = ACT == ACT_COUNT && a.count_visits ? visits : count;
+                a.counts[qi] = count;
             if constexpr (ACT == ACT_REDUCE) {
 #pragma unroll
                 for (int c = 0; c < KDT_PAYLOAD_MAX_C; ++c)
@@ -244,42 +275,221 @@ struct RangeLane : FillStage<ACT == ACT_FILL> {
     }
 };
 
+// One lane's place in the box tree for a fixed range, in the machine's order:
+// node, left subtree, right subtree.  A record's node is binary node v, its
+// boxes are v's grandchildren, and v's point and its children's points come
+// from the level-order nodes.  What is left to do below v are five bits in
+// order: the left child's two subtrees, the right child's point, its two
+// subtrees (v's and the left child's points are dealt with on entry).  The
+// range is fixed, so the bits set on entry stay true and no record is read
+// twice.  The records above keep theirs in `trail`, five bits each, the root's
+// in root_bits: 12 records below the root for N < 2^30.
+struct RangeWalk {
+    uint32_t v, bits, root_bits;
+    unsigned long long trail;
+    __device__ __forceinline__ void start(uint32_t root)
+    {
+        v = root;
+        bits = 0;
+        root_bits = 0;
+        trail = 0;
+    }
+    __device__ __forceinline__ void descend(uint32_t root, uint32_t c)
+    {
+        if (v == root)
+            root_bits = bits;
+        else
+            trail = trail << 5 | bits;
+        v = 4 * v + c;
+        bits = 0;
+    }
+    // to the nearest record with something left; false: none
+    __device__ __forceinline__ bool pop(uint32_t root)
+    {
+        if (trail) {
+            const int up = (__ffsll((long long)trail) - 1) / 5;
+            v >>= 2 * (up + 1);
+            trail >>= 5 * up;
+            bits = (uint32_t)trail & 31u;
+            trail >>= 5;
+            return true;
+        }
+        v = root;
+        bits = root_bits;
+        root_bits = 0;
+        return bits != 0;
+    }
+};
+
 // KIND 0: ball of squared radius r2 around a[q]; KIND 1: box [a[q], b[q]].
-// Persistent blocks; every lane claims its next query when its current one
-// ends (checked every RANGE_CLAIM_STEPS steps), as in the kNN kernel; the step
-// bound 3N + 3 is checked once per round.  A node entered from its parent
-// whose subtree spans at most L + 1 levels (L the action's level constant; index >=
-// floor(N / 2^(L+1)) for L levels below it: its leftmost descendant L + 1
-// levels down, 2^(L+1) (i + 1) - 1, does not exist) is walked whole in one
-// step: its descendants are loaded together, then entered in the machine's
-// order (node, left subtree, right subtree) under the same cull tests, and
-// the step returns to the parent as the machine would after the node's right
-// subtree.  Hits, their order and the processed nodes are those of the
-// one-node-per-step machine.
+// Persistent lanes, and the warp's turns between records and buckets, as in
+// box_knn_kernel.  The bucket's point from above is some other node's: it is
+// met there.
+//
+// Bound: records of incoherent lanes (dependent loads) and, in the fill, the
+// hits' stores with few lanes active.  Against the state machine's kernels
+// (one plane a test; its bottom nodes walked with their leaves): see
+// RANGE_RECORD_LANES.
+constexpr int RANGE_RECORD_LANES = 4, RANGE_FREE_LANES = 16;
+
 template <int LAYOUT, int KIND, int ACT>
-__global__ void __launch_bounds__(RANGE_THREADS) range_kernel(const RangeArgs a)
+__global__ void __launch_bounds__(RANGE_THREADS) box_range_kernel(const RangeArgs a, const BoxArgs b)
 {
-    // levels below a node walked within its step (two float4 per node in layout 2: no inlining there)
-    constexpr int LEVELS =
-        ACT == ACT_COUNT ? RANGE_COUNT_LEVELS : (ACT == ACT_FILL ? RANGE_FILL_LEVELS : RANGE_REDUCE_LEVELS);
-    constexpr int INL = LAYOUT != 2 ? LEVELS : 0;
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    const BoxRef tree = b.tree;
+    const f32x2 one = pair(b.one, b.one);
+    const bool odd = (tree.leaf & 0xaaaaaaaau) != 0;
+    const uint32_t root = odd ? 0u : 1u;
     RangeLane<LAYOUT, KIND, ACT> L;
+    RangeWalk w;
+    w.start(root);
+    int64_t qi = -1;
+    bool busy = false, first = true, exhausted = false;
+    const int64_t lanes = (int64_t)gridDim.x * blockDim.x;
+    // a node's point: hit or not
+    auto at_node = [&](uint32_t u) {
+        const NodeVal<LAYOUT> nd = fetch<LAYOUT, false>(a.nodes, nullptr, 0, (int)u - 1);
+        float d2 = 0.f;
+        if (L.test(a, nd, d2))
+            L.hit(a, (int)u - 1, node_id<LAYOUT>(nd, a.ids, (int)u - 1), d2);
+    };
+    // the next thing to do at v or above: leaves v at a node to enter
+    auto advance = [&]() {
+        for (;;) {
+            if (w.bits == 0 && !w.pop(root))
+                return false;
+            const uint32_t c = __ffs(w.bits) - 1;
+            w.bits &= w.bits - 1;
+            if (c == 2) {
+                at_node(2 * w.v + 1);
+            } else {
+                w.descend(root, c < 2 ? c : c - 1);
+                return true;
+            }
+        }
+    };
+    for (;;) {
+        const unsigned free_lanes = __ballot_sync(0xffffffffu, !busy && !exhausted);
+        const unsigned busy_lanes = __ballot_sync(0xffffffffu, busy);
+        if (!busy_lanes || __popc(free_lanes) >= RANGE_FREE_LANES) {
+            if (!busy && qi >= 0) {
+                L.finish(a, qi);
+                qi = -1;
+            }
+            const bool need = !busy && !exhausted;
+            int64_t slot;
+            if (first)
+                slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+            else if (lanes >= a.Q)
+                slot = a.Q;
+            else
+                slot = claim_slot(need, a.counter);
+            if (need) {
+                if (!first && slot < a.Q)
+                    slot += lanes;
+                if (slot < a.Q) {
+                    qi = a.perm ? (int64_t)a.perm[slot] : slot;
+                    busy = L.start(a, qi);
+                    w.start(root);
+                    // with an odd LB the root's point is no record's node
+                    if (busy && odd)
+                        at_node(1);
+                } else {
+                    exhausted = true;
+                }
+            }
+            first = false;
+            if (__all_sync(0xffffffffu, !busy && exhausted && qi < 0))
+                break;
+        }
+        for (;;) {
+            if (busy && w.v < tree.leaf) {
+                uint32_t in = L.boxes(a, tree.rec + (size_t)w.v * BoxFormat<NC>::REC, one);
+                uint32_t right = 0;
+                if (w.v == 0) {
+                    in &= 12u;
+                } else {
+                    at_node(w.v);
+                    const NodeVal<LAYOUT> l = fetch<LAYOUT, false>(a.nodes, nullptr, 0, 2 * (int)w.v - 1);
+                    const NodeVal<LAYOUT> r = fetch<LAYOUT, false>(a.nodes, nullptr, 0, 2 * (int)w.v);
+                    float d2 = 0.f, dr = 0.f;
+                    if (L.test(a, l, d2))
+                        L.hit(a, 2 * (int)w.v - 1, node_id<LAYOUT>(l, a.ids, 2 * (int)w.v - 1), d2);
+                    right = L.test(a, r, dr);
+                }
+                w.bits = (in & 3u) | right << 2 | (in & 12u) << 1;
+                busy = advance();
+            }
+            if (__popc(__ballot_sync(0xffffffffu, busy && w.v < tree.leaf)) <= RANGE_RECORD_LANES)
+                break;
+        }
+        if (busy && w.v >= tree.leaf) {
+            const uint32_t i = w.v - tree.leaf;
+            const float4 *g = tree.grp + (size_t)(i + min(i, tree.big)) * BoxFormat<NC>::GRP;
+            const bool two = i < tree.big;
+            float d[2][8];
+            uint32_t in0 = L.points(a, g, one, d[0]) & 127u, in1 = 0;
+            if (two)
+                in1 = L.points(a, g + BoxFormat<NC>::GRP, one, d[1]);
+            if constexpr (ACT == ACT_COUNT) {
+                L.count += __popc(in0) + __popc(in1);
+            } else {
+                // place p of the two groups is the bucket's node h = p + 1
+                // (first group) or p, counted from its root 1; hits in the
+                // order node, left, right: rank of h = 1 .. 15 there, and back
+                constexpr int RANK[16] = {0, 0, 1, 8, 2, 5, 9, 12, 3, 4, 6, 7, 10, 11, 13, 14};
+                constexpr unsigned long long NODE_AT = 0xFE7DC63BA598421ull;  // h of rank 0, 1, ... from the low nibble
+                uint32_t order = 0;
+#pragma unroll
+                for (int h = 1; h < 16; ++h)
+                    order |= (h < 8 ? in0 >> (h - 1) & 1u : in1 >> (h - 8) & 1u) << RANK[h];
+                while (order) {
+                    const int rank = __ffs(order) - 1;
+                    order &= order - 1;
+                    const int h = (int)(NODE_AT >> (4 * rank)) & 15;
+                    const int up = 31 - __clz(h);
+                    const int p = h < 8 ? h - 1 : h - 8;
+                    const float4 *gp = h < 8 ? g : g + BoxFormat<NC>::GRP;
+                    const uint32_t id = __ldg(reinterpret_cast<const uint32_t *>(gp + 2 * NC) + p);
+                    float d2 = 0.f;
+                    if constexpr (KIND == 0 && ACT == ACT_FILL) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            d2 = p == j ? (h < 8 ? d[0][j] : d[1][j]) : d2;
+                    }
+                    L.hit(a, (int)((w.v << up) + (uint32_t)(h - (1 << up))) - 1, id, d2);
+                }
+            }
+            busy = advance();
+        }
+    }
+}
+
+// The unordered machine of Sec. 3.2 with a fixed range: processed nodes of
+// every query.  The step bound 3N + 3 is checked once a round.
+template <int LAYOUT, int KIND>
+__global__ void __launch_bounds__(RANGE_THREADS) range_visits_kernel(const RangeArgs a)
+{
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    float lo[NC], hi[NC];
     int64_t qi = -1;
     bool exhausted = false;
-    int curr = 0, prev = -1, dim = 0;
+    int curr = 0, prev = -1, dim = 0, visits = 0;
     uint32_t steps = 0;
     const uint32_t cap = 3u * (uint32_t)a.N + 3u;
-    const int last = a.N - 1, bottom = a.N >> (INL + 1);
     for (;;) {
         const bool need = qi < 0 && !exhausted;
         const int64_t slot = claim_slot(need, a.counter);
         if (need) {
             if (slot < a.Q) {
                 qi = a.perm ? (int64_t)a.perm[slot] : slot;
-                L.start(a, qi);
+                load_query<LAYOUT>(a.a, qi, a.D, lo);
+                if (KIND == 1)
+                    load_query<LAYOUT>(a.b, qi, a.D, hi);
                 curr = 0;
                 prev = -1;
                 dim = 0;
+                visits = 0;
                 steps = 0;
             } else {
                 exhausted = true;
@@ -300,60 +510,29 @@ __global__ void __launch_bounds__(RANGE_THREADS) range_kernel(const RangeArgs a)
             const bool from_parent = prev < curr;
             const int lc = 2 * curr + 1, rc = lc + 1;
             const int parent = (curr - 1) >> 1;
-            int next;
-            if (INL > 0 && from_parent && curr >= bottom) {
-                // children lc, rc (one 32-byte sector); with two levels also
-                // the grandchildren 2 lc + 1 .. 2 rc + 2 (indices clamped to
-                // the last node for the loads, tested before use)
-                const int c1 = min(lc, last), c2 = min(rc, last);
-                const NodeVal<LAYOUT> n1 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, c1);
-                const NodeVal<LAYOUT> n2 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, c2);
-                NodeVal<LAYOUT> m1, m2, m3, m4;
-                if constexpr (INL >= 2) {
-                    m1 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, min(2 * c1 + 1, last));
-                    m2 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, min(2 * c1 + 2, last));
-                    m3 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, min(2 * c2 + 1, last));
-                    m4 = fetch<LAYOUT, false>(a.nodes, nullptr, 0, min(2 * c2 + 2, last));
-                }
-                const int dim1 = dim + 1 == a.D ? 0 : dim + 1;
-                bool l, r, l1, r1;
-                L.node(a, nd, curr);
-                L.cull(a, nd, split_dim_of<LAYOUT>(nd, dim), l, r);
-                if (l && lc < a.N) {
-                    L.node(a, n1, lc);
-                    if constexpr (INL >= 2) {
-                        L.cull(a, n1, split_dim_of<LAYOUT>(n1, dim1), l1, r1);
-                        if (l1 && 2 * lc + 1 < a.N)
-                            L.node(a, m1, 2 * lc + 1);
-                        if (r1 && 2 * lc + 2 < a.N)
-                            L.node(a, m2, 2 * lc + 2);
-                    }
-                }
-                if (r && rc < a.N) {
-                    L.node(a, n2, rc);
-                    if constexpr (INL >= 2) {
-                        L.cull(a, n2, split_dim_of<LAYOUT>(n2, dim1), l1, r1);
-                        if (l1 && 2 * rc + 1 < a.N)
-                            L.node(a, m3, 2 * rc + 1);
-                        if (r1 && 2 * rc + 2 < a.N)
-                            L.node(a, m4, 2 * rc + 2);
-                    }
-                }
-                next = parent;
+            visits += from_parent;
+            const int sdim = split_dim_of<LAYOUT>(nd, dim);
+            const float split_at = select_dim<NC>(nd.c, sdim);
+            bool left_ok, right_ok;
+            if constexpr (KIND == 0) {
+                const float sd = __fsub_rn(select_dim<NC>(lo, sdim), split_at);
+                const float sd2 = __fmul_rn(sd, sd);
+                left_ok = sd <= 0.f || sd2 <= a.r2;
+                right_ok = sd > 0.f || sd2 <= a.r2;
             } else {
-                if (from_parent)
-                    L.node(a, nd, curr);
-                bool left_ok, right_ok;
-                L.cull(a, nd, split_dim_of<LAYOUT>(nd, dim), left_ok, right_ok);
-                left_ok = left_ok && lc < a.N;
-                right_ok = right_ok && rc < a.N;
-                if (from_parent)
-                    next = left_ok ? lc : (right_ok ? rc : parent);
-                else if (prev == lc)
-                    next = right_ok ? rc : parent;
-                else
-                    next = parent;
+                // left subtree coordinates are <= split, right ones >= split
+                left_ok = select_dim<NC>(lo, sdim) <= split_at;
+                right_ok = select_dim<NC>(hi, sdim) >= split_at;
             }
+            left_ok = left_ok && lc < a.N;
+            right_ok = right_ok && rc < a.N;
+            int next;
+            if (from_parent)
+                next = left_ok ? lc : (right_ok ? rc : parent);
+            else if (prev == lc)
+                next = right_ok ? rc : parent;
+            else
+                next = parent;
             if (next < 0) {
                 done = true;
                 break;
@@ -367,33 +546,52 @@ __global__ void __launch_bounds__(RANGE_THREADS) range_kernel(const RangeArgs a)
         }
         if (!done)
             continue;
-        L.finish(a, qi);
+        a.counts[qi] = visits;
         qi = -1;
     }
 }
 
 template <int LAYOUT, int KIND, int ACT>
-int launch_one(const RangeArgs &a, cudaStream_t s)
+int launch_one(const RangeArgs &a, const BoxArgs &b, cudaStream_t s)
 {
-    const int grid = grid_for_kernel((const void *)range_kernel<LAYOUT, KIND, ACT>, RANGE_THREADS, 0);
-    KDT_LAUNCH range_kernel<LAYOUT, KIND, ACT><<<grid, RANGE_THREADS, 0, s>>>(a);
+    const void *fn = (const void *)box_range_kernel<LAYOUT, KIND, ACT>;
+    // few queries: small blocks, so that they spread over the SMs
+    int threads = RANGE_THREADS;
+    while (threads > 32 && a.Q < (int64_t)num_sms() * threads)
+        threads >>= 1;
+    const int64_t grid = std::min<int64_t>(grid_for_kernel(fn, threads, 0), (a.Q + threads - 1) / threads);
+    if (grid * threads < a.Q)
+        KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
+    KDT_LAUNCH box_range_kernel<LAYOUT, KIND, ACT><<<(unsigned)grid, threads, 0, s>>>(a, b);
+    KDT_CUDA(cudaGetLastError());
+    return KDT_OK;
+}
+
+template <int LAYOUT, int KIND>
+int launch_visits(const RangeArgs &a, cudaStream_t s)
+{
+    KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
+    const int grid = grid_for_kernel((const void *)range_visits_kernel<LAYOUT, KIND>, RANGE_THREADS, 0);
+    KDT_LAUNCH range_visits_kernel<LAYOUT, KIND><<<grid, RANGE_THREADS, 0, s>>>(a);
     KDT_CUDA(cudaGetLastError());
     return KDT_OK;
 }
 
 template <int LAYOUT>
-int launch_range_layout(int kind, int act, const RangeArgs &a, cudaStream_t s)
+int launch_range_layout(int kind, int act, bool visits, const RangeArgs &a, const BoxArgs &b, cudaStream_t s)
 {
+    if (visits)
+        return kind == 0 ? launch_visits<LAYOUT, 0>(a, s) : launch_visits<LAYOUT, 1>(a, s);
     if (kind == 0) {
         if (act == ACT_COUNT)
-            return launch_one<LAYOUT, 0, ACT_COUNT>(a, s);
+            return launch_one<LAYOUT, 0, ACT_COUNT>(a, b, s);
         if (act == ACT_FILL)
-            return launch_one<LAYOUT, 0, ACT_FILL>(a, s);
-        return launch_one<LAYOUT, 0, ACT_REDUCE>(a, s);
+            return launch_one<LAYOUT, 0, ACT_FILL>(a, b, s);
+        return launch_one<LAYOUT, 0, ACT_REDUCE>(a, b, s);
     }
     if (act == ACT_COUNT)
-        return launch_one<LAYOUT, 1, ACT_COUNT>(a, s);
-    return launch_one<LAYOUT, 1, ACT_FILL>(a, s);
+        return launch_one<LAYOUT, 1, ACT_COUNT>(a, b, s);
+    return launch_one<LAYOUT, 1, ACT_FILL>(a, b, s);
 }
 
 int run_range(const kdt_tree *t, int kind, int act, int flags, RangeArgs a, cudaStream_t s)
@@ -412,12 +610,14 @@ int run_range(const kdt_tree *t, int kind, int act, int flags, RangeArgs a, cuda
     a.perm = nullptr;
     if (morton)
         KDT_TRY(query_order(t, a.a, a.Q, false, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
-    KDT_CUDA(cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s));
+    BoxArgs b;
+    b.tree = box_ref(t->N, t->box_rec, t->box_grp);
+    const bool visits = flags & KDT_RANGE_VISITS;
     switch (t->layout) {
-    case 0: return launch_range_layout<0>(kind, act, a, s);
-    case 1: return launch_range_layout<1>(kind, act, a, s);
-    case 3: return launch_range_layout<3>(kind, act, a, s);
-    default: return launch_range_layout<2>(kind, act, a, s);
+    case 0: return launch_range_layout<0>(kind, act, visits, a, b, s);
+    case 1: return launch_range_layout<1>(kind, act, visits, a, b, s);
+    case 3: return launch_range_layout<3>(kind, act, visits, a, b, s);
+    default: return launch_range_layout<2>(kind, act, visits, a, b, s);
     }
 }
 
@@ -532,7 +732,6 @@ int kdt_radius_count(const kdt_tree *t, const float *d_q, int64_t Q, float radiu
     a.Q = Q;
     a.r2 = radius * radius;
     a.counts = d_counts;
-    a.count_visits = flags & KDT_RANGE_VISITS;
     return run_range(t, 0, ACT_COUNT, flags, a, (cudaStream_t)stream);
 }
 
@@ -571,7 +770,6 @@ int kdt_box_count(const kdt_tree *t, const float *d_lo, const float *d_hi, int64
     a.b = d_hi;
     a.Q = Q;
     a.counts = d_counts;
-    a.count_visits = flags & KDT_RANGE_VISITS;
     return run_range(t, 1, ACT_COUNT, flags, a, (cudaStream_t)stream);
 }
 
