@@ -260,9 +260,19 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(BoxBuild a
 constexpr int BOX_RECORD_LANES = 4;
 constexpr int BOX_FREE_LANES = 24;
 
+// Resident blocks to build for.  Closest points in 4-D, bound by L1 wavefronts
+// whose latency more warps cover: 10 (10^7 of them 5.58 -> 5.33 ms against 8; in
+// 3-D 10 costs a scan of 5003 24.5 -> 27 us).  3-D: 7 to k = 8 (forest 2.32 -> 2.28
+// ms against 6), 6 at k = 16 (surface 2.85 -> 2.77 ms against 5).  Elsewhere the
+// registers that more blocks leave are too few (spills).
+constexpr int box_blocks_per_sm(int layout, int k)
+{
+    return k <= 1 ? (layout == 1 ? 10 : (layout == 0 ? 8 : 6)) : (k <= 8 ? (layout == 0 ? 7 : 6) : (k <= 16 && layout == 0 ? 6 : 1));
+}
+
 // FOREST: a lane's query finds its tree by its place in the query offsets.
 template <int LAYOUT, int K, int MODE, bool FOREST>
-__global__ void __launch_bounds__(BOX_THREADS, K <= 8 ? 6 : 1) box_knn_kernel(const QueryArgs a, const BoxArgs b)
+__global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box_knn_kernel(const QueryArgs a, const BoxArgs b)
 {
     constexpr int NC = LayoutTraits<LAYOUT>::NC;
     using List = typename std::conditional<(K <= MAX_REG_K), RegList<K <= MAX_REG_K ? K : 1>, SmemList>::type;

@@ -105,6 +105,21 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
     return r;
 }
 
+// 32 bytes in one load (records and groups are multiples of 32 bytes on
+// 32-byte boundaries): half the L1 wavefronts of two 16-byte loads, which bound
+// the walks of incoherent lanes.
+struct Float8 {
+    float v[8];
+};
+__device__ __forceinline__ Float8 load8(const void *p)
+{
+    Float8 r;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]), "=f"(r.v[7])
+        : "l"(p));
+    return r;
+}
+
 // t_j squared and summed in the order of dist2
 template <int NC>
 __device__ __forceinline__ void box_dist4(const float4 *__restrict__ rec, const float (&q)[NC], f32x2 one, float (&d)[4])
@@ -112,13 +127,14 @@ __device__ __forceinline__ void box_dist4(const float4 *__restrict__ rec, const 
     f32x2 s[2];
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-        const float4 lo = __ldg(rec + 2 * j), hi = __ldg(rec + 2 * j + 1);
-        const f32x2 l[2] = {pair(lo.x, lo.y), pair(lo.z, lo.w)}, h[2] = {pair(hi.x, hi.y), pair(hi.z, hi.w)};
+        const Float8 b = load8(rec + 2 * j);  // lo[4], hi[4]
+        const f32x2 l[2] = {pair(b.v[0], b.v[1]), pair(b.v[2], b.v[3])};
+        const f32x2 h[2] = {pair(b.v[4], b.v[5]), pair(b.v[6], b.v[7])};
         const f32x2 qq = pair(q[j], q[j]);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            const float2 a = split(sub2(l[c], qq)), b = split(sub2(qq, h[c]));
-            const f32x2 t = pair(fmaxf(fmaxf(a.x, b.x), 0.f), fmaxf(fmaxf(a.y, b.y), 0.f));
+            const float2 u = split(sub2(l[c], qq)), w = split(sub2(qq, h[c]));
+            const f32x2 t = pair(fmaxf(fmaxf(u.x, w.x), 0.f), fmaxf(fmaxf(u.y, w.y), 0.f));
             const f32x2 tt = mul2(t, t);
             s[c] = j == 0 ? tt : add2(s[c], tt, one);
         }
@@ -136,8 +152,8 @@ __device__ __forceinline__ void group_dist8(const float4 *__restrict__ g, const 
     f32x2 s[4];
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-        const float4 a = __ldg(g + 2 * j), b = __ldg(g + 2 * j + 1);
-        const f32x2 x[4] = {pair(a.x, a.y), pair(a.z, a.w), pair(b.x, b.y), pair(b.z, b.w)};
+        const Float8 b = load8(g + 2 * j);
+        const f32x2 x[4] = {pair(b.v[0], b.v[1]), pair(b.v[2], b.v[3]), pair(b.v[4], b.v[5]), pair(b.v[6], b.v[7])};
         const f32x2 qq = pair(q[j], q[j]);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -303,12 +319,11 @@ __device__ __forceinline__ void box_bucket(const BoxRef &b, uint32_t i, const fl
         if constexpr (K == 8 || K == 16) {
             const int most = __reduce_max_sync(__activemask(), __popc(take));
             if (most >= BOX_MERGE_FROM) {
-                const uint4 u = __ldg(reinterpret_cast<const uint4 *>(ids)), v = __ldg(reinterpret_cast<const uint4 *>(ids) + 1);
-                const uint32_t id[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+                const Float8 id = load8(ids);
                 unsigned long long key[8];
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
-                    key[c] = take >> c & 1u ? pack_key(d[c], id[c]) : ~0ull;
+                    key[c] = take >> c & 1u ? pack_key(d[c], __float_as_uint(id.v[c])) : ~0ull;
                 merge8<K>(list.L, key);
                 continue;
             }
