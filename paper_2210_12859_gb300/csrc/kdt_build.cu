@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(BT) part_scatter_kernel(const uint32_t *__rest
     }
 }
 
-// ---- single trees: one pass a list and level
+// ---- single trees: two kernels a level
 
 // The in-order layout of a complete tree of n < 2^30 points in 32 bits.
 struct Layout32 {
@@ -487,17 +487,21 @@ __device__ __forceinline__ int part_dest(const Layout32 &t, int l, int u, int lu
 
 constexpr int TOP_ITEMS = 8;
 constexpr int TOP_TILE = BT * TOP_ITEMS;
-constexpr int TOP_LISTS = 3;  // lists of one launch
-constexpr unsigned long long TOP_OWN = 1ull << 62, TOP_ALL = 2ull << 62, TOP_VALUE = (1ull << 62) - 1;
-constexpr int TOP_POLLS = 1 << 16;
+constexpr int TOP_WORDS = TOP_TILE / 32;  // vote words of a tile
+constexpr int TOP_LISTS = 3;              // lists of one launch
+constexpr int TOP_GROUP = 64;             // tiles whose counts are also summed
+static_assert(TOP_WORDS <= 64 && TOP_WORDS % 32 == 0, "the words of a tile are scanned by two warps");
+
+inline int64_t top_tiles_of(int64_t n) { return (n + TOP_TILE - 1) / TOP_TILE; }
+inline int64_t top_groups_of(int64_t n) { return (top_tiles_of(n) + TOP_GROUP - 1) / TOP_GROUP; }
 
 struct PartArgs {
     const uint32_t *in[TOP_LISTS];
     uint32_t *out[TOP_LISTS];
     const uint8_t *side;
-    unsigned long long *state;  // [list][tiles]
-    uint32_t *ticket;           // [list]
-    int n, l, tiles;
+    uint2 *votes;               // [list][tiles][TOP_WORDS]: lefts and nodes of 32 places
+    unsigned long long *count;  // [list][tiles + groups]: nodes << 32 | lefts; the groups start at zero
+    int n, l, tiles, groups;
     // the list that splits the next level also records that level's sides and
     // emits its nodes (-1: none does)
     int next;
@@ -508,117 +512,136 @@ struct PartArgs {
     int32_t *ids;
 };
 
-// Stable partition of up to three lists by the level's sides in one pass each.
+// Stable partition of up to three lists by the level's sides, in two kernels.
 // A plain count of the left elements suffices, no segmented one: how many the
-// earlier subtrees of the level hold is a closed form of the layout.  The count
-// of the tiles before comes from a bounded look-back as in the radix sort (a
-// silent predecessor is counted from its elements).
+// earlier subtrees of the level hold is a closed form of the layout.
 //
-// Bound: the random bytes, a gather an element and list and a store an element
-// for the next level's sides (L1-to-L2 requests 56 % busy), and the wait for the
-// look-back.  It replaced a count, a single-block scan and a scatter with 64-bit
-// segmented scans a list, and a pass that assigned the next level's sides: a
-// level of 2^24 points takes 0.42 ms instead of 0.71.  Tiles of 4 / 8 / 16 elements
-// a thread: the build of 2^24 points 11.4 / 11.0 / 12.9 ms.
-__global__ void __launch_bounds__(BT, 4) part_kernel(const PartArgs a)
+// part_votes_kernel gathers the sides once and keeps them as vote words, with
+// the counts of tiles and of groups of tiles; part_move_kernel sums the counts
+// before its tile (a group's and a tile's count a thread) and moves the elements.
+//
+// Bound: the random bytes, a gather an element and list in the first and a
+// store an element for the next level's sides in the second, beside 12 bytes
+// an element of list traffic.  One kernel with a look-back took 0.42 ms a level
+// of 2^24 points (its blocks waited for the look-back with the gathers of two
+// blocks an SM in flight; windows of 32 and of 256 tiles alike), the
+// count, scan, scatter and assign kernels before it 0.71.
+__global__ void __launch_bounds__(BT) part_votes_kernel(const PartArgs a)
 {
-    __shared__ uint32_t s_cnt[BT / 32];
-    __shared__ unsigned long long s_before;
-    __shared__ uint32_t s_tile;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, y = blockIdx.y;
+    __shared__ uint32_t s_cnt;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, y = blockIdx.y, tile = blockIdx.x;
     if (tid == 0)
-        s_tile = atomicAdd(a.ticket + y, 1u);
+        s_cnt = 0;
     __syncthreads();
-    const int tile = (int)s_tile;
+    const uint32_t *in = y == 0 ? a.in[0] : (y == 1 ? a.in[1] : a.in[2]);
+    const Layout32 t(a.n);
+    const int first = tile * TOP_TILE + w * 32 * TOP_ITEMS + lane;
+    uint32_t pid[TOP_ITEMS], side[TOP_ITEMS];
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j) {
+        const int p = first + 32 * j;
+        pid[j] = p < a.n && Layout32::level(t.node_at(p)) >= a.l ? in[p] : 0xffffffffu;
+    }
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j)
+        side[j] = pid[j] != 0xffffffffu ? a.side[pid[j]] : 3u;  // 3: not in a subtree of the level
+    uint32_t run = 0;
+    uint2 words = make_uint2(0, 0);
+#pragma unroll
+    for (int j = 0; j < TOP_ITEMS; ++j) {
+        const uint32_t bl = __ballot_sync(0xffffffffu, side[j] == SIDE_LEFT);
+        const uint32_t bn = __ballot_sync(0xffffffffu, side[j] == SIDE_NODE);
+        if (lane == j)
+            words = make_uint2(bl, bn);
+        run += __popc(bl) | __popc(bn) << 16;
+    }
+    if (lane < TOP_ITEMS)
+        a.votes[((size_t)y * a.tiles + tile) * TOP_WORDS + w * TOP_ITEMS + lane] = words;
+    if (lane == 0)
+        atomicAdd(&s_cnt, run);  // at most TOP_TILE of each
+    __syncthreads();
+    if (tid == 0) {
+        const unsigned long long c = (unsigned long long)(s_cnt >> 16) << 32 | (s_cnt & 0xffffu);
+        unsigned long long *count = a.count + (size_t)y * (a.tiles + a.groups);
+        count[tile] = c;
+        atomicAdd(count + a.tiles + tile / TOP_GROUP, c);
+    }
+}
+
+__global__ void __launch_bounds__(BT) part_move_kernel(const PartArgs a)
+{
+    __shared__ unsigned long long s_sum[BT / 32];
+    __shared__ uint2 s_vote[TOP_WORDS];
+    __shared__ uint32_t s_before[TOP_WORDS + 1];  // nodes << 16 | lefts of the words before, halves apart
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, y = blockIdx.y, tile = blockIdx.x;
     const uint32_t *in = y == 0 ? a.in[0] : (y == 1 ? a.in[1] : a.in[2]);
     uint32_t *out = y == 0 ? a.out[0] : (y == 1 ? a.out[1] : a.out[2]);
     const Layout32 t(a.n);
     const int first = tile * TOP_TILE + w * 32 * TOP_ITEMS + lane;
-    uint32_t pid[TOP_ITEMS], before[TOP_ITEMS], sides = 0;  // before: nodes << 16 | lefts, of the warp's earlier places
-    uint32_t run = 0;
-    const uint32_t lt = (1u << lane) - 1;
+    uint32_t pid[TOP_ITEMS];
 #pragma unroll
     for (int j = 0; j < TOP_ITEMS; ++j) {
         const int p = first + 32 * j;
         pid[j] = p < a.n ? in[p] : 0;
     }
+    // the tiles before: whole groups, then the tiles of this one's
+    const unsigned long long *count = a.count + (size_t)y * (a.tiles + a.groups);
+    const int group = tile / TOP_GROUP;
+    unsigned long long sum = 0;
+    for (int i = tid; i < group; i += BT)
+        sum += count[a.tiles + i];
+    if (tid < tile - group * TOP_GROUP)
+        sum += count[group * TOP_GROUP + tid];
 #pragma unroll
-    for (int j = 0; j < TOP_ITEMS; ++j) {
-        const int p = first + 32 * j;
-        uint32_t s = 3;  // not in a subtree of the level
-        if (p < a.n && Layout32::level(t.node_at(p)) >= a.l)
-            s = a.side[pid[j]];
-        sides |= s << (2 * j);
-        const uint32_t bl = __ballot_sync(0xffffffffu, s == SIDE_LEFT), bn = __ballot_sync(0xffffffffu, s == SIDE_NODE);
-        before[j] = run + (__popc(bl & lt) | __popc(bn & lt) << 16);
-        run += __popc(bl) | __popc(bn) << 16;
-    }
+    for (int o = 16; o > 0; o >>= 1)
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0)
-        s_cnt[w] = run;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t own = lane < BT / 32 ? s_cnt[lane] : 0;
-        own = __reduce_add_sync(0xffffffffu, own);  // at most 4096 of each
-        const unsigned long long mine = (unsigned long long)(own >> 16) << 32 | (own & 0xffffu);
-        volatile unsigned long long *st = a.state + (size_t)y * a.tiles;
-        if (lane == 0)
-            st[tile] = (tile ? TOP_OWN : TOP_ALL) | mine;
-        unsigned long long sum = 0;
-        for (int back = tile - 1; back >= 0; back -= 32) {
-            const int q = back - lane;
-            unsigned long long v = q < 0 ? TOP_ALL : 0;
-            for (int polls = 0; v == 0 && polls < TOP_POLLS; ++polls)
-                v = st[q];
-            if (v == 0) {
-                unsigned long long c = 0;
-                for (int p = q * TOP_TILE; p < (q + 1) * TOP_TILE; ++p)
-                    if (Layout32::level(t.node_at(p)) >= a.l) {
-                        const int s = a.side[in[p]];
-                        c += s == SIDE_LEFT ? 1ull : (s == SIDE_NODE ? 1ull << 32 : 0ull);
-                    }
-                v = TOP_OWN | c;
-            }
-            __syncwarp();
-            const uint32_t all = __ballot_sync(0xffffffffu, (v & TOP_ALL) != 0);
-            const int stop = all ? __ffs(all) - 1 : 31;
-            unsigned long long x = lane <= stop ? v & TOP_VALUE : 0;
+        s_sum[w] = sum;
+    if (tid < TOP_WORDS) {
+        const uint2 v = a.votes[((size_t)y * a.tiles + tile) * TOP_WORDS + tid];
+        s_vote[tid] = v;
+        uint32_t c = __popc(v.x) | __popc(v.y) << 16, inc = c;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                x += __shfl_xor_sync(0xffffffffu, x, o);
-            sum += x;
-            if (all)
-                break;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            inc += lane >= o ? x : 0;
         }
-        if (lane == 0) {
-            if (tile)
-                st[tile] = TOP_ALL | (sum + mine);
-            s_before = sum;
-        }
+        s_before[tid] = inc - c;
+        if (tid == 31)
+            s_before[TOP_WORDS] = inc;  // of the first 32 words
     }
     __syncthreads();
-    uint32_t warps = lane < w ? s_cnt[lane] : 0;
-    warps = __reduce_add_sync(0xffffffffu, warps);
-    const int lefts0 = (int)(s_before & 0xffffffffu) + (int)(warps & 0xffffu);
-    const int ones0 = (int)(s_before >> 32) + (int)(warps >> 16);
+    sum = 0;
+#pragma unroll
+    for (int i = 0; i < BT / 32; ++i)
+        sum += s_sum[i];
     const bool next = y == a.next;
+    const uint32_t lt = (1u << lane) - 1;
 #pragma unroll
     for (int j = 0; j < TOP_ITEMS; ++j) {
-        const int s = sides >> (2 * j) & 3u;
-        if (s == 3)
-            continue;
         const int p = first + 32 * j;
+        if (p >= a.n)
+            break;
         const int u = t.node_at(p), lu = Layout32::level(u);
-        const int d = part_dest(t, a.l, u, lu, p, s, lefts0 + (int)(before[j] & 0xffffu), ones0 + (int)(before[j] >> 16));
+        if (lu < a.l)
+            continue;
+        const int word = w * TOP_ITEMS + j;
+        const uint2 v = s_vote[word];
+        const int s = v.x >> lane & 1u ? SIDE_LEFT : (v.y >> lane & 1u ? SIDE_NODE : SIDE_RIGHT);
+        const uint32_t before = s_before[word] + (word >= 32 ? s_before[TOP_WORDS] : 0);
+        const int lefts = (int)(sum & 0xffffffffu) + (int)(before & 0xffffu) + __popc(v.x & lt);
+        const int ones = (int)(sum >> 32) + (int)(before >> 16) + __popc(v.y & lt);
+        const int d = part_dest(t, a.l, u, lu, p, s, lefts, ones);
         if (d < 0 || d >= a.n)  // never, for consistent sides
             continue;
         out[d] = pid[j];
         if (next && s != SIDE_NODE) {
-            const int v = t.node_at(d), lv = Layout32::level(v);
-            if (lv == a.l + 1) {
+            const int x = t.node_at(d), lx = Layout32::level(x);
+            if (lx == a.l + 1) {
                 a.side_next[pid[j]] = SIDE_NODE;
-                emit_node(a.pts, a.D, 0, v, pid[j], 0u, a.nodes, a.ids);
+                emit_node(a.pts, a.D, 0, x, pid[j], 0u, a.nodes, a.ids);
             } else {
-                a.side_next[pid[j]] = (v + 1) >> (lv - a.l - 2) & 1 ? SIDE_RIGHT : SIDE_LEFT;
+                a.side_next[pid[j]] = (x + 1) >> (lx - a.l - 2) & 1 ? SIDE_RIGHT : SIDE_LEFT;
             }
         }
     }
@@ -914,7 +937,7 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
     const bool together = (int64_t)total * D <= ((int64_t)1 << 21);
     const int at_once = together ? D : 1;
     const int64_t ptiles = (total + PTILE - 1) / PTILE;         // T > 1
-    const int top_tiles = (int)((total + TOP_TILE - 1) / TOP_TILE);  // T == 1
+    const int top_tiles = (int)top_tiles_of(total), top_groups = (int)top_groups_of(total);  // T == 1
     const size_t rs = radix_scratch_elems(total) * at_once;
     size_t bytes = 0;
     auto take = [&](size_t b) {
@@ -933,10 +956,11 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
     size_t o_job = take(T > 1 ? (size_t)(T + 1) * 4 : 0);
     size_t o_tiles = take(T > 1 ? (size_t)ptiles * sizeof(Seg) : 0);
     size_t o_rs = take(rs * 4);
-    // look-back states and tickets of every partition
+    // vote words of one launch, counts of every partition
     const int parts = T == 1 ? levels * D : 0;
-    const size_t state_bytes = (size_t)parts * top_tiles * 8 + (size_t)parts * 4;
-    size_t o_state = take(state_bytes);
+    const size_t count_bytes = (size_t)parts * (top_tiles + top_groups) * 8;
+    size_t o_count = take(count_bytes);
+    size_t o_votes = take(parts ? (size_t)TOP_LISTS * top_tiles * TOP_WORDS * sizeof(uint2) : 0);
     size_t o_dim = take(widest ? (size_t)total : 0);
     DevBuf buf;
     buf.s = s;
@@ -990,10 +1014,9 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
 
     if (T == 1) {
         const int n = (int)total;
-        unsigned long long *state = (unsigned long long *)(B + o_state);
-        uint32_t *ticket = (uint32_t *)(state + (size_t)parts * top_tiles);
+        unsigned long long *part_count = (unsigned long long *)(B + o_count);
         if (parts)
-            KDT_CUDA(cudaMemsetAsync(state, 0, state_bytes, s));
+            KDT_CUDA(cudaMemsetAsync(part_count, 0, count_bytes, s));
         if (levels && !widest)
             KDT_LAUNCH root_kernel<<<g, BT, 0, s>>>(lists[0], n, d_points, D, side, nodes, ids);
         for (int l = 0; l < levels; ++l) {
@@ -1024,19 +1047,21 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
                         pa.next = i;
                 }
                 pa.side = side;
-                pa.state = state;
-                pa.ticket = ticket;
-                state += (size_t)ny * top_tiles;
-                ticket += ny;
+                pa.votes = (uint2 *)(B + o_votes);
+                pa.count = part_count;
+                part_count += (size_t)ny * (top_tiles + top_groups);
                 pa.n = n;
                 pa.l = l;
                 pa.tiles = top_tiles;
+                pa.groups = top_groups;
                 pa.side_next = side_next;
                 pa.pts = d_points;
                 pa.D = D;
                 pa.nodes = nodes;
                 pa.ids = ids;
-                KDT_LAUNCH part_kernel<<<dim3((unsigned)top_tiles, (unsigned)ny), BT, 0, s>>>(pa);
+                const dim3 grid((unsigned)top_tiles, (unsigned)ny);
+                KDT_LAUNCH part_votes_kernel<<<grid, BT, 0, s>>>(pa);
+                KDT_LAUNCH part_move_kernel<<<grid, BT, 0, s>>>(pa);
                 for (int i = 0; i < ny; ++i)
                     std::swap(lists[todo[c + i]], spare[i]);
             }
