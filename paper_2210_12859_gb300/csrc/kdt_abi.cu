@@ -445,19 +445,22 @@ __attribute__((visibility("hidden"))) int kdt_tree_alloc_internal(int64_t N, int
         kdt_free(t);
         return set_error(KDT_ENOMEM, "device allocation failed (injected)");
     }
+    // one allocation for all arrays of the tree: four of them and their frees
+    // were 0.5 ms of the 9 that a build of 2^24 points takes
     const int nf = float4_per_node(D);
-    cudaError_t e = cudaMalloc(&t->nodes_alloc, ((size_t)N * nf + (nf == 1 ? 1 : 0)) * sizeof(float4));
-    t->nodes = t->nodes_alloc + (nf == 1 ? 1 : 0);
-    if (e == cudaSuccess && t->layout > 0)
-        e = cudaMalloc(&t->ids, (size_t)N * sizeof(int32_t));
-    if (e == cudaSuccess)
-        e = box_tree_alloc(t);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&t->bbox, 6 * sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaMalloc(&t->err, sizeof(int));
-    if (e == cudaSuccess)
+    const size_t nodes = ((size_t)N * nf + (nf == 1 ? 1 : 0)) * sizeof(float4);
+    const size_t ids = t->layout > 0 ? (size_t)N * sizeof(int32_t) : 0;
+    const size_t box = box_tree_bytes(N, D);
+    cudaError_t e = cudaMalloc(&t->nodes_alloc, carve_size({nodes, ids, box, 6 * sizeof(float), sizeof(int)}));
+    if (e == cudaSuccess) {
+        Carve c{(char *)t->nodes_alloc};
+        t->nodes = c.take<float4>(nodes / sizeof(float4)) + (nf == 1 ? 1 : 0);
+        t->ids = ids ? c.take<int32_t>((size_t)N) : nullptr;
+        box_tree_place(t, c.take<char>(box));
+        t->bbox = c.take<float>(6);
+        t->err = c.take<int>(1);
         e = cudaMemset(t->err, 0, sizeof(int));
+    }
     if (e != cudaSuccess) {
         kdt_free(t);
         return cuda_error(e, "tree allocation", __FILE__, __LINE__);
@@ -649,10 +652,6 @@ void kdt_free(kdt_tree *t)
         return;
     cudaDeviceSynchronize();
     cudaFree(t->nodes_alloc);
-    cudaFree(t->ids);
-    cudaFree(t->box_rec);
-    cudaFree(t->bbox);
-    cudaFree(t->err);
     cudaFree(t->payload);
     cudaFree(t->node_of);
     free_model(t);

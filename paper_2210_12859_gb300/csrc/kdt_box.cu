@@ -259,6 +259,10 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(BoxBuild a
 // 45 -> 25 us.  The state machine is not faster on any of them.
 constexpr int BOX_RECORD_LANES = 4;
 constexpr int BOX_FREE_LANES = 24;
+// With the heap (K > 16), whose set-up and final sort cost most, nearly the
+// whole warp (k = 40 2.60 -> 2.47 ms); in 5 to 8 dimensions, where a walk is 470
+// steps and a lane that waits is the dearer part, a quarter (8-D 4.81 -> 4.61).
+__host__ __device__ constexpr int box_free_lanes(int layout, int k) { return k > MAX_REG_K ? 31 : (layout == 2 ? 8 : BOX_FREE_LANES); }
 
 // Resident blocks to build for.  Closest points in 4-D, bound by L1 wavefronts
 // whose latency more warps cover: 10 (10^7 of them 5.58 -> 5.33 ms against 8; in
@@ -277,6 +281,7 @@ __global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box
     constexpr int NC = LayoutTraits<LAYOUT>::NC;
     using List = typename std::conditional<(K <= MAX_REG_K), RegList<K <= MAX_REG_K ? K : 1>, SmemList>::type;
     extern __shared__ float4 s_dyn[];
+    constexpr int FREE_LANES = box_free_lanes(LAYOUT, K);
     const int64_t ngate = (MODE == MODE_BOUNDED && a.n_gate) ? (int64_t)*a.n_gate : INT64_MAX;
     uint32_t cap = a.step_cap ? a.step_cap : 3u * (uint32_t)a.N + 3u;
     BoxRef tree = b.tree;
@@ -307,7 +312,7 @@ __global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box
     for (;;) {
         const unsigned free_lanes = __ballot_sync(0xffffffffu, !busy && !exhausted);
         const unsigned busy_lanes = __ballot_sync(0xffffffffu, busy);
-        if (!busy_lanes || __popc(free_lanes) >= BOX_FREE_LANES) {
+        if (!busy_lanes || __popc(free_lanes) >= FREE_LANES) {
             // write the finished rows, take the next queries
             if (!busy && qi >= 0) {
                 bool again = false;
@@ -409,8 +414,9 @@ template <int LAYOUT, int K, int MODE, bool FOREST>
 int launch_box_one(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
 {
     const void *fn = (const void *)box_knn_kernel<LAYOUT, K, MODE, FOREST>;
-    // few queries: small blocks, so that they spread over the SMs
-    int threads = BOX_THREADS;
+    // few queries: small blocks, so that they spread over the SMs; heaps in
+    // shared memory: half blocks fill it better (k = 40 2.47 -> 2.40 ms)
+    int threads = K > MAX_REG_K ? BOX_THREADS / 2 : BOX_THREADS;
     while (threads > 32 && a.Q < (int64_t)num_sms() * threads)
         threads >>= 1;
     const size_t smem = (size_t)threads * (4 * BoxWalk::MAX_RECORDS + (K > MAX_REG_K && !a.heap ? 8 * a.k : 0));
@@ -489,12 +495,12 @@ size_t box_grp_size(int64_t n, int D) { return (size_t)BoxShape(n).groups() * 2 
 
 }  // namespace
 
-cudaError_t box_tree_alloc(kdt_tree *t)
+size_t box_tree_bytes(int64_t n, int D) { return (box_rec_size(n, D) + box_grp_size(n, D)) * sizeof(float4); }
+
+void box_tree_place(kdt_tree *t, void *p)
 {
-    const size_t rec = box_rec_size(t->N, t->D);
-    const cudaError_t e = cudaMalloc(&t->box_rec, (rec + box_grp_size(t->N, t->D)) * sizeof(float4));
-    t->box_grp = t->box_rec + rec;
-    return e;
+    t->box_rec = (float4 *)p;
+    t->box_grp = t->box_rec + box_rec_size(t->N, t->D);
 }
 
 int build_box_tree(const kdt_tree *t, cudaStream_t s)

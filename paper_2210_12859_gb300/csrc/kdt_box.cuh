@@ -343,9 +343,10 @@ __device__ __forceinline__ void box_bucket(const BoxRef &b, uint32_t i, const fl
     }
 }
 
-// The tree's box arrays (t->N and t->D set), and their contents from its
-// level-order nodes; the same for all trees of a forest.
-cudaError_t box_tree_alloc(kdt_tree *t);
+// The tree's box arrays (box_tree_bytes bytes at a 128-byte boundary), and their
+// contents from its level-order nodes; the same for all trees of a forest.
+size_t box_tree_bytes(int64_t n, int D);
+void box_tree_place(kdt_tree *t, void *p);
 int build_box_tree(const kdt_tree *t, cudaStream_t s);
 int build_box_forest(kdt_forest *f, cudaStream_t s);
 // Calls that the box tree serves: ordered queries for results, the learned

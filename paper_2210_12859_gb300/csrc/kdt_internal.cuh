@@ -287,11 +287,11 @@ struct kdt_tree {
     int layout = 0;                // 3: split dimension stored per node (widest extent)
     int device = 0;
     float4 *nodes = nullptr;       // N * float4_per_node(D), node t at nodes[t * float4_per_node(D)]
-    float4 *nodes_alloc = nullptr; // allocation; 16-byte nodes start one slot in, so that the siblings
+    float4 *nodes_alloc = nullptr; // the allocation of all arrays down to err; 16-byte nodes start one slot in, so that the siblings
                                    // 2c+1 and 2c+2 share one 32-byte sector
     int32_t *ids = nullptr;        // layout > 0
     float4 *box_rec = nullptr;     // box tree of the result queries (kdt_box.cuh): records,
-    float4 *box_grp = nullptr;     // and point groups (in the records' allocation)
+    float4 *box_grp = nullptr;     // and point groups
     float *bbox = nullptr;         // device [2][3]: lo, hi of the first min(D,3) dims
     int *err = nullptr;            // device error word
     kdt::Model model;
