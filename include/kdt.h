@@ -51,9 +51,10 @@ extern "C" {
 #define KDT_UNORDERED  0x1 /* left child first; a child is entered iff the query is on its
                               side or the splitting plane is within the cull radius
                               (Sec. 3: unordered traversal as a simplification) */
-#define KDT_MORTON     0x2 /* sort queries along a 30-bit Morton curve before traversal so
-                              that the threads of a warp walk nearby paths; results are
-                              written to the caller's query order */
+#define KDT_MORTON     0x2 /* sort queries by the path of their greedy descent in the tree
+                              before traversal (a space-filling order that follows the
+                              points) so that the threads of a warp walk nearby paths;
+                              results are written to the caller's query order */
 #define KDT_LEARNED    0x4 /* seed each query's cull radius with the trained radius model
                               and re-run the queries that find fewer than k points with
                               the caller's radius (not in the paper; results unchanged) */
@@ -62,7 +63,7 @@ extern "C" {
                               classes, most expensive first (judged by how far the greedy
                               descent ends from its leaf point, relative to the mean point
                               spacing: one class per power of two of that squared distance
-                              beyond 64 spacings squared, three below), Morton order within a
+                              beyond 64 spacings squared, three below), path order within a
                               class.  Pays when a few queries cost far more than the rest
                               (queries outside the data); costs one descent per query */
 /* Traversal ablations (ordered kNN / fcp, k <= 16, D <= 4; at most one; not
@@ -171,7 +172,7 @@ int kdt_knn_visits(const kdt_tree *tree, const float *d_queries, int64_t Q, int 
  * d_offsets int64 [Q+1] (exclusive prefix sums, offsets[Q] = total); *_fill
  * writes query q's point ids (and, for balls, squared distances if d_d2 is not
  * NULL) to [offsets[q], offsets[q+1]) in traversal order, the same on every
- * call.  flags: 0 or KDT_MORTON (queries run in Morton order; results are the
+ * call.  flags: 0 or KDT_MORTON (queries run in path order; results are the
  * same), plus KDT_RANGE_VISITS for the count calls; any other bit is
  * KDT_EINVAL.  A fill whose hits do not match its
  * offsets writes nothing outside the query's slice and is reported by
@@ -425,6 +426,14 @@ void kdt_forest_free(kdt_forest *forest);
 
 /* ---- launch tuning -------------------------------------------------------- */
 
+/* Ordered result queries (kdt_knn, kdt_fcp, kdt_knn_static, kdt_knn_host and
+ * kdt_knn_batched without KDT_UNORDERED or an ablation flag) walk a box tree
+ * that every build makes beside the level-order tree: the bounding boxes of
+ * subtrees, in all coordinates, instead of one splitting plane a test.  The
+ * result is the same.  The staging depth, claim steps, inline depth and light
+ * run below are choices of the state machine's kernels (unordered queries,
+ * counts of processed nodes, the learned counts) and change nothing there. */
+
 /* The traversal kernels copy the top `levels` levels of the tree (2^levels - 1
  * nodes) into shared memory once per block.  Staging trades L1 capacity (the
  * same on-chip array) for the latency of the top-level loads; the best depth
@@ -489,7 +498,8 @@ int kdt_large_k_list(const kdt_tree *tree, int k, int *placement);
 int kdt_tuned_params(const kdt_tree *tree, int k, int *stage_levels, int *claim_steps, int *inline_depth,
                      int *light_run);
 
-/* Time the plain traversal of up to 2^20 of the given queries and remember
+/* Time the state machine on up to 2^20 of the given queries (ordered: its
+ * count of processed nodes; unordered: the query) and remember
  * the fastest launch parameters for this tree's shape (GPU name, D, k bucket,
  * floor(log2 N)): a coordinate search over the inline depth {2, 1, 0}, the
  * light run {1, 4, 8}, then the claim steps {16, 32, 64, 128}, then the
@@ -497,7 +507,7 @@ int kdt_tuned_params(const kdt_tree *tree, int k, int *stage_levels, int *claim_
  * candidate timed over two launches after a warm-up and taken only when it is
  * faster than the best so far by 2 % (staging: 5 %).  Later queries on trees of that shape use the choice unless
  * the kdt_set_* calls override.  Synchronous.  *best_levels and *best_ms (may
- * be NULL) receive the staging depth and the best time per launch;
+ * be NULL) receive the staging depth and the time of the query itself per launch;
  * kdt_tuned_params reports all three. */
 int kdt_autotune(kdt_tree *tree, const float *d_queries, int64_t Q, int k, int flags, int *best_levels,
                  float *best_ms, void *stream);

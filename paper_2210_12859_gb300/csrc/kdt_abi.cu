@@ -304,19 +304,22 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
 {
     pool_setup_once();
     const bool morton = flags & KDT_MORTON;
-    const bool gheap = heap_in_global(t, k);
+    QueryArgs a;
+    a.group = list_group_for(t, k);
+    a.out_ids = d_ids;
+    a.visits = d_visits;
+    const bool boxed = box_query_serves(a, flags, mode);
+    const bool gheap = heap_in_global(t, k, boxed);
     const size_t heap_bytes = gheap ? (size_t)heap_scratch_threads() * k * 8 : 0;
     size_t bytes = carve_size({64, heap_bytes}) + (morton ? morton_scratch_bytes(Q) : 0);
     Scratch sc(s);
     KDT_TRY(sc.alloc(bytes));
     Carve c{(char *)sc.p};
     unsigned long long *counter = c.take<unsigned long long>(8);
-    QueryArgs a;
     if (gheap) {
         a.heap = c.take<unsigned long long>(heap_bytes / 8);
         a.heap_threads = heap_scratch_threads();
     }
-    a.group = list_group_for(t, k);
     if (morton)
         KDT_TRY(query_order(t, d_q, Q, flags & KDT_COST_ORDER, c.base + c.off, const_cast<uint32_t **>(&a.perm), s));
     a.nodes = t->nodes;
@@ -346,7 +349,7 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
         a.inline_depth = 1;
     if (flags & (KDT_PLAIN_STEP | KDT_CLOSE_FIRST | KDT_STACK))
         KDT_TRY(launch_ablation(t->layout, a, flags, mode, s));
-    else if (box_query_serves(a, flags, mode))
+    else if (boxed)
         KDT_TRY(launch_box_query(t, a, mode, s));
     else if (simple)
         KDT_TRY(launch_ablation(t->layout, a, KDT_PLAIN_STEP, mode, s));

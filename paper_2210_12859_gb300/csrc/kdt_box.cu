@@ -251,12 +251,12 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(BoxBuild a
 // point in 4-D 6.81 -> 6.58 ms).
 //
 // Bound: the arithmetic and selects of buckets and lists in 3-D with k >= 8
-// (issue slots 59 %, the ALU pipe 90 % busy), L1 wavefronts in 4-D and above
-// with incoherent queries (98 %).  Against the state machine's kernel: clustered
-// 2^24, k = 8 1040 -> 18.5 ms (13.3 k processed nodes a query -> 56 records and
-// 14 buckets), surface 2^22, k = 16 10.2 -> 3.8 ms, 8-D k = 10 23.3 -> 5.4 ms,
-// 10^7 closest points in 4-D 8.8 -> 6.6 ms, a scan of 5003 closest points
-// 45 -> 25 us.  The state machine is not faster on any of them.
+// (12 to 14 of 32 lanes active), L1 wavefronts in 4-D with incoherent queries
+// (98 %).  Whole passes against the state machine's kernel: clustered 2^24, k = 8
+// 1060 -> 19.2 ms (13.3 k processed nodes a query -> 56 records and 14 buckets),
+// surface 4 M, k = 16 10.3 -> 2.76 ms, 8-D k = 10 24.4 -> 4.49 ms, 10^7 closest
+// points in 4-D 8.76 -> 5.24 ms, a scan of 5003 closest points 46 -> 25 us.  The
+// state machine is not faster on any of them.
 constexpr int BOX_RECORD_LANES = 4;
 constexpr int BOX_FREE_LANES = 24;
 // With the heap (K > 16), whose set-up and final sort cost most, nearly the

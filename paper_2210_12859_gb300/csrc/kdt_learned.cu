@@ -326,7 +326,8 @@ int run_learned_query(kdt_tree *t, const float *d_q, int64_t Q, int k, float r2,
     if (gate == KDT_GATE_FAR)
         flags |= KDT_MORTON | KDT_COST_ORDER;
     const bool morton = flags & KDT_MORTON;
-    const size_t heap_bytes = heap_in_global(t, k) ? (size_t)heap_scratch_threads() * k * 8 : 0;
+    const bool boxed = d_ids && !d_visits && !(flags & KDT_UNORDERED);
+    const size_t heap_bytes = heap_in_global(t, k, boxed) ? (size_t)heap_scratch_threads() * k * 8 : 0;
     size_t off_w = 0, off_r2 = 1 << 15;
     size_t off_h = off_r2 + (((size_t)Q * 4 + 255) & ~(size_t)255);
     size_t off_m = off_h + heap_bytes;

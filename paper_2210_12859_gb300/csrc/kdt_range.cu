@@ -513,6 +513,7 @@ __global__ void __launch_bounds__(RANGE_THREADS) range_visits_kernel(const Range
     int curr = 0, prev = -1, dim = 0, visits = 0;
     uint32_t steps = 0;
     const uint32_t cap = 3u * (uint32_t)a.N + 3u;
+    const int bottom = a.N >> 2;  // from here on a node's children have no children
     for (;;) {
         const bool need = qi < 0 && !exhausted;
         const int64_t slot = claim_slot(need, a.counter);
@@ -563,7 +564,11 @@ __global__ void __launch_bounds__(RANGE_THREADS) range_visits_kernel(const Range
             left_ok = left_ok && lc < a.N;
             right_ok = right_ok && rc < a.N;
             int next;
-            if (from_parent)
+            if (from_parent && curr >= bottom) {
+                // the children are leaves: entered and left again
+                visits += left_ok + right_ok;
+                next = parent;
+            } else if (from_parent)
                 next = left_ok ? lc : (right_ok ? rc : parent);
             else if (prev == lc)
                 next = right_ok ? rc : parent;

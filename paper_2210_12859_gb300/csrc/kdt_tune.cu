@@ -1,4 +1,6 @@
-// Launch tuning of the traversal kernels.  Three choices never change a result
+// Launch tuning of the state machine's kernels (unordered queries, counts of
+// processed nodes, forms asked for by name; ordered result queries walk the box
+// tree, kdt_box.cu, and take none of these).  The choices never change a result
 // (every combination processes the same nodes in the same order) but move its
 // speed, and the best values depend on how much work a query does:
 //   * stage_levels: top tree levels staged in shared memory (saves the latency
@@ -144,7 +146,10 @@ static int large_k_list_of(const kdt_tree *t, int k)
     return tuned_for(t, k, &v) ? v.large_k_list : DEFAULT_LARGE_K_LIST;
 }
 
-bool heap_in_global(const kdt_tree *t, int k) { return k > 16 && large_k_list_of(t, k) == KDT_LIST_GLOBAL; }
+bool heap_in_global(const kdt_tree *t, int k, bool box)
+{
+    return k > 16 && (box ? t->large_k_list : large_k_list_of(t, k)) == KDT_LIST_GLOBAL;
+}
 
 int list_group_for(const kdt_tree *t, int k)
 {
@@ -272,6 +277,10 @@ int kdt_autotune(kdt_tree *t, const float *d_q, int64_t Q, int k, int flags, int
                DEFAULT_LARGE_K_LIST};
     float best_t = 3.4e38f;
     int rc = KDT_OK;
+    // the choices belong to the state machine: of the ordered calls it still
+    // serves the counts of processed nodes, so they are timed on these
+    const bool ordered = !(flags & KDT_UNORDERED);
+    int mode = ordered ? MODE_VISITS : MODE_RESULTS;
     auto measure = [&](const Tuned &c, float *out) {
         t->stage_levels = c.stage_levels;
         t->claim_steps = c.claim_steps;
@@ -279,7 +288,9 @@ int kdt_autotune(kdt_tree *t, const float *d_q, int64_t Q, int k, int flags, int
         t->light_run = c.light_run;
         t->large_k_list = c.large_k_list;
         for (int rep = 0; rep < 3 && rc == KDT_OK; ++rep) {
-            rc = run_query(t, d_q, n, k, INFINITY, flags & ~KDT_NO_STAGE, MODE_RESULTS, ids, d2, nullptr, s);
+            rc = mode == MODE_RESULTS
+                     ? run_query(t, d_q, n, k, INFINITY, flags & ~KDT_NO_STAGE, MODE_RESULTS, ids, d2, nullptr, s)
+                     : run_query(t, d_q, n, k, INFINITY, flags & ~KDT_NO_STAGE, MODE_VISITS, nullptr, nullptr, ids, s);
             if (rc == KDT_OK && rep == 0)
                 rc = cudaEventRecord(e0, s) == cudaSuccess ? KDT_OK : set_error(KDT_ECUDA, "event record");
         }
@@ -347,6 +358,13 @@ int kdt_autotune(kdt_tree *t, const float *d_q, int64_t Q, int k, int flags, int
             if (rc == KDT_OK && stage_fits(t, lv, 64 * 1024))
                 consider(c, 0.05f);
         }
+    }
+    if (ordered && rc == KDT_OK) {
+        // the reported time is the query's
+        mode = MODE_RESULTS;
+        Tuned c = best;
+        c.large_k_list = saved_list;
+        measure(c, &best_t);
     }
     t->stage_levels = saved_stage;
     t->claim_steps = saved_claim;

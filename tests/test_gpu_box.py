@@ -116,3 +116,15 @@ def test_forests(kdt, D):
             want = kdt.kdt_knn_batched(forest, dq, qoff, k, r, kdt.KDT_UNORDERED)
             for flags in (0, kdt.KDT_MORTON, kdt.KDT_PER_TREE):
                 assert same(kdt.kdt_knn_batched(forest, dq, qoff, k, r, flags), want), (k, r, flags)
+
+
+@pytest.mark.parametrize("Q", [1, 2, 33, 1023, 1024, 1025, 4097, 16384, 16385, (1 << 19) + 3])
+def test_ordered_queries_at_the_edges_of_the_sort(kdt, Q):
+    """Queries that run in path or cost order give every row, whatever the
+    number of queries: tiles of the radix sort and the numbers of its passes."""
+    g = np.random.default_rng(Q)
+    tree = kdt.kdt_build(torch.from_numpy(g.random((30011, 3), dtype=np.float32)).cuda())
+    dq = torch.from_numpy(g.random((Q, 3), dtype=np.float32) * 1.4 - 0.2).cuda()
+    want = kdt.kdt_knn(tree, dq, 4)
+    for flags in (kdt.KDT_MORTON, kdt.KDT_MORTON | kdt.KDT_COST_ORDER):
+        assert same(kdt.kdt_knn(tree, dq, 4, flags=flags), want)
