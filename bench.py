@@ -221,7 +221,7 @@ def workload_config(log2n):
     return {
         "workload": f"gmm_large: N=2^{log2n} 3-D float32 points, 64-component Gaussian mixture (sigma 0.01, "
                     f"centres U[0,1]^3); Q=2^{log2n} queries (90% mixture, 10% uniform [0,1]^3); kNN k=8, "
-                    "max_radius=inf, ordered stack-free traversal, Morton query order with expensive queries first; "
+                    "max_radius=inf, ordered queries by subtree boxes, in the order of their paths with expensive queries first; "
                     "step = tree build + "
                     "all queries",
         "N": 1 << log2n, "Q": 1 << log2n, "D": 3, "k": K_NN,
@@ -231,7 +231,7 @@ def workload_config(log2n):
 
 # ---------------------------------------------------------------- profile data
 
-KERNEL_SOURCES = ("kdt_traverse.cuh", "kdt_query_impl.cuh", "kdt_query.cuh")
+KERNEL_SOURCES = ("kdt_box.cuh", "kdt_box.cu", "kdt_traverse.cuh", "kdt_query.cuh")
 
 
 def kernel_source_hash() -> str:
@@ -246,7 +246,7 @@ def kernel_source_hash() -> str:
 def profiled_traffic():
     """DRAM bytes per launch of the traversal kernel from the committed ncu
     summary, or None when the kernel source changed since it was captured."""
-    path = os.path.join(ROOT, "profiles", "knn_kernel_gmm2p24_dram.txt")
+    path = os.path.join(ROOT, "profiles", "box_knn_gmm2p24_dram.txt")
     try:
         kv = dict(line.split(":", 1) for line in open(path) if ":" in line and not line.startswith("#"))
     except OSError:
@@ -391,7 +391,9 @@ def main():
         hbm = 6800.0
         peak_src = "fallback"
     kern_ms = trav_ms / max(trav_launches, 1)
-    bytes_per_launch = n * (4 * 3 + 8 * K_NN) + v_sum * 16.0
+    # what no kernel can do without: queries and points (with their ids) read
+    # once, results written once
+    bytes_per_launch = n * (4 * 3 + 8 * K_NN) + n * 16.0
     achieved = bytes_per_launch / (kern_ms / 1000.0) / 1e9
     traffic = profiled_traffic()
     # the same algorithmic bytes against L2: the read bandwidth of a 32 MiB
@@ -400,9 +402,9 @@ def main():
     l2_note = "L2 read bandwidth measured by the library's probe (32 MiB buffer, 16-byte L1-bypassing loads)"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                 "traffic": traffic, "peak_source": peak_src,
-                "kernel": "knn_kernel<layout0,K=8,ordered> (stack-free traversal)",
+                "kernel": "box_knn_kernel<layout0,K=8> (walk of the box tree)",
                 "kernel_ms": kern_ms, "bytes_per_query": bytes_per_launch / n,
-                "visits_per_query": v_mean,
+                "state_machine_visits_per_query": v_mean,
                 "l2": {"achieved": achieved, "peak": l2_gbs, "unit": "GB/s", "frac": achieved / l2_gbs,
                        "peak_source": l2_note}}
 
@@ -428,9 +430,8 @@ def main():
         same = bool(torch.equal(li, out_i) and torch.equal(ld.view(torch.int32), out_d.view(torch.int32)))
         lv = kdt.kdt_knn_visits(tree, dq, K_NN, math.inf, flags | kdt.KDT_LEARNED)
         lv_sum = float(lv.double().sum().item())
-        # algorithmic bytes: as the plain query, with the processed nodes of
-        # the bounded and re-run passes, plus 16 B of features per gated query
-        l_bytes = n * (4 * 3 + 8 * K_NN) + lv_sum * 16.0 + 16.0 * gated
+        # as the plain query, plus 16 B of features per gated query
+        l_bytes = bytes_per_launch + 16.0 * gated
         l_ach = l_bytes / (learned_ms / 1000.0) / 1e9
         learned = {"query_qps": n / (learned_ms / 1000.0), "query_ms": learned_ms,
                    "plain_query_qps": n / (plain_loop_ms / 1000.0), "plain_query_ms": plain_loop_ms,

@@ -175,8 +175,8 @@ def run_config(args):
                   timing=f"{steps} calls of each form after {warm} warm-up calls",
                   fallback_rate=fb / n, radius_ratio=ratio,
                   plain_visits=pv / n, learned_visits=lv / n, identical=same, train_s=train_s, train_loss=loss,
-                  roofline_plain=_roofline(n * (12 + 8 * k) + 16.0 * pv, plain_ms, hbm, src, l2, "plain query call"),
-                  roofline_learned=_roofline(n * (12 + 8 * k) + 16.0 * lv + 16.0 * gated, learned_ms, hbm, src, l2,
+                  roofline_plain=_roofline(n * (12 + 8 * k) + 16.0 * n, plain_ms, hbm, src, l2, "plain query call"),
+                  roofline_learned=_roofline(n * (12 + 8 * k) + 16.0 * n + 16.0 * gated, learned_ms, hbm, src, l2,
                                              "learned query call (features and network included)"),
                   bit_exact_sample=_exact(oracle, pts, qs, out_i.cpu().numpy(), out_d.cpu().numpy(), k))
         return
@@ -248,9 +248,9 @@ def run_config(args):
         ok = all(np.array_equal(np.sort(idsh[offh[q]:offh[q + 1]]), wids[woff[j]:woff[j + 1]])
                  for j, q in enumerate(sample))
         visits = kdt.kdt_radius_count(tree, dq, r, F | kdt.KDT_RANGE_VISITS).double().sum().item()
-        # algorithmic bytes of the fill pass: query 12 B + 16 B per processed
-        # node + 8 B per hit (id, d2) + 16 B of offsets, against measured HBM
-        fill_bytes = nq * (12 + 16) + 16.0 * visits + 8.0 * total
+        # bytes the fill pass cannot do without: query 12 B + 16 B of offsets,
+        # the points once (at most one per hit), 8 B per hit (id, d2)
+        fill_bytes = nq * (12 + 16) + 16.0 * min(len(pts), total) + 8.0 * total
         try:
             peaks = json.load(open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "MEASURED_PEAKS.json")))
             hbm = float(peaks.get("hbm_gbs", 6800.0))
@@ -280,14 +280,15 @@ def run_config(args):
                                  lwids[lwoff[j]:lwoff[j + 1]]) for j, q in enumerate(lsample))
         del ld2
         lvisits = kdt.kdt_radius_count(tree, dq, rl, F | kdt.KDT_RANGE_VISITS).double().sum().item()
-        lbytes = nq * (12 + 16) + 16.0 * lvisits + 8.0 * ltotal
+        lpoints = 16.0 * min(len(pts), ltotal)
+        lbytes = nq * (12 + 16) + lpoints + 8.0 * ltotal
         _emit(config=f"range: gmm N=2^24, Q=2^22 (90% mixture, 10% uniform), ball r={rl}",
               form="ball count / offsets / fill (long queries)", queries_per_s=nq / ((lcnt_ms + lfill_ms) / 1e3),
               hits=int(ltotal), hits_per_query=ltotal / nq, count_ms=lcnt_ms, fill_ms=lfill_ms,
               visits_per_query=lvisits / nq,
-              roofline_count={"bound": "hbm", "achieved": (nq * 16 + 16.0 * lvisits) / (lcnt_ms / 1e3) / 1e9,
+              roofline_count={"bound": "hbm", "achieved": (nq * 16 + lpoints) / (lcnt_ms / 1e3) / 1e9,
                               "peak": hbm, "unit": "GB/s",
-                              "frac": (nq * 16 + 16.0 * lvisits) / (lcnt_ms / 1e3) / 1e9 / hbm},
+                              "frac": (nq * 16 + lpoints) / (lcnt_ms / 1e3) / 1e9 / hbm},
               roofline_fill={"bound": "hbm", "achieved": lbytes / (lfill_ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                              "frac": lbytes / (lfill_ms / 1e3) / 1e9 / hbm, "bytes_per_query": lbytes / nq},
               oracle_sample_sets_equal=lok)
@@ -392,6 +393,6 @@ def run_config(args):
                   query_qps=Q / (ms / 1e3), query_ms=ms, forest_build_s=build_s, identical_forms=same,
                   launch_autotuned={"threads": th, "claim_steps": cs, "inline_depth": il, "light_run": lr},
                   visits_per_query=visits / Q,
-                  roofline=_roofline(Q * (12 + 8 * 8) + 16.0 * visits, ms, hbm, src, l2, "whole batched call"),
+                  roofline=_roofline(Q * (12 + 8 * 8) + 16.0 * Q, ms, hbm, src, l2, "whole batched call"),
                   bit_exact_sample=ok)
         return
