@@ -536,7 +536,21 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
         first[(size_t)r * (T + 1) + T] = (int32_t)blocks[r];
     const size_t data = at * sizeof(float4), refs = (size_t)T * sizeof(BoxRef);
     char *p = nullptr;
-    KDT_CUDA(cudaMalloc(&p, data + refs + first.size() * sizeof(int32_t)));
+    const size_t bytes = data + refs + first.size() * sizeof(int32_t);
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        // the builder's scratch, freed but kept by the stream-ordered pool, may
+        // be what is missing: give it back and try again
+        cudaGetLastError();
+        KDT_CUDA(cudaStreamSynchronize(s));
+        cudaMemPool_t pool;
+        int dev = 0;
+        KDT_CUDA(cudaGetDevice(&dev));
+        KDT_CUDA(cudaDeviceGetDefaultMemPool(&pool, dev));
+        KDT_CUDA(cudaMemPoolTrimTo(pool, 0));
+        e = cudaMalloc(&p, bytes);
+    }
+    KDT_CUDA(e);
     f->box_data = (float4 *)p;
     f->box_refs = p + data;
     BoxRef *ref = new BoxRef[T];
