@@ -383,8 +383,8 @@ int kdt_build_batched(const float *d_points, const int64_t *h_offsets, int T, in
 /* kNN of each query set against its own tree: queries of tree i are rows
  * [h_qoffsets[i], h_qoffsets[i+1]) of d_queries; result rows follow the query
  * rows; ids are indices within cloud i.  One persistent launch serves all
- * trees (captured once into a CUDA graph and replayed while the arguments are
- * unchanged).  With KDT_PER_TREE the same kernel is launched once per tree
+ * trees (captured into a CUDA graph when the same arguments come again, and replayed
+ * while they are unchanged).  With KDT_PER_TREE the same kernel is launched once per tree
  * instead (for comparison). */
 #define KDT_PER_TREE 0x10
 int kdt_knn_batched(kdt_forest *forest, const float *d_queries, const int64_t *h_qoffsets,
@@ -399,6 +399,8 @@ int kdt_forest_export(const kdt_forest *forest, float *d_coords, int32_t *d_ids,
  * warp (0 = the default for k, 32 for k = 1 and 64 otherwise; up to 256), the
  * inline depth (0 = default 2, or 1; see kdt_set_inline_depth) and the light
  * run (0 = default 1, up to 64; see kdt_set_light_run).
+ * They are choices of the unordered form; ordered queries walk the trees' box
+ * trees and take none of them.
  * Shared-memory staging does not apply to forests: the lanes of a warp walk
  * different trees.  The next kdt_knn_batched re-captures its graph. */
 int kdt_forest_set_launch(kdt_forest *forest, int threads, int claim_steps, int inline_depth, int light_run);
