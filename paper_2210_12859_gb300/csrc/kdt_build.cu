@@ -23,7 +23,7 @@
 // These passes run over arrays of N elements only for the levels whose subtrees
 // are larger than SUB_N points; then one block a subtree builds all the levels
 // that are left in shared memory (sub_kernel).  With them the build of 2^24
-// points is 12 passes over the lists instead of 24, and that of 20 k points 16
+// points is 12 passes over the lists instead of 24, and that of 20 k points 23
 // launches instead of 160.  T > 1 trees are built in the same passes: lists are
 // first sorted by (tree, coordinate, index) and every position knows its tree.
 #include <algorithm>
