@@ -1010,12 +1010,15 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         g = new ForestGraph();
         f->graph = g;
     }
-    const bool same = g->q == d_q && g->ids == d_ids && g->d2 == d_d2 && g->k == k && g->r2 == r2 &&
+    const bool same = g->scratch && g->q == d_q && g->ids == d_ids && g->d2 == d_d2 && g->k == k && g->r2 == r2 &&
                       g->flags == flags && g->threads == f->threads && g->claim_steps == f->claim_steps &&
                       g->inline_depth == f->inline_depth && g->light_run == f->light_run &&
                       g->qoff.size() == (size_t)T + 1 &&
                       std::equal(g->qoff.begin(), g->qoff.end(), h_qoff);
     if (!same) {
+        // the old arguments are forgotten before anything that they stand for
+        // goes: a call that fails below leaves nothing that looks in order
+        g->q = nullptr;
         if (g->exec) {
             cudaGraphExecDestroy(g->exec);
             g->exec = nullptr;
@@ -1026,10 +1029,11 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
             cudaFree(g->scratch);
             g->scratch = nullptr;
             g->scratch_bytes = 0;
+            if (debug_alloc_fails())
+                return set_error(KDT_ENOMEM, "device allocation failed (injected)");
             KDT_CUDA(cudaMalloc(&g->scratch, need));
             g->scratch_bytes = need;
         }
-        g->q = nullptr;  // set once the offsets are on their way
         g->ids = d_ids;
         g->d2 = d_d2;
         g->k = k;
