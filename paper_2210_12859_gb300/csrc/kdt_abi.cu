@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <new>
 #include <unordered_map>
 #include <vector>
 
@@ -811,7 +812,12 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
     f->f.T = T;
     f->f.D = D;
     f->f.total = h_off[T];
-    f->h_offsets = new int64_t[T + 1];
+    f->h_offsets = new (std::nothrow) int64_t[(size_t)T + 1];
+    f->h_first = new (std::nothrow) int32_t[(1 + BOX_LAUNCHES) * ((size_t)T + 1)];
+    if (!f->h_offsets || !f->h_first) {
+        kdt_forest_free(f);
+        return set_error(KDT_ENOMEM, "host allocation failed");
+    }
     memcpy(f->h_offsets, h_off, (T + 1) * sizeof(int64_t));
     int64_t total = std::max<int64_t>(h_off[T], 1);
     cudaError_t e = cudaMalloc(&f->nodes, (size_t)total * float4_per_node(D) * sizeof(float4));
@@ -829,7 +835,7 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
         e = cudaMemcpyAsync(f->f.d_offsets, h_off, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     int rc = e == cudaSuccess ? KDT_OK : cuda_error(e, "forest allocation", __FILE__, __LINE__);
     if (rc == KDT_OK)
-        rc = build_forest(d_points, h_off, T, D, f->nodes, f->ids, f->bbox, f->err, s);
+        rc = build_forest(d_points, h_off, T, D, f->nodes, f->ids, f->bbox, f->err, s, false, f->h_first);
     if (rc == KDT_OK)
         rc = build_box_forest(f, s);
     if (rc == KDT_OK) {
@@ -846,6 +852,8 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
         kdt_forest_free(f);
         return rc;
     }
+    delete[] f->h_first;  // the stream is past the build
+    f->h_first = nullptr;
     *out = f;
     return KDT_OK;
 }
@@ -1215,6 +1223,7 @@ void kdt_forest_free(kdt_forest *f)
     cudaFree(f->err);
     delete[] (BoxRef *)f->box_host;
     delete[] f->h_offsets;
+    delete[] f->h_first;
     delete f;
 }
 

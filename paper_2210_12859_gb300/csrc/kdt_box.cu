@@ -1,6 +1,6 @@
 // Build of the box tree and the kNN kernels that walk it (layout in kdt_box.cuh).
 #include <algorithm>
-#include <vector>
+#include <new>
 
 #include "kdt_box.cuh"
 
@@ -461,7 +461,6 @@ int64_t box_blocks(int64_t n, int up)
 // A block writes the boxes of five levels of the record tree (256 nodes and
 // their 64, 16, 4 and 1 ancestors), the next launch starts above them; `blocks`
 // and `first` (device, T > 1) of each launch, none after one without blocks.
-constexpr int BOX_LAUNCHES = 3;  // LB <= 26
 constexpr int BOX_LAUNCH_LEVELS = 10;
 
 template <int LAYOUT>
@@ -492,6 +491,8 @@ int build_boxes(int layout, const BoxBuild &a, const int64_t *blocks, const int3
 // float4s of a tree's records, rounded up to a 128-byte line, and of its groups
 size_t box_rec_size(int64_t n, int D) { return ((size_t)BoxShape(n).records() * 2 * box_coords(D) + 7) & ~(size_t)7; }
 size_t box_grp_size(int64_t n, int D) { return (size_t)BoxShape(n).groups() * 2 * (box_coords(D) + 1); }
+// of a forest's tree: the next one starts on a 128-byte line too
+size_t box_tree_size(int64_t n, int D) { return (box_rec_size(n, D) + box_grp_size(n, D) + 7) & ~(size_t)7; }
 
 }  // namespace
 
@@ -517,9 +518,12 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
 {
     const int T = f->f.T, D = f->f.D;
     // [records and groups of every tree][BoxRef of every tree][first blocks of every launch]
+    BoxRef *ref = new (std::nothrow) BoxRef[T];
+    if (!ref)
+        return set_error(KDT_ENOMEM, "host allocation failed");
+    f->box_host = ref;
+    int32_t *first = f->h_first + T + 1;  // behind the builder's
     size_t at = 0;
-    std::vector<size_t> rec(T), grp(T);
-    std::vector<int32_t> first((size_t)BOX_LAUNCHES * (T + 1), 0);
     int64_t blocks[BOX_LAUNCHES] = {0, 0, 0};
     for (int i = 0; i < T; ++i) {
         const int64_t n = f->h_offsets[i + 1] - f->h_offsets[i];
@@ -527,16 +531,14 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
             first[(size_t)r * (T + 1) + i] = (int32_t)blocks[r];
             blocks[r] += box_blocks(n, BOX_LAUNCH_LEVELS * r);
         }
-        rec[i] = at;
-        at += n ? box_rec_size(n, D) : 0;
-        grp[i] = at;
-        at += n ? (box_grp_size(n, D) + 7) & ~(size_t)7 : 0;
+        at += n ? box_tree_size(n, D) : 0;
     }
     for (int r = 0; r < BOX_LAUNCHES; ++r)
         first[(size_t)r * (T + 1) + T] = (int32_t)blocks[r];
+    const size_t first_bytes = (size_t)BOX_LAUNCHES * (T + 1) * sizeof(int32_t);
     const size_t data = at * sizeof(float4), refs = (size_t)T * sizeof(BoxRef);
     char *p = nullptr;
-    const size_t bytes = data + refs + first.size() * sizeof(int32_t);
+    const size_t bytes = data + refs + first_bytes;
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e == cudaErrorMemoryAllocation) {
         // the builder's scratch, freed but kept by the stream-ordered pool, may
@@ -553,19 +555,19 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
     KDT_CUDA(e);
     f->box_data = (float4 *)p;
     f->box_refs = p + data;
-    BoxRef *ref = new BoxRef[T];
-    f->box_host = ref;
+    at = 0;
     for (int i = 0; i < T; ++i) {
         const int64_t n = f->h_offsets[i + 1] - f->h_offsets[i];
-        ref[i] = n ? box_ref(n, f->box_data + rec[i], f->box_data + grp[i]) : BoxRef{nullptr, nullptr, 0, 0};
+        ref[i] = n ? box_ref(n, f->box_data + at, f->box_data + at + box_rec_size(n, D)) : BoxRef{nullptr, nullptr, 0, 0};
+        at += n ? box_tree_size(n, D) : 0;
     }
     KDT_CUDA(cudaMemcpyAsync(p + data, ref, refs, cudaMemcpyHostToDevice, s));
-    KDT_CUDA(cudaMemcpyAsync(p + data + refs, first.data(), first.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    KDT_CUDA(cudaMemcpyAsync(p + data + refs, first, first_bytes, cudaMemcpyHostToDevice, s));
     BoxBuild a = {f->nodes, f->ids, f->f.total, D, nullptr, nullptr, T, (const BoxRef *)f->box_refs, f->f.d_offsets,
                   nullptr};
     if (T == 1 && f->f.total) {
-        a.rec = f->box_data + rec[0];
-        a.grp = f->box_data + grp[0];
+        a.rec = const_cast<float4 *>(ref[0].rec);
+        a.grp = const_cast<float4 *>(ref[0].grp);
     }
     const int32_t *d_first[BOX_LAUNCHES];
     for (int r = 0; r < BOX_LAUNCHES; ++r)

@@ -43,6 +43,7 @@
 namespace kdt {
 
 constexpr int BOX_GROUP = 8;  // points per group
+constexpr int BOX_LAUNCHES = 3;  // launches of a box tree's build, for LB <= 26 (kdt_box.cu)
 
 template <int NC>
 struct BoxFormat {

@@ -27,7 +27,6 @@
 // launches instead of 160.  T > 1 trees are built in the same passes: lists are
 // first sorted by (tree, coordinate, index) and every position knows its tree.
 #include <algorithm>
-#include <vector>
 
 #include "kdt_internal.cuh"
 
@@ -910,7 +909,7 @@ struct DevBuf {
 }  // namespace
 
 int build_forest(const float *d_points, const int64_t *h_off, int T, int D, float4 *nodes, int32_t *ids, float *bbox,
-                 int *err, cudaStream_t s, bool widest)
+                 int *err, cudaStream_t s, bool widest, int32_t *h_jobs)
 {
     const int64_t total = h_off[T];
     if (total == 0)
@@ -918,7 +917,8 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
     // levels built by passes over the whole lists, and the blocks of sub_kernel
     const int sub_log2 = sub_log2_of(total);
     int levels = 0;
-    std::vector<int32_t> first_job(T + 1, 0);
+    int32_t one_tree[2];
+    int32_t *first_job = T > 1 ? h_jobs : one_tree;
     int64_t jobs = 0;
     for (int i = 0; i < T; ++i) {
         const int64_t n = h_off[i + 1] - h_off[i];
@@ -983,7 +983,7 @@ int build_forest(const float *d_points, const int64_t *h_off, int T, int D, floa
     const unsigned g = grid_for(total);
     if (T > 1) {
         KDT_CUDA(cudaMemcpyAsync(d_off, h_off, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        KDT_CUDA(cudaMemcpyAsync(d_job, first_job.data(), (T + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        KDT_CUDA(cudaMemcpyAsync(d_job, first_job, (T + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         KDT_LAUNCH tree_of_kernel<<<g, BT, 0, s>>>(d_off, T, total, tree_of);
     }
     int tbits = T > 1 ? floor_log2((uint64_t)(T - 1)) + 1 : 0;

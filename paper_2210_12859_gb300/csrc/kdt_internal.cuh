@@ -333,6 +333,10 @@ struct kdt_forest {
     void *box_host = nullptr;
     float *bbox = nullptr;         // [T][2][3]
     int64_t *h_offsets = nullptr;  // host copy [T+1]
+    // first blocks of every tree in the build's launches, [1 + BOX_LAUNCHES][T+1]:
+    // copied to the device by the build (a copy from pageable memory may still
+    // read it when the call that enqueued it has returned), given back after it
+    int32_t *h_first = nullptr;
     int *err = nullptr;
     void *graph = nullptr;         // cached graph of the batched query
     int threads = 0;               // block size of the batched kernel (0: default 128)
@@ -371,6 +375,9 @@ inline int64_t heap_scratch_threads() { return (int64_t)num_sms() * 1024; }
 // builder shared by kdt_build and kdt_build_batched: fills nodes / ids / bbox
 // widest: split dimension per node = widest extent of its points (T == 1,
 // D <= 3), stored in the node (layout 3); else level mod D
+// h_jobs: [T + 1] for T > 1, filled here and copied to the device; it has to
+// last until the stream has come past the build, as h_offsets has
 int build_forest(const float *d_points, const int64_t *h_offsets, int T, int D, float4 *nodes,
-                 int32_t *ids, float *bbox, int *err, cudaStream_t s, bool widest = false);
+                 int32_t *ids, float *bbox, int *err, cudaStream_t s, bool widest = false,
+                 int32_t *h_jobs = nullptr);
 }  // namespace kdt

@@ -67,3 +67,33 @@ def test_after_a_failed_growth_of_the_scratch(kdt, forest):
     assert e.value.code == kdt.KDT_ENOMEM
     assert same(run_small(), want_small)  # the very arguments of the first call
     assert same(kdt.kdt_knn_batched(forest, large, q_large, k, flags=flags), want_large)
+
+
+def test_many_small_clouds_built_behind_other_work(kdt):
+    """40000 clouds of 0 to 12 points and one large one, on a stream that is
+    still busy when the build enqueues its tables of first blocks (hundreds of
+    kilobytes, copied from the host): every tree and every row is right."""
+    import oracle
+
+    g = np.random.default_rng(23)
+    sizes = g.integers(0, 13, 40001)
+    sizes[20000] = 30011
+    off = offsets(*sizes)
+    pts = np.floor(g.random((off[-1], 3)) * 32).astype(np.float32)  # many ties
+    dp = cu(pts)
+    nq = g.integers(0, 4, len(sizes))
+    qoff = offsets(*nq)
+    dq = cu((g.random((qoff[-1], 3)) * 32).astype(np.float32))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(100_000_000)
+        forest = kdt.kdt_build_batched(dp, off)
+        ids = kdt.kdt_forest_export(forest)[1].cpu().numpy()
+        got = kdt.kdt_knn_batched(forest, dq, qoff, 4, flags=kdt.KDT_MORTON)
+        want = kdt.kdt_knn_batched(forest, dq, qoff, 4, flags=kdt.KDT_UNORDERED)
+        s.synchronize()
+    assert same(got, want)
+    for i in [20000, *g.choice(len(sizes), 400, replace=False)]:
+        if sizes[i]:
+            assert np.array_equal(ids[off[i]:off[i + 1]], oracle.build(pts[off[i]:off[i + 1]])), i
