@@ -420,8 +420,9 @@ int launch_box_one(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
     while (threads > 32 && a.Q < (int64_t)num_sms() * threads)
         threads >>= 1;
     const size_t smem = (size_t)threads * (4 * BoxWalk::MAX_RECORDS + (K > MAX_REG_K && !a.heap ? 8 * a.k : 0));
-    if (smem > 48 * 1024)
-        KDT_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static_assert(BOX_THREADS / 2 * (4 * BoxWalk::MAX_RECORDS + 8 * 64) <= 48 * 1024 &&
+                      BOX_THREADS * 4 * BoxWalk::MAX_RECORDS <= 48 * 1024,
+                  "the lists fit without a raised limit");
     int64_t grid = grid_for_kernel(fn, threads, smem);
     if (a.heap)
         grid = std::max<int64_t>(1, std::min<int64_t>(grid, a.heap_threads / threads));

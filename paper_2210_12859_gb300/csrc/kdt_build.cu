@@ -867,8 +867,10 @@ template <int SUB_LOG2>
 int launch_sub(const SubArgs &a, int64_t jobs, cudaStream_t s)
 {
     const size_t smem = sub_smem(a.D, SUB_LOG2);
+    // the limit is the kernel's, for all threads: the same value from every
+    // call, so that none lowers it between another's setting and its launch
     KDT_CUDA(cudaFuncSetAttribute((const void *)sub_kernel<SUB_LOG2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem));
+                                  (int)sub_smem(8, SUB_LOG2)));
     KDT_LAUNCH sub_kernel<SUB_LOG2><<<(unsigned)jobs, (1 << SUB_LOG2) / SUB_ITEMS, smem, s>>>(a);
     KDT_CUDA(cudaGetLastError());
     return KDT_OK;

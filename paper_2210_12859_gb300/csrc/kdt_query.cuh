@@ -9,6 +9,7 @@ namespace kdt {
 constexpr int REG_THREADS = 128;   // block size of the register-list kernels
 constexpr int SMEM_THREADS = 128;  // block size of the shared-memory-list kernels
 constexpr int MAX_REG_K = 16;
+constexpr int STAGE_BYTES = 160 * 1024;  // most that staged nodes may take of shared memory
 constexpr int STEPS_PER_CLAIM = 16; // traversal steps between two query claims of a warp
 
 struct QueryArgs {

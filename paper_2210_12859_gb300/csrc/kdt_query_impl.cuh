@@ -207,8 +207,12 @@ __global__ void __launch_bounds__(K <= MAX_REG_K ? REG_THREADS : SMEM_THREADS)
 template <typename Kern>
 inline int launch_kernel(Kern fn, int threads, size_t smem, const QueryArgs &a, cudaStream_t s)
 {
+    // the limit is the kernel's, for all threads: the same value from every
+    // call (the most that staging and the lists of k = 64 take together), so
+    // that none lowers it between another's setting and its launch
     if (smem > 48 * 1024)
-        KDT_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        KDT_CUDA(cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      STAGE_BYTES + 64 * SMEM_THREADS * 8));
     int grid = grid_for_kernel((const void *)fn, threads, smem);
     if (a.heap && (int64_t)grid * threads > a.heap_threads)
         grid = (int)std::max<int64_t>(1, a.heap_threads / threads);

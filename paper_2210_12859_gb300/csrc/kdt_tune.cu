@@ -179,7 +179,7 @@ int kdt_set_stage_levels(kdt_tree *t, int levels)
         return set_error(KDT_EINVAL, "tree is NULL");
     if (levels < -1 || levels > 16)
         return set_error(KDT_EINVAL, "levels must be in [-1, 16] (got %d)", levels);
-    if (!stage_fits(t, levels, 160 * 1024))
+    if (!stage_fits(t, levels, STAGE_BYTES))
         return set_error(KDT_EINVAL, "%d staged levels exceed the shared-memory budget", levels);
     t->stage_levels = levels;
     return KDT_OK;
