@@ -274,6 +274,18 @@ constexpr int box_blocks_per_sm(int layout, int k)
     return k <= 1 ? (layout == 1 ? 10 : (layout == 0 ? 8 : 6)) : (k <= 8 ? (layout == 0 ? 7 : 6) : (k <= 16 && layout == 0 ? 6 : 1));
 }
 
+// No distance to a NaN query passes a test, but every box's would: the maximum
+// that clamps its coordinates at 0 drops the NaN.  Such a query is not walked.
+template <int NC>
+__device__ __forceinline__ bool is_nan(const float (&q)[NC])
+{
+    bool nan = false;
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+        nan = nan || q[j] != q[j];
+    return nan;
+}
+
 // FOREST: a lane's query finds its tree by its place in the query offsets.
 template <int LAYOUT, int K, int MODE, bool FOREST>
 __global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box_knn_kernel(const QueryArgs a, const BoxArgs b)
@@ -328,7 +340,7 @@ __global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box
                         list.init(a.k, r2);
                         w.start(tree.leaf, s_far);
                         steps = 0;
-                        busy = true;
+                        busy = again = !is_nan(q);
                     } else if (gated && full && list.cull() > 0.f && r2 < __int_as_float(0x7f800000)) {
                         ratio += sqrt((double)r2 / (double)list.cull());
                     }
@@ -371,12 +383,7 @@ __global__ void __launch_bounds__(BOX_THREADS, box_blocks_per_sm(LAYOUT, K)) box
                     list.init(a.k, r2);
                     w.start(tree.leaf, s_far);
                     steps = 0;
-                    // no distance to a NaN query passes a test
-                    bool nan = false;
-#pragma unroll
-                    for (int j = 0; j < NC; ++j)
-                        nan = nan || q[j] != q[j];
-                    busy = !nan && (!FOREST || tree.leaf > 0);
+                    busy = !is_nan(q) && (!FOREST || tree.leaf > 0);
                 } else {
                     exhausted = true;
                 }

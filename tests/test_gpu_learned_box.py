@@ -1,0 +1,43 @@
+"""The learned radius on the box tree's walk: queries that are not numbers."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kdt():
+    from paper_2210_12859_gb300 import build
+
+    build.build_library()
+    from paper_2210_12859_gb300 import kdt as k
+
+    return k
+
+
+def test_nan_queries_are_not_walked(kdt):
+    """The network gives a NaN query a finite radius (its ReLUs drop the NaN),
+    so its empty list is looked at once more: without a walk, which the step
+    bound shows (no box is out of a NaN query's range: a walk would visit all
+    of the 2^15 points' buckets)."""
+    g = np.random.default_rng(8)
+    tree = kdt.kdt_build(torch.from_numpy(g.random((1 << 15, 3), dtype=np.float32)).cuda())
+    train = torch.from_numpy(g.random((1 << 13, 3), dtype=np.float32)).cuda()
+    kdt.kdt_radius_model_train(tree, train, 8, epochs=4, batch=1024, seed=2, gate=kdt.KDT_GATE_ALL)
+    qs = g.random((1000, 3), dtype=np.float32)
+    qs[::7, 0] = np.nan
+    qs[3::7] = np.nan
+    nan = np.isnan(qs).any(1)
+    dq = torch.from_numpy(qs).cuda()
+    want = kdt.kdt_knn(tree, dq, 8)
+    got = kdt.kdt_knn(tree, dq, 8, flags=kdt.KDT_LEARNED)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1].view(torch.int32), want[1].view(torch.int32))
+    assert bool((got[0][torch.from_numpy(nan).cuda()] == -1).all())
+    kdt.kdt_status(tree)
+    only = torch.from_numpy(qs[nan]).cuda()
+    kdt.kdt_debug_set_step_cap(tree, 1000)
+    got = kdt.kdt_knn(tree, only, 8, flags=kdt.KDT_LEARNED)
+    kdt.kdt_status(tree)
+    assert bool((got[0] == -1).all()) and bool(torch.isinf(got[1]).all())
+    assert kdt.kdt_learned_stats(tree)[0] == only.shape[0]
