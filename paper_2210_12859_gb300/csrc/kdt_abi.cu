@@ -782,6 +782,8 @@ struct ForestGraph {
     int64_t max_q = 0;         // most queries of one tree
     void *scratch = nullptr;   // persistent scratch referenced by the graph
     size_t scratch_bytes = 0;
+    bool shared = false;       // a caller's graph uses the scratch too
+    std::vector<void *> retired;  // scratch that a caller's graph may still use
     int threads = 0;           // launch parameters the graph was captured with
     int claim_steps = 0;
     int inline_depth = 0;
@@ -856,6 +858,19 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
     f->h_first = nullptr;
     *out = f;
     return KDT_OK;
+}
+
+// query offsets by value
+struct OffsetChunk {
+    static constexpr int MAX = 256;
+    int n;
+    int64_t v[MAX];
+};
+
+static __global__ void put_offsets_kernel(const OffsetChunk c, int64_t *__restrict__ out)
+{
+    if ((int)threadIdx.x < c.n)
+        out[threadIdx.x] = c.v[threadIdx.x];
 }
 
 static int forest_enqueue(kdt_forest *f, ForestGraph *g, const float *d_q, int64_t Q, const int64_t *d_qoff, int k,
@@ -1018,6 +1033,9 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         g = new ForestGraph();
         f->graph = g;
     }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    KDT_CUDA(cudaStreamIsCapturing(s, &cs));
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
     const bool same = g->scratch && g->q == d_q && g->ids == d_ids && g->d2 == d_d2 && g->k == k && g->r2 == r2 &&
                       g->flags == flags && g->threads == f->threads && g->claim_steps == f->claim_steps &&
                       g->inline_depth == f->inline_depth && g->light_run == f->light_run &&
@@ -1034,7 +1052,14 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         size_t need = carve_size({64, (size_t)(T + 1) * 8}) + ((flags & KDT_MORTON) ? morton_scratch_bytes(Q) : 0);
         if (need > g->scratch_bytes) {
             KDT_CUDA(cudaStreamSynchronize(s));
-            cudaFree(g->scratch);
+            if (g->shared) {
+                // a caller's graph writes there on every replay: kept to the
+                // forest's end, and each one at least twice as large
+                g->retired.push_back(g->scratch);
+                need = std::max(need, 2 * g->scratch_bytes);
+            } else {
+                cudaFree(g->scratch);
+            }
             g->scratch = nullptr;
             g->scratch_bytes = 0;
             if (debug_alloc_fails())
@@ -1055,22 +1080,32 @@ int kdt_knn_batched(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int 
         g->max_q = 1;
         for (int i = 0; i < T; ++i)
             g->max_q = std::max(g->max_q, h_qoff[i + 1] - h_qoff[i]);
+        g->q = d_q;
     }
     Carve c{(char *)g->scratch};
     c.take<unsigned long long>(8);
     int64_t *d_qoff = c.take<int64_t>(T + 1);
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    KDT_CUDA(cudaStreamIsCapturing(s, &cs));
-    if (!same) {
+    // The offsets in the scratch are taken as they are only by a replay of the
+    // forest's own graph, and not once a caller's graph holds a query of this
+    // forest: its replay puts its own offsets there.  A captured query carries
+    // them in its kernels' arguments, as it runs whenever the caller likes and
+    // the caller's array may be gone by then.
+    const bool replay = same && g->exec && !capturing && s != nullptr;
+    if (capturing) {
+        g->shared = true;
+        for (int i = 0; i <= T; i += OffsetChunk::MAX) {
+            OffsetChunk c;
+            c.n = std::min(OffsetChunk::MAX, T + 1 - i);
+            memcpy(c.v, h_qoff + i, c.n * sizeof(int64_t));
+            KDT_LAUNCH put_offsets_kernel<<<1, OffsetChunk::MAX, 0, s>>>(c, d_qoff + i);
+            KDT_CUDA(cudaGetLastError());
+        }
+    } else if (!replay || g->shared)
         KDT_CUDA(cudaMemcpyAsync(d_qoff, h_qoff, (T + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-        // a captured copy has not run: the next call makes its own
-        if (cs == cudaStreamCaptureStatusNone)
-            g->q = d_q;
-    }
     // arguments seen for the first time are enqueued as they are; a graph is
     // captured when they come again (capture and instantiation cost more than
     // the launches that one replay saves)
-    if (!same || cs != cudaStreamCaptureStatusNone || s == nullptr)
+    if (!same || capturing || s == nullptr)
         return forest_enqueue(f, g, d_q, Q, d_qoff, k, r2, flags, d_ids, d_d2, s);
     if (!g->exec) {
         cudaGraph_t graph = nullptr;
@@ -1213,6 +1248,8 @@ void kdt_forest_free(kdt_forest *f)
         if (g->exec)
             cudaGraphExecDestroy(g->exec);
         cudaFree(g->scratch);
+        for (void *p : g->retired)
+            cudaFree(p);
         delete g;
     }
     cudaFree(f->nodes);

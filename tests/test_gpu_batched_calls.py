@@ -97,3 +97,64 @@ def test_many_small_clouds_built_behind_other_work(kdt):
     for i in [20000, *g.choice(len(sizes), 400, replace=False)]:
         if sizes[i]:
             assert np.array_equal(ids[off[i]:off[i + 1]], oracle.build(pts[off[i]:off[i + 1]])), i
+
+
+def test_repeated_arguments_on_a_stream(kdt, forest):
+    """The same buffers again and again on a stream (enqueued, captured,
+    replayed), with new queries in them each time; other offsets in between."""
+    g = np.random.default_rng(4)
+    k, flags = 5, kdt.KDT_MORTON
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        dq = torch.empty((400, 3), device="cuda")
+        out_i, out_d = outputs(400, k)
+        for step in range(9):
+            dq.copy_(cu(g.random((400, 3), dtype=np.float32)))
+            qoff = offsets(100, 250, 50) if step not in (4, 7) else offsets(0, 390, 10)
+            got = kdt.kdt_knn_batched(forest, dq, qoff, k, flags=flags, out_ids=out_i, out_d2=out_d)
+            assert same(got, kdt.kdt_knn_batched(forest, dq, qoff, k, flags=kdt.KDT_PER_TREE)), step
+    s.synchronize()
+
+
+@pytest.mark.parametrize("before", ["none", "default stream", "stream"])
+def test_in_a_graph_of_the_caller(kdt, forest, before):
+    """A captured query keeps its own offsets: whether its arguments have run
+    before, whatever runs between its replays, also once the forest has needed
+    a larger scratch and the caller's offsets array is gone; and a replay
+    between repeated calls does not change theirs."""
+    g = np.random.default_rng(5)
+    k, flags = 5, kdt.KDT_MORTON
+    a, b = (cu(g.random((400, 3), dtype=np.float32)) for _ in range(2))
+    big = cu(g.random((40000, 3), dtype=np.float32))
+    qa, qb, qbig = [0, 100, 350, 400], [0, 0, 390, 400], [0, 40000, 40000, 40000]
+    want = [kdt.kdt_knn_batched(forest, x, o, k, flags=kdt.KDT_PER_TREE) for x, o in ((a, qa), (b, qb), (big, qbig))]
+    out_a, out_b = outputs(400, k), outputs(400, k)
+
+    def call(x, o, out):
+        return kdt.kdt_knn_batched(forest, x, o, k, flags=flags, out_ids=out[0], out_d2=out[1])
+
+    s = torch.cuda.Stream()
+    call(b, qb, out_b)  # the scratch is there
+    if before == "default stream":
+        call(a, qa, out_a)
+    torch.cuda.synchronize()
+    if before == "stream":
+        with torch.cuda.stream(s):
+            for _ in range(3):
+                call(a, qa, out_a)
+    s.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        call(a, list(qa), out_a)
+    with torch.cuda.stream(s):
+        for rep in range(4):
+            assert same(call(b, qb, out_b), want[1]), rep  # repeated: by the forest's own graph in the end
+            out_a[0].fill_(-7)
+            graph.replay()
+            assert same(out_a, want[0]), rep
+        assert same(call(b, qb, out_b), want[1])
+        assert same(kdt.kdt_knn_batched(forest, big, qbig, k, flags=flags), want[2])
+        out_a[0].fill_(-7)
+        graph.replay()
+        assert same(out_a, want[0])
+    s.synchronize()
