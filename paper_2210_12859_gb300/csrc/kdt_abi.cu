@@ -815,7 +815,7 @@ int kdt_build_batched(const float *d_points, const int64_t *h_off, int T, int D,
     f->f.D = D;
     f->f.total = h_off[T];
     f->h_offsets = new (std::nothrow) int64_t[(size_t)T + 1];
-    f->h_first = new (std::nothrow) int32_t[(1 + BOX_LAUNCHES) * ((size_t)T + 1)];
+    f->h_first = new (std::nothrow) int32_t[(SUB_CLASSES + BOX_LAUNCHES) * ((size_t)T + 1)];
     if (!f->h_offsets || !f->h_first) {
         kdt_forest_free(f);
         return set_error(KDT_ENOMEM, "host allocation failed");

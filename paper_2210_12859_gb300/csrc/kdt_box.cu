@@ -11,6 +11,7 @@ int grid_for_kernel(const void *fn, int threads, size_t smem);
 namespace {
 
 constexpr int BOX_BUILD_THREADS = 256;
+constexpr int BOX_TINY_THREADS = 32;  // blocks of a forest's trees of at most as many buckets
 constexpr int BOX_THREADS = 128;
 
 template <int NC>
@@ -49,10 +50,10 @@ __device__ __forceinline__ void put_box(float4 *rec, uint32_t v, const Box<NC> &
 // The block's boxes (thread i: node v0 + i of one level, `count` of them, a
 // power of two or a multiple of the block) into the records above, four
 // levels up the record tree as far as the block holds whole subtrees.
-template <int NC>
+template <int NC, int THREADS>
 __device__ __forceinline__ void reduce_boxes(float4 *rec, uint32_t v, int count, Box<NC> b)
 {
-    __shared__ float s_box[BOX_BUILD_THREADS][2 * NC + 1];
+    __shared__ float s_box[THREADS][2 * NC + 1];
     const int tid = threadIdx.x;
     for (;;) {
         if (tid < count && v > 1)
@@ -99,7 +100,8 @@ struct BoxBuild {
     int T;
     const BoxRef *trees;
     const int64_t *off;
-    const int32_t *first_block;
+    const int32_t *first_block;  // or, for whole_trees, the tree of every block
+    bool whole_trees;
 };
 
 // the block's tree in `a` (nodes, ids, N, rec, grp) and its number within the tree
@@ -109,6 +111,8 @@ __device__ __forceinline__ uint32_t box_build_tree(BoxBuild &a)
     if (a.T == 1)
         return blockIdx.x;
     int lo = 0, hi = a.T - 1;  // last tree that starts at or before the block
+    if (a.whole_trees)
+        lo = hi = a.first_block[blockIdx.x];
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (a.first_block[mid] <= (int)blockIdx.x)
@@ -122,11 +126,11 @@ __device__ __forceinline__ uint32_t box_build_tree(BoxBuild &a)
     a.ids = a.ids ? a.ids + base : nullptr;
     a.rec = const_cast<float4 *>(a.trees[lo].rec);
     a.grp = const_cast<float4 *>(a.trees[lo].grp);
-    return blockIdx.x - a.first_block[lo];
+    return a.whole_trees ? 0 : blockIdx.x - a.first_block[lo];
 }
 
-template <int LAYOUT>
-__global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(BoxBuild a)
+template <int LAYOUT, int THREADS>
+__global__ void __launch_bounds__(THREADS) box_leaf_kernel(BoxBuild a)
 {
     constexpr int NC = LayoutTraits<LAYOUT>::NC;
     const uint32_t block = box_build_tree<LAYOUT>(a);
@@ -135,8 +139,8 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(BoxBuild a)
     float4 *rec = a.rec, *grp = a.grp;
     const int N = (int)a.N, D = a.D;
     const BoxShape sh(N);
-    const uint32_t first = block * BOX_BUILD_THREADS, i = first + threadIdx.x;
-    const int count = (int)min((int64_t)BOX_BUILD_THREADS, sh.buckets - (int64_t)first);
+    const uint32_t first = block * THREADS, i = first + threadIdx.x;
+    const int count = (int)min((int64_t)THREADS, sh.buckets - (int64_t)first);
     Box<NC> box;
     box.none();
     if ((int64_t)i < sh.buckets) {
@@ -210,7 +214,7 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_leaf_kernel(BoxBuild a)
         }
     }
     if (sh.LB > 0)
-        reduce_boxes<NC>(rec, (uint32_t)sh.buckets + i, count, box);
+        reduce_boxes<NC, THREADS>(rec, (uint32_t)sh.buckets + i, count, box);
 }
 
 // Thread i: node i of the level `up` levels above the buckets, whose records
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(BOX_BUILD_THREADS) box_upper_kernel(BoxBuild a
             box.hi[j] = fmaxf(fmaxf(hi.x, hi.y), fmaxf(hi.z, hi.w));
         }
     }
-    reduce_boxes<NC>(rec, v0 + i, count, box);
+    reduce_boxes<NC, BOX_BUILD_THREADS>(rec, v0 + i, count, box);
 }
 
 // ---- kNN
@@ -457,27 +461,41 @@ int launch_box_k(const QueryArgs &a, const BoxArgs &b, cudaStream_t s)
     return launch_box_one<LAYOUT, 64, MODE, FOREST>(a, b, s);
 }
 
-// blocks of the launch `up` levels above the buckets of a tree of n points
-int64_t box_blocks(int64_t n, int up)
-{
-    const BoxShape sh(n);
-    if (n < 1 || sh.LB - up < (up ? 1 : 0))
-        return 0;
-    return (((int64_t)1 << (sh.LB - up)) + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS;
-}
-
 // A block writes the boxes of five levels of the record tree (256 nodes and
 // their 64, 16, 4 and 1 ancestors), the next launch starts above them; `blocks`
-// and `first` (device, T > 1) of each launch, none after one without blocks.
+// and `first` (device, T > 1) of each launch.  Launch BOX_TINY is for a forest's
+// trees of at most 32 buckets: a warp holds the whole of one (100 000 clouds of
+// 10 points: 587 us in blocks of 256 that search their tree, 57 in warps that are given it).
 constexpr int BOX_LAUNCH_LEVELS = 10;
+constexpr int BOX_TINY = BOX_LAUNCHES - 1;
+
+// adds the blocks of every launch for a tree of n points, one of a forest's or
+// the only one
+void add_box_blocks(int64_t n, bool forest, int64_t *blocks)
+{
+    const BoxShape sh(n);
+    if (n < 1)
+        return;
+    if (forest && sh.buckets <= BOX_TINY_THREADS) {
+        ++blocks[BOX_TINY];
+        return;
+    }
+    for (int r = 0, level = sh.LB; r == 0 || level >= 1; ++r, level -= BOX_LAUNCH_LEVELS)
+        blocks[r] += (((int64_t)1 << level) + BOX_BUILD_THREADS - 1) / BOX_BUILD_THREADS;
+}
 
 template <int LAYOUT>
 int build_box_layout(BoxBuild a, const int64_t *blocks, const int32_t *const *first, cudaStream_t s)
 {
-    for (int r = 0; r < BOX_LAUNCHES && blocks[r] > 0; ++r) {
+    for (int r = 0; r < BOX_LAUNCHES; ++r) {
+        if (blocks[r] == 0)
+            continue;
         a.first_block = first[r];
-        if (r == 0)
-            KDT_LAUNCH box_leaf_kernel<LAYOUT><<<(unsigned)blocks[r], BOX_BUILD_THREADS, 0, s>>>(a);
+        a.whole_trees = r == BOX_TINY;
+        if (r == BOX_TINY)
+            KDT_LAUNCH box_leaf_kernel<LAYOUT, BOX_TINY_THREADS><<<(unsigned)blocks[r], BOX_TINY_THREADS, 0, s>>>(a);
+        else if (r == 0)
+            KDT_LAUNCH box_leaf_kernel<LAYOUT, BOX_BUILD_THREADS><<<(unsigned)blocks[r], BOX_BUILD_THREADS, 0, s>>>(a);
         else
             KDT_LAUNCH box_upper_kernel<LAYOUT><<<(unsigned)blocks[r], BOX_BUILD_THREADS, 0, s>>>(
                 a, BOX_LAUNCH_LEVELS * r);
@@ -514,11 +532,10 @@ void box_tree_place(kdt_tree *t, void *p)
 
 int build_box_tree(const kdt_tree *t, cudaStream_t s)
 {
-    BoxBuild a = {t->nodes, t->ids, t->N, t->D, t->box_rec, t->box_grp, 1, nullptr, nullptr, nullptr};
-    int64_t blocks[BOX_LAUNCHES];
-    const int32_t *first[BOX_LAUNCHES] = {nullptr, nullptr, nullptr};
-    for (int r = 0; r < BOX_LAUNCHES; ++r)
-        blocks[r] = box_blocks(t->N, BOX_LAUNCH_LEVELS * r);
+    BoxBuild a = {t->nodes, t->ids, t->N, t->D, t->box_rec, t->box_grp, 1, nullptr, nullptr, nullptr, false};
+    int64_t blocks[BOX_LAUNCHES] = {};
+    const int32_t *first[BOX_LAUNCHES] = {};
+    add_box_blocks(t->N, false, blocks);
     return build_boxes(t->layout, a, blocks, first, s);
 }
 
@@ -530,18 +547,18 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
     if (!ref)
         return set_error(KDT_ENOMEM, "host allocation failed");
     f->box_host = ref;
-    int32_t *first = f->h_first + T + 1;  // behind the builder's
+    int32_t *first = f->h_first + (size_t)SUB_CLASSES * (T + 1);  // behind the builder's
     size_t at = 0;
-    int64_t blocks[BOX_LAUNCHES] = {0, 0, 0};
+    int64_t blocks[BOX_LAUNCHES] = {};
     for (int i = 0; i < T; ++i) {
         const int64_t n = f->h_offsets[i + 1] - f->h_offsets[i];
-        for (int r = 0; r < BOX_LAUNCHES; ++r) {
+        for (int r = 0; r < BOX_TINY; ++r)
             first[(size_t)r * (T + 1) + i] = (int32_t)blocks[r];
-            blocks[r] += box_blocks(n, BOX_LAUNCH_LEVELS * r);
-        }
+        first[(size_t)BOX_TINY * (T + 1) + blocks[BOX_TINY]] = i;  // stands if the tree is such a one
+        add_box_blocks(n, true, blocks);
         at += n ? box_tree_size(n, D) : 0;
     }
-    for (int r = 0; r < BOX_LAUNCHES; ++r)
+    for (int r = 0; r < BOX_TINY; ++r)
         first[(size_t)r * (T + 1) + T] = (int32_t)blocks[r];
     const size_t first_bytes = (size_t)BOX_LAUNCHES * (T + 1) * sizeof(int32_t);
     const size_t data = at * sizeof(float4), refs = (size_t)T * sizeof(BoxRef);
@@ -570,16 +587,20 @@ int build_box_forest(kdt_forest *f, cudaStream_t s)
         at += n ? box_tree_size(n, D) : 0;
     }
     KDT_CUDA(cudaMemcpyAsync(p + data, ref, refs, cudaMemcpyHostToDevice, s));
-    KDT_CUDA(cudaMemcpyAsync(p + data + refs, first, first_bytes, cudaMemcpyHostToDevice, s));
     BoxBuild a = {f->nodes, f->ids, f->f.total, D, nullptr, nullptr, T, (const BoxRef *)f->box_refs, f->f.d_offsets,
-                  nullptr};
+                  nullptr, false};
     if (T == 1 && f->f.total) {
         a.rec = const_cast<float4 *>(ref[0].rec);
         a.grp = const_cast<float4 *>(ref[0].grp);
     }
-    const int32_t *d_first[BOX_LAUNCHES];
-    for (int r = 0; r < BOX_LAUNCHES; ++r)
-        d_first[r] = (const int32_t *)(p + data + refs) + (size_t)r * (T + 1);
+    int32_t *d_first[BOX_LAUNCHES];
+    for (int r = 0; r < BOX_LAUNCHES; ++r) {
+        d_first[r] = (int32_t *)(p + data + refs) + (size_t)r * (T + 1);
+        if (blocks[r])
+            KDT_CUDA(cudaMemcpyAsync(d_first[r], first + (size_t)r * (T + 1),
+                                     (r == BOX_TINY ? blocks[r] : T + 1) * sizeof(int32_t), cudaMemcpyHostToDevice,
+                                     s));
+    }
     return build_boxes(layout_of(D), a, blocks, d_first, s);
 }
 

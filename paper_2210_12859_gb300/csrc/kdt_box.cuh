@@ -43,7 +43,7 @@
 namespace kdt {
 
 constexpr int BOX_GROUP = 8;  // points per group
-constexpr int BOX_LAUNCHES = 3;  // launches of a box tree's build, for LB <= 26 (kdt_box.cu)
+constexpr int BOX_LAUNCHES = 4;  // launches of a box tree's build: three for LB <= 26, one for small trees (kdt_box.cu)
 
 template <int NC>
 struct BoxFormat {

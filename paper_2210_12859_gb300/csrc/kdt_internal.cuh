@@ -333,7 +333,7 @@ struct kdt_forest {
     void *box_host = nullptr;
     float *bbox = nullptr;         // [T][2][3]
     int64_t *h_offsets = nullptr;  // host copy [T+1]
-    // first blocks of every tree in the build's launches, [1 + BOX_LAUNCHES][T+1]:
+    // first blocks of every tree in the build's launches, [SUB_CLASSES + BOX_LAUNCHES][T+1]:
     // copied to the device by the build (a copy from pageable memory may still
     // read it when the call that enqueued it has returned), given back after it
     int32_t *h_first = nullptr;
@@ -372,10 +372,11 @@ bool heap_in_global(const kdt_tree *t, int k, bool box);
 int list_group_for(const kdt_tree *t, int k);
 // per-thread heap scratch for the traversal kernels (threads x k keys)
 inline int64_t heap_scratch_threads() { return (int64_t)num_sms() * 1024; }
+constexpr int SUB_CLASSES = 3;  // launches of the builder's last step, by the size of the trees (kdt_build.cu)
 // builder shared by kdt_build and kdt_build_batched: fills nodes / ids / bbox
 // widest: split dimension per node = widest extent of its points (T == 1,
 // D <= 3), stored in the node (layout 3); else level mod D
-// h_jobs: [T + 1] for T > 1, filled here and copied to the device; it has to
+// h_jobs: [SUB_CLASSES][T + 1] for T > 1, filled here and copied to the device; it has to
 // last until the stream has come past the build, as h_offsets has
 int build_forest(const float *d_points, const int64_t *h_offsets, int T, int D, float4 *nodes,
                  int32_t *ids, float *bbox, int *err, cudaStream_t s, bool widest = false,

@@ -158,3 +158,26 @@ def test_in_a_graph_of_the_caller(kdt, forest, before):
         graph.replay()
         assert same(out_a, want[0])
     s.synchronize()
+
+
+@pytest.mark.parametrize("D", [1, 3, 4, 6])
+def test_classes_of_tree_sizes(kdt, D):
+    """Trees on both sides of the builder's classes (128, 1024 and 4096 points)
+    and of the box build's (32 buckets), in one forest of more than 2^18 points."""
+    import oracle
+
+    g = np.random.default_rng(40 + D)
+    sizes = [0, 1, 8, 127, 128, 129, 0, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 4096, 4097, 3, 270000, 64, 0]
+    sizes += list(g.integers(100, 160, 50))
+    off = offsets(*sizes)
+    pts = np.floor(g.random((off[-1], D)) * 200).astype(np.float32)
+    forest = kdt.kdt_build_batched(cu(pts), off)
+    ids = kdt.kdt_forest_export(forest)[1].cpu().numpy()
+    for i, n in enumerate(sizes):
+        if n:
+            assert np.array_equal(ids[off[i]:off[i + 1]], oracle.build(pts[off[i]:off[i + 1]])), i
+    qoff = offsets(*g.integers(0, 60, len(sizes)))
+    dq = cu((g.random((qoff[-1], D)) * 200).astype(np.float32))
+    for k in (1, 9):
+        want = kdt.kdt_knn_batched(forest, dq, qoff, k, flags=kdt.KDT_UNORDERED)
+        assert same(kdt.kdt_knn_batched(forest, dq, qoff, k), want)
