@@ -82,12 +82,17 @@ bool debug_alloc_fails()
 // share the nodes of their walks for as many levels as the order resolves,
 // whatever the points' density and dimensions: a Morton code cuts the space on
 // planes of its own and sees three coordinates.  One dependent 4-byte load a
-// level, the upper levels from L1.
+// level, the upper levels from L1.  The query is read once, into registers: it
+// may lie in page-locked host memory (kdt_knn_host), where a load a level through
+// the link cost 1.1 of 9.8 ms (2^20 points, 2^22 queries, k = 8; 4-D 1.2 of 9.4).
 // LAYOUT as in kdt_internal.cuh; nodes, n: the tree's.
 template <int LAYOUT>
-__device__ __forceinline__ uint32_t descent_path(const float *__restrict__ q, int D, const float4 *__restrict__ nodes,
-                                                 int64_t n, int levels)
+__device__ __forceinline__ uint32_t descent_path(const float *__restrict__ qs, int64_t i, int D,
+                                                 const float4 *__restrict__ nodes, int64_t n, int levels)
 {
+    constexpr int NC = LayoutTraits<LAYOUT>::NC;
+    float q[NC];
+    load_query<LAYOUT>(qs, i, D, q);
     constexpr int STRIDE = LAYOUT == 2 ? 8 : 4;
     const float *c = reinterpret_cast<const float *>(nodes);
     const int full = min(levels, floor_log2((uint64_t)n));  // the levels above the last are full
@@ -97,7 +102,7 @@ __device__ __forceinline__ uint32_t descent_path(const float *__restrict__ q, in
         const size_t at = (size_t)(v - 1) * STRIDE;
         if (LAYOUT == 3)
             dim = (int)(__float_as_uint(__ldg(c + at + 3)) >> NODE_DIM_SHIFT);
-        const bool right = __ldg(q + dim) > __ldg(c + at + dim);
+        const bool right = select_dim<NC>(q, dim) > __ldg(c + at + dim);
         v = 2 * v + right;
         if (LAYOUT != 3)
             dim = dim + 1 == D ? 0 : dim + 1;
@@ -110,7 +115,7 @@ __global__ void path_kernel(const float *__restrict__ qs, int64_t Q, int D, cons
                             int64_t n, int levels, uint32_t *__restrict__ keys)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x)
-        keys[i] = descent_path<LAYOUT>(qs + i * D, D, nodes, n, levels);
+        keys[i] = descent_path<LAYOUT>(qs, i, D, nodes, n, levels);
 }
 
 // Forests: the tree's index above the path in its tree, so that one sort
@@ -131,7 +136,7 @@ __global__ void forest_path_kernel(const float *__restrict__ qs, int64_t Q, int 
         }
         const int64_t base = node_off[lo], n = node_off[lo + 1] - base;
         const uint32_t path =
-            n > 0 ? descent_path<LAYOUT>(qs + i * D, D, nodes + base * LayoutTraits<LAYOUT>::NF, n, levels) : 0u;
+            n > 0 ? descent_path<LAYOUT>(qs, i, D, nodes + base * LayoutTraits<LAYOUT>::NF, n, levels) : 0u;
         keys[i] = ((uint32_t)lo << levels) | path;
     }
 }
