@@ -292,9 +292,12 @@ typedef struct kdt_train_opts {
                              probabilities; the margin's fallback target is then a share of
                              that work.  1: every query weighs the same */
     int gate;             /* KDT_GATE_* (default KDT_GATE_AUTO: on up to 2^20 of the training
-                             queries, with query_flags, the processed nodes of the plain traversal
-                             and of the learned forms (all queries gated, the far ones) are counted,
-                             and the network pass's cost per gated query is measured in
+                             queries, with query_flags.  Ordered queries: the whole call is timed
+                             with every gate, on these queries and on up to 2^22 copies of them,
+                             and a learned form is kept when it is at least 3 % faster than the
+                             plain one both times, else KDT_GATE_NONE.  Unordered queries: the
+                             processed nodes of the plain traversal and of the learned forms are
+                             counted, and the network pass's cost per gated query is measured in
                              processed-node equivalents (its time per query over the plain
                              traversal's time per processed node); a gated call's nodes are
                              charged 1.08 plain nodes each (the bounded pass's measured

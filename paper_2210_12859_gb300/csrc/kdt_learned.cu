@@ -381,18 +381,95 @@ int run_learned_query(kdt_tree *t, const float *d_q, int64_t Q, int k, float r2,
     return launch_query(t->layout, a, ordered, MODE_BOUNDED, false, s);
 }
 
-// The automatic gate, from the training queries: the processed nodes the
-// plain traversal needs and those the learned forms need (all queries gated,
-// or the far ones), counted exactly, and the cost of the network pass (the
-// descent for the features, the MLP) per gated query in processed-node
-// equivalents: its time per query over the plain traversal's time per
-// processed node.  A form's score is the nodes it saves minus that cost times
-// the queries it gates; the best positive score wins, else no query is gated.
-// (Timing the whole forms on the training set does not transfer: at 2^20
+// The automatic gate of ordered queries, which walk the box tree: the three
+// forms of the whole call are timed on the training queries, once as they are
+// and once many times over, and a learned form is kept when it is faster than
+// the plain one by GATE_MARGIN both times.  (A short call ends with its longest
+// walks alone, which a proposal shortens; a long one is bound by all walks, and
+// by the network.  By the training queries alone the far gate was kept for 2^22
+// clustered points, k = 4, where a full call takes 15 % longer with it.  By both
+// times none of 48 workloads (clustered, surface and uniform points, k = 1 to 64,
+// 2^18 training queries against calls of 2^18 to 2^22) kept a slower form; 7 kept
+// one that is 3 to 6 % faster.  The processed nodes that a proposal saves say
+// little here: on clustered data they are the state machine's walks between the
+// clusters, of which the box walk has hardly any.)
+constexpr float GATE_MARGIN = 0.03f;
+constexpr int64_t GATE_QUERIES = (int64_t)1 << 22, GATE_RESULTS = (int64_t)1 << 26;  // of the long call, at most
+int choose_gate_timed(kdt_tree *t, const float *d_q, int64_t n, int k, int qflags, cudaStream_t s)
+{
+    int64_t copies = std::max<int64_t>(1, std::min(GATE_QUERIES, GATE_RESULTS / k) / n);
+    Dev buf(s);
+    const size_t row = (size_t)n * t->D * 4;
+    size_t q_b, out_b;
+    for (;;) {
+        q_b = (copies * row + 255) & ~(size_t)255;
+        out_b = ((size_t)copies * n * k * 4 + 255) & ~(size_t)255;
+        const cudaError_t e = cudaMallocAsync(&buf.p, q_b + 2 * out_b, s);
+        if (e != cudaErrorMemoryAllocation || copies == 1) {
+            KDT_CUDA(e);
+            break;
+        }
+        cudaGetLastError();
+        copies = 1;  // the queries as they are, then
+    }
+    char *B = (char *)buf.p;
+    int32_t *ids = (int32_t *)(B + q_b);
+    float *d2 = (float *)(B + q_b + out_b);
+    for (int64_t c = 0; c < copies; ++c)
+        KDT_CUDA(cudaMemcpyAsync(B + c * row, d_q, row, cudaMemcpyDeviceToDevice, s));
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    int rc = KDT_OK;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
+        rc = set_error(KDT_ECUDA, "event create");
+    const int forms[3] = {KDT_GATE_NONE, KDT_GATE_ALL, KDT_GATE_FAR};
+    float worst[3] = {0.f, 0.f, 0.f};  // of the two times, each over the plain form's
+    for (int64_t q : {n, copies * n}) {
+        float best[3] = {3.4e38f, 3.4e38f, 3.4e38f};
+        // in turn, so that a change of clocks meets all of them
+        for (int rep = 0; rep < 6; ++rep)
+            for (int f = 0; f < 3 && rc == KDT_OK; ++f) {
+                float ms = 0.f;
+                t->model.gate = forms[f];
+                if (cudaEventRecord(e0, s) != cudaSuccess)
+                    rc = set_error(KDT_ECUDA, "event record");
+                if (rc == KDT_OK)
+                    rc = run_learned_query(t, (const float *)B, q, k, INFINITY, qflags, ids, d2, nullptr, s);
+                if (rc == KDT_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                                     cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+                    rc = set_error(KDT_ECUDA, "event timing failed");
+                if (rep > 0)
+                    best[f] = std::min(best[f], ms);
+            }
+        for (int f = 0; f < 3; ++f)
+            worst[f] = std::max(worst[f], best[f] / best[0]);
+    }
+    if (e0)
+        cudaEventDestroy(e0);
+    if (e1)
+        cudaEventDestroy(e1);
+    t->model.gate = KDT_GATE_NONE;
+    if (rc != KDT_OK)
+        return rc;
+    const int f = worst[1] < worst[2] ? 1 : 2;
+    if (worst[f] < 1.f - GATE_MARGIN)
+        t->model.gate = forms[f];
+    return KDT_OK;
+}
+
+// The automatic gate of unordered queries, which run on the state machine: the
+// processed nodes the plain traversal needs and those the learned forms need
+// (all queries gated, or the far ones), counted exactly, and the cost of the
+// network pass (the descent for the features, the MLP) per gated query in
+// processed-node equivalents: its time per query over the plain traversal's
+// time per processed node.  A form's score is the nodes it saves minus that
+// cost times the queries it gates; the best positive score wins, else no query
+// is gated.  (Timing these forms on the training set does not transfer: at 2^20
 // queries the traversal's launch tail weighs differently than at full size.)
 int choose_gate(kdt_tree *t, const float *d_q, int64_t n, int k, int qflags, cudaStream_t s)
 {
     qflags &= ~(KDT_LEARNED | KDT_PLAIN_STEP | KDT_CLOSE_FIRST | KDT_STACK);
+    if (!(qflags & KDT_UNORDERED))
+        return choose_gate_timed(t, d_q, n, k, qflags, s);
     Dev buf(s);
     const size_t vis_b = ((size_t)n * 4 + 255) & ~(size_t)255;
     const size_t out_b = ((size_t)n * k * 4 + 255) & ~(size_t)255;

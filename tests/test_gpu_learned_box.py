@@ -41,3 +41,39 @@ def test_nan_queries_are_not_walked(kdt):
     kdt.kdt_status(tree)
     assert bool((got[0] == -1).all()) and bool(torch.isinf(got[1]).all())
     assert kdt.kdt_learned_stats(tree)[0] == only.shape[0]
+
+
+@pytest.mark.parametrize("k", [4, 8])
+def test_automatic_gate_is_not_slower(kdt, k):
+    """The gate that training keeps for ordered queries: on clustered points
+    with far queries the learned call takes no longer than the plain one, but
+    for the 3 % by which the choice has to be clear and 1 % of noise (medians
+    of runs in turn).  Judged by the state machine's nodes it took 12 % (k = 4)
+    and 7 % longer."""
+    g = torch.Generator(device="cuda").manual_seed(32)
+
+    def sample(n, centres):
+        at = torch.randint(0, 64, (n,), generator=g, device="cuda")
+        return centres[at] + 0.01 * torch.randn((n, 3), generator=g, device="cuda")
+
+    n = 1 << 22
+    centres = torch.rand((64, 3), generator=g, device="cuda")
+    tree = kdt.kdt_build(sample(n, centres))
+    qs = sample(n, centres)
+    far = torch.rand((n, 1), generator=g, device="cuda") < 0.1
+    qs = torch.where(far, torch.rand((n, 3), generator=g, device="cuda"), qs)
+    flags = kdt.KDT_MORTON | kdt.KDT_COST_ORDER
+    kdt.kdt_radius_model_train(tree, qs[: 1 << 18].contiguous(), k, epochs=20, seed=1)
+    out = torch.empty((n, k), dtype=torch.int32, device="cuda"), torch.empty((n, k), device="cuda")
+    ms = {0: [], kdt.KDT_LEARNED: []}
+    for rep in range(13):
+        for f in ms:
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            kdt.kdt_knn(tree, qs, k, flags=flags | f, out_ids=out[0], out_d2=out[1])
+            b.record()
+            b.synchronize()
+            if rep > 1:
+                ms[f].append(a.elapsed_time(b))
+    plain, learned = (float(np.median(ms[f])) for f in (0, kdt.KDT_LEARNED))
+    assert learned < 1.04 * plain, (learned, plain, kdt.kdt_radius_model_gate(tree))
