@@ -386,8 +386,11 @@ int kdt_build_batched(const float *d_points, const int64_t *h_offsets, int T, in
 /* kNN of each query set against its own tree: queries of tree i are rows
  * [h_qoffsets[i], h_qoffsets[i+1]) of d_queries; result rows follow the query
  * rows; ids are indices within cloud i.  One persistent launch serves all
- * trees (captured into a CUDA graph when the same arguments come again, and replayed
- * while they are unchanged).  With KDT_PER_TREE the same kernel is launched once per tree
+ * trees (on a stream other than the default one captured into a CUDA graph when the
+ * same arguments come a second time, and replayed from the third on while they are
+ * unchanged).  In a capture of the caller's the call takes its offsets by value, so
+ * that h_qoffsets need not outlive it; the first call of a forest, and one that needs
+ * more scratch than those before, allocates and cannot be captured.  With KDT_PER_TREE the same kernel is launched once per tree
  * instead (for comparison). */
 #define KDT_PER_TREE 0x10
 int kdt_knn_batched(kdt_forest *forest, const float *d_queries, const int64_t *h_qoffsets,
@@ -405,7 +408,7 @@ int kdt_forest_export(const kdt_forest *forest, float *d_coords, int32_t *d_ids,
  * They are choices of the unordered form; ordered queries walk the trees' box
  * trees and take none of them.
  * Shared-memory staging does not apply to forests: the lanes of a warp walk
- * different trees.  The next kdt_knn_batched re-captures its graph. */
+ * different trees.  A graph that earlier calls captured is not replayed any more. */
 int kdt_forest_set_launch(kdt_forest *forest, int threads, int claim_steps, int inline_depth, int light_run);
 
 /* Processed nodes (first visits) of every query of a kdt_knn_batched call
@@ -416,12 +419,14 @@ int kdt_forest_set_launch(kdt_forest *forest, int threads, int claim_steps, int 
 int kdt_knn_batched_visits(kdt_forest *forest, const float *d_queries, const int64_t *h_query_offsets, int k,
                            float max_radius, int flags, int32_t *d_visits, void *stream);
 
-/* Time the batched query (kdt_knn_batched with these arguments, graph
- * included; it writes d_ids / d_d2 like that call) for inline depths {2, 1},
- * light runs {1, 4, 8}, block sizes {128, 64}, then claim steps {16, 32, 64,
- * 128}, one warm-up and
- * one timed run each, and keep the fastest on the forest (a candidate must win
- * by 2 %).  Synchronous.  The out pointers may be NULL. */
+/* Time the batched query (kdt_knn_batched with these arguments, as it runs
+ * when they repeat: a graph's replay on a stream of the caller's; it writes
+ * d_ids / d_d2 like that call).  Unordered: for inline depths {2, 1}, light runs
+ * {1, 4, 8}, block sizes {128, 64}, then claim steps {16, 32, 64, 128}, two
+ * warm-ups and one timed run each; the fastest is kept on the forest (a
+ * candidate must win by 2 %).  Ordered queries take none of these parameters:
+ * the query is timed, and the forest's parameters are reported and stay.
+ * Synchronous.  The out pointers may be NULL. */
 int kdt_forest_autotune(kdt_forest *forest, const float *d_queries, const int64_t *h_query_offsets, int k,
                         float max_radius, int flags, int32_t *d_ids, float *d_d2, int *best_threads,
                         int *best_claim, int *best_inline, int *best_light, float *best_ms, void *stream);

@@ -1150,11 +1150,12 @@ int kdt_forest_set_launch(kdt_forest *f, int threads, int claim_steps, int inlin
     return KDT_OK;
 }
 
-// Coordinate search over the batched launch: inline depth {2, 1}, light run
-// {1, 4, 8}, block size {128, 64}, then claim steps {16, 32, 64, 128}; each
-// candidate is the whole
-// batched query (graph included), one warm-up and one timed run, and is taken
-// when it is faster than the best so far by 2 %.
+// Unordered queries: coordinate search over the batched launch: inline depth
+// {2, 1}, light run {1, 4, 8}, block size {128, 64}, then claim steps {16, 32, 64,
+// 128}; each candidate is the whole batched query, two warm-up runs (the second
+// captures the graph) and one timed run (its replay), and is taken when it is
+// faster than the best so far by 2 %.  Ordered queries walk the box trees, which
+// take none of these: the query is timed and the launch parameters stay.
 int kdt_forest_autotune(kdt_forest *f, const float *d_q, const int64_t *h_qoff, int k, float max_radius, int flags,
                         int32_t *d_ids, float *d_d2, int *best_threads, int *best_claim, int *best_inline,
                         int *best_light, float *best_ms, void *stream)
@@ -1177,7 +1178,8 @@ int kdt_forest_autotune(kdt_forest *f, const float *d_q, const int64_t *h_qoff, 
         f->claim_steps = cs;
         f->inline_depth = inl;
         f->light_run = lr;
-        rc = kdt_knn_batched(f, d_q, h_qoff, k, max_radius, flags, d_ids, d_d2, stream);
+        for (int warm = 0; warm < 2 && rc == KDT_OK; ++warm)
+            rc = kdt_knn_batched(f, d_q, h_qoff, k, max_radius, flags, d_ids, d_d2, stream);
         float ms = 0.f;
         if (rc == KDT_OK && cudaEventRecord(e0, s) != cudaSuccess)
             rc = set_error(KDT_ECUDA, "event record");
@@ -1194,17 +1196,21 @@ int kdt_forest_autotune(kdt_forest *f, const float *d_q, const int64_t *h_qoff, 
             bl = lr;
         }
     };
-    trial(0, 0, 2, 1);
-    trial(0, 0, 1, 1);
-    const int i_best = bi;
-    trial(0, 0, i_best, 4);
-    trial(0, 0, i_best, 8);
-    const int l_best = bl;
-    trial(64, 0, i_best, l_best);
-    const int t_best = bt;
-    for (int cs : {16, 32, 64, 128})
-        if (cs != default_claim_steps_k(k))
-            trial(t_best, cs, i_best, l_best);
+    if (!(flags & KDT_UNORDERED)) {
+        trial(saved_t, saved_c, saved_i, saved_l);
+    } else {
+        trial(0, 0, 2, 1);
+        trial(0, 0, 1, 1);
+        const int i_best = bi;
+        trial(0, 0, i_best, 4);
+        trial(0, 0, i_best, 8);
+        const int l_best = bl;
+        trial(64, 0, i_best, l_best);
+        const int t_best = bt;
+        for (int cs : {16, 32, 64, 128})
+            if (cs != default_claim_steps_k(k))
+                trial(t_best, cs, i_best, l_best);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != KDT_OK) {
@@ -1219,9 +1225,9 @@ int kdt_forest_autotune(kdt_forest *f, const float *d_q, const int64_t *h_qoff, 
     f->inline_depth = bi;
     f->light_run = bl;
     if (best_inline)
-        *best_inline = bi;
+        *best_inline = bi ? bi : 2;
     if (best_light)
-        *best_light = bl;
+        *best_light = bl ? bl : 1;
     if (best_threads)
         *best_threads = bt ? bt : REG_THREADS;
     if (best_claim)

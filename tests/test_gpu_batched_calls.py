@@ -181,3 +181,33 @@ def test_classes_of_tree_sizes(kdt, D):
     for k in (1, 9):
         want = kdt.kdt_knn_batched(forest, dq, qoff, k, flags=kdt.KDT_UNORDERED)
         assert same(kdt.kdt_knn_batched(forest, dq, qoff, k), want)
+
+
+def test_autotune(kdt):
+    """Ordered queries take no launch parameter: they are timed and the
+    forest's parameters stay.  Unordered ones are timed as they run when their
+    arguments repeat, without the capture of the graph: on a tiny forest, where
+    that would be most of the time, the reported time is within the time that a
+    replay takes with the binding's own overhead, measured here."""
+    g = np.random.default_rng(6)
+    f = kdt.kdt_build_batched(cu(g.random((400, 3), dtype=np.float32)), offsets(100, 100, 100, 100))
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        dq = cu(g.random((64, 3), dtype=np.float32))
+        qoff, out = offsets(16, 16, 16, 16), outputs(64, 8)
+        kdt.kdt_forest_set_launch(f, 32, 17, 1, 5)
+        assert kdt.kdt_forest_autotune(f, dq, qoff, 8, flags=kdt.KDT_MORTON)[:4] == (32, 17, 1, 5)
+        kdt.kdt_forest_set_launch(f, 0, 0)
+        flags = kdt.KDT_MORTON | kdt.KDT_UNORDERED
+        reported = min(kdt.kdt_forest_autotune(f, dq, qoff, 8, flags=flags)[4] for _ in range(3))
+        ms = []
+        for _ in range(23):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            kdt.kdt_knn_batched(f, dq, qoff, 8, flags=flags, out_ids=out[0], out_d2=out[1])
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        assert reported <= np.median(ms[3:]), (reported, ms)
+        kdt.kdt_forest_set_launch(f, 0, 0)
