@@ -495,14 +495,15 @@ int kdt_set_light_run(kdt_tree *tree, int steps);
 #define KDT_LIST_GROUP4 2
 #define KDT_LIST_GROUP8 3
 int kdt_set_large_k_list(kdt_tree *tree, int placement);
-/* The placement kdt_knn uses for this tree and k: set on the tree, else tuned
- * for its shape (for k > 16 kdt_autotune takes the global heap when its query
- * sample processes at least 1024 nodes per query, the shared-memory heap
- * otherwise), else KDT_LIST_SHARED. */
+/* The placement that ordered kdt_knn queries use for this tree and k: set on
+ * the tree, else KDT_LIST_SHARED.  Unordered queries and counts of processed
+ * nodes take the one set on the tree, else the one tuned for its shape (for k >
+ * 16 kdt_autotune takes the global heap when its query sample processes at least
+ * 1024 nodes per query, the shared-memory heap otherwise), else KDT_LIST_SHARED. */
 int kdt_large_k_list(const kdt_tree *tree, int k, int *placement);
 
-/* The launch parameters kdt_knn uses for this tree and k: set on the tree,
- * else tuned for its shape (kdt_autotune / kdt_tuning_load), else defaults
+/* The launch parameters of the state machine's kernels for this tree and k (kdt_knn
+ * with KDT_UNORDERED, kdt_knn_visits): set on the tree, else tuned for its shape (kdt_autotune / kdt_tuning_load), else defaults
  * (no staging, 32 claim steps for k = 1 and 64 otherwise, inline depth 2,
  * light run 1).  Any out pointer may be NULL. */
 int kdt_tuned_params(const kdt_tree *tree, int k, int *stage_levels, int *claim_steps, int *inline_depth,

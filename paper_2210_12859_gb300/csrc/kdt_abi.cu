@@ -311,9 +311,9 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
     pool_setup_once();
     const bool morton = flags & KDT_MORTON;
     QueryArgs a;
-    a.group = list_group_for(t, k);
     a.out_ids = d_ids;
     a.visits = d_visits;
+    a.group = list_group_for(t, k, box_query_serves(a, flags, mode));  // a group list set on the tree: not by box tree
     const bool boxed = box_query_serves(a, flags, mode);
     const bool gheap = heap_in_global(t, k, boxed);
     const size_t heap_bytes = gheap ? (size_t)heap_scratch_threads() * k * 8 : 0;

@@ -363,13 +363,14 @@ int claim_steps_for(const kdt_tree *t, int k);
 int default_claim_steps_k(int k);
 int inline_depth_for(const kdt_tree *t, int k);
 int light_run_for(const kdt_tree *t, int k);
-// whether a query for k neighbours keeps its heap in global scratch; box: a
-// query by box tree, which does so only if it is set on the tree (its queries
-// are short whatever the data: clustered k = 40 2.6 ms with the shared heap, 5.2
-// with the global one), while the state machine follows the tuned choice too
+// Where the lists of a query for k > 16 neighbours live; box: a query that the
+// box tree serves.  It follows what is set on the tree and not what was tuned,
+// which is judged by the state machine's walks: its own are short whatever the
+// data (clustered k = 40 2.6 ms with the shared heap, 5.2 with the global one).
+// Whether the heap is kept in global scratch:
 bool heap_in_global(const kdt_tree *t, int k, bool box);
-// lanes per query of the shuffle-inserted group list (1: one lane per query)
-int list_group_for(const kdt_tree *t, int k);
+// lanes per query of the shuffle-inserted group list (1: one lane per query):
+int list_group_for(const kdt_tree *t, int k, bool box);
 // per-thread heap scratch for the traversal kernels (threads x k keys)
 inline int64_t heap_scratch_threads() { return (int64_t)num_sms() * 1024; }
 constexpr int SUB_CLASSES = 3;  // launches of the builder's last step, by the size of the trees (kdt_build.cu)

@@ -138,24 +138,25 @@ int light_run_for(const kdt_tree *t, int k)
     return tuned_for(t, k, &v) ? v.light_run : DEFAULT_LIGHT_RUN;
 }
 
-static int large_k_list_of(const kdt_tree *t, int k)
+// set on the tree, else, for what the state machine serves, tuned
+static int large_k_list_of(const kdt_tree *t, int k, bool box)
 {
     if (t->large_k_list >= 0)
         return t->large_k_list;
     Tuned v;
-    return tuned_for(t, k, &v) ? v.large_k_list : DEFAULT_LARGE_K_LIST;
+    return !box && tuned_for(t, k, &v) ? v.large_k_list : DEFAULT_LARGE_K_LIST;
 }
 
 bool heap_in_global(const kdt_tree *t, int k, bool box)
 {
-    return k > 16 && (box ? t->large_k_list : large_k_list_of(t, k)) == KDT_LIST_GLOBAL;
+    return k > 16 && large_k_list_of(t, k, box) == KDT_LIST_GLOBAL;
 }
 
-int list_group_for(const kdt_tree *t, int k)
+int list_group_for(const kdt_tree *t, int k, bool box)
 {
     if (k <= 16)
         return 1;
-    const int p = large_k_list_of(t, k);
+    const int p = large_k_list_of(t, k, box);
     return p == KDT_LIST_GROUP8 ? 8 : (p == KDT_LIST_GROUP4 ? 4 : 1);
 }
 
@@ -229,7 +230,7 @@ int kdt_large_k_list(const kdt_tree *t, int k, int *placement)
 {
     if (!t || k < 1 || k > 64 || !placement)
         return set_error(KDT_EINVAL, "bad tree, k or out pointer");
-    *placement = k > 16 ? large_k_list_of(t, k) : KDT_LIST_SHARED;
+    *placement = k > 16 ? large_k_list_of(t, k, true) : KDT_LIST_SHARED;
     return KDT_OK;
 }
 
