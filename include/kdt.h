@@ -512,10 +512,9 @@ int kdt_tuned_params(const kdt_tree *tree, int k, int *stage_levels, int *claim_
 /* Time the state machine on up to 2^20 of the given queries (ordered: its
  * count of processed nodes; unordered: the query) and remember
  * the fastest launch parameters for this tree's shape (GPU name, D, k bucket,
- * floor(log2 N)): a coordinate search over the inline depth {2, 1, 0}, the
- * light run {1, 4, 8}, then the claim steps {16, 32, 64, 128}, then the
- * staging depth {0, 4, 6, 8}, each
- * candidate timed over two launches after a warm-up and taken only when it is
+ * floor(log2 N)): a coordinate search over the inline depth {2, 3, 4, 1, 0}, the
+ * light run {1, 4, 8} (unordered queries; the counts take none), then the claim
+ * steps {16, 32, 64, 128}, then the staging depth {0, 4, 6, 8}, each candidate timed over two launches after a warm-up and taken only when it is
  * faster than the best so far by 2 % (staging: 5 %).  Later queries on trees of that shape use the choice unless
  * the kdt_set_* calls override.  Synchronous.  *best_levels and *best_ms (may
  * be NULL) receive the staging depth and the time of the query itself per launch;

@@ -340,10 +340,12 @@ int kdt_autotune(kdt_tree *t, const float *d_q, int64_t Q, int k, int flags, int
         if (rc == KDT_OK && (d > 0 || simple_ok))
             consider(c, 0.02f);
     }
+    // (the counts of processed nodes, by which ordered calls are judged, take no
+    // light runs: a candidate would win by noise)
     for (int lr : {4, 8}) {
         Tuned c = best;
         c.light_run = lr;
-        if (rc == KDT_OK && best.inline_depth > 0)
+        if (rc == KDT_OK && best.inline_depth > 0 && !ordered)
             consider(c, 0.02f);
     }
     for (int cs : {16, 32, 64, 128}) {

@@ -42,3 +42,15 @@ def test_tuned_placement(kdt, tmp_path, placement):
         assert torch.equal(kdt.kdt_knn(tree, q, 30)[0], want[0])
     finally:
         load(kdt.KDT_LIST_SHARED)
+
+
+def test_ordered_autotune_takes_no_light_run(kdt):
+    """Ordered calls are judged by their counts of processed nodes, whose
+    kernel has no light runs: none may be picked by noise (and then slow down
+    unordered queries)."""
+    g = torch.Generator(device="cuda").manual_seed(10)
+    q = torch.rand((2000, 3), generator=g, device="cuda")
+    tree = kdt.kdt_build(torch.rand((611, 3), generator=g, device="cuda"))
+    for _ in range(20):
+        kdt.kdt_autotune(tree, q, 3, 0)
+        assert kdt.kdt_tuned_params(tree, 3)[3] == 1
