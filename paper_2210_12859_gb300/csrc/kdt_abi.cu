@@ -348,9 +348,10 @@ int run_query(const kdt_tree *t, const float *d_q, int64_t Q, int k, float r2, i
     a.inline_depth = inline_depth_for(t, k);
     cudaEvent_t stop;
     KDT_TRY(prof_begin(const_cast<kdt_tree *>(t), s, &stop));
-    // inline depth 0: the one-node-per-step kernel, where it applies
+    // inline depth 0: the one-node-per-step kernel, where it applies (counts of
+    // ordered queries; their results are the box tree's)
     const bool simple = a.inline_depth == 0 && a.staged == 0 && !(flags & KDT_UNORDERED) && k <= 16 &&
-                        t->layout != 2 && (mode == MODE_RESULTS || mode == MODE_VISITS);
+                        t->layout != 2 && mode == MODE_VISITS;
     if (a.inline_depth == 0 && !simple)
         a.inline_depth = 1;
     if (flags & (KDT_PLAIN_STEP | KDT_CLOSE_FIRST | KDT_STACK))

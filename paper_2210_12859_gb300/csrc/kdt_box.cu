@@ -170,18 +170,14 @@ __global__ void __launch_bounds__(THREADS) box_leaf_kernel(BoxBuild a)
             dim = dim + 1 == D ? 0 : dim + 1;
         }
         const int root = (1 << sh.LB) - 1 + (int)i;
-        const int groups = (int64_t)i < sh.big ? 2 : 1;
-        float4 *g = grp + (size_t)(i + min((int64_t)i, sh.big)) * BoxFormat<NC>::GRP;
+        const int groups = sh.count(i);
+        float4 *g = grp + (size_t)sh.group(i) * BoxFormat<NC>::GRP;
         for (int k = 0; k < groups; ++k, g += BoxFormat<NC>::GRP) {
             float c[NC][BOX_GROUP];
             uint32_t id[BOX_GROUP];
 #pragma unroll
             for (int m = 0; m < BOX_GROUP; ++m) {
-                // place m of the first group: node 0 .. 6 of the bucket's
-                // first three levels, then the one from above; of the second:
-                // the fourth level's nodes
-                const int up = k ? 3 : (m < 1 ? 0 : (m < 3 ? 1 : 2));
-                const int node = ((root + 1) << up) - 1 + (k ? m : m + 1 - (1 << up));
+                const int node = bucket_node(root, k, m);
                 const bool above = k == 0 && m == 7;
                 const bool ok = above ? held : node < N;
                 if (!above && ok) {

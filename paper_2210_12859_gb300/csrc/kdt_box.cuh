@@ -66,7 +66,19 @@ struct BoxShape {
     }
     __host__ __device__ __forceinline__ int64_t records() const { return LB ? buckets / 2 : 0; }
     __host__ __device__ __forceinline__ int64_t groups() const { return buckets + big; }
+    // first group of bucket i, and how many it has
+    __host__ __device__ __forceinline__ int64_t group(int64_t i) const { return i + (i < big ? i : big); }
+    __host__ __device__ __forceinline__ int count(int64_t i) const { return i < big ? 2 : 1; }
 };
+
+// Node at place m of a bucket's group k, root: the bucket's (m = 7 of the first
+// group holds the point from above instead).  First group: the seven nodes of the
+// bucket's first three levels; second: the eight of its fourth.
+__host__ __device__ __forceinline__ int bucket_node(int root, int k, int m)
+{
+    const int up = k ? 3 : (m < 1 ? 0 : (m < 3 ? 1 : 2));
+    return ((root + 1) << up) - 1 + (k ? m : m + 1 - (1 << up));
+}
 
 // Two FP32 values in one 64-bit register: sm_103a adds and multiplies such
 // pairs in one instruction, each half rounded like the single operation.
