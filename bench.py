@@ -3,7 +3,7 @@
 Workload (default): N = 2^24 3-D points from a 64-component isotropic Gaussian
 mixture (sigma 0.01, centres uniform in [0,1]^3), Q = 2^24 queries (90% from
 the mixture, 10% uniform in [0,1]^3); kNN with k = 8, unbounded radius,
-ordered stack-free traversal with Morton query order.  One step = rebuild the
+ordered queries by subtree boxes in the order of their descent paths.  One step = rebuild the
 tree from the points + answer all Q queries (every stage of the single-tree
 hot path).  The learned-radius form of the same query is timed beside it.
 
@@ -445,7 +445,7 @@ def main():
                    "roofline": {"bound": "hbm", "achieved": l_ach, "peak": hbm, "unit": "GB/s", "frac": l_ach / hbm,
                                 "bytes_per_query": l_bytes / n, "peak_source": peak_src,
                                 "l2": {"peak": l2_gbs, "frac": l_ach / l2_gbs, "peak_source": l2_note},
-                                "time": "whole learned call (Morton pass, features and network for the gated "
+                                "time": "whole learned call (query order, features and network for the gated "
                                         "queries, bounded traversal)"}}
 
     # ---- the same queries on a tree with a stored per-node split dimension

@@ -2,9 +2,13 @@
  * kdt.h - C ABI of the GB300 k-d tree query library.
  *
  * Find-closest-point (fcp) and k-nearest-neighbour (kNN) queries over a
- * left-balanced, complete k-d tree stored in level order, traversed with the
- * stack-free (curr, prev) state machine of Wald, "A Stack-Free Traversal
- * Algorithm for Left-Balanced k-d Trees" (arXiv 2210.12859), Sec. 3.
+ * left-balanced, complete k-d tree stored in level order, as in Wald, "A
+ * Stack-Free Traversal Algorithm for Left-Balanced k-d Trees" (arXiv
+ * 2210.12859).  Unordered queries, counts of processed nodes and the traversal
+ * ablations run the paper's stack-free (curr, prev) state machine (Sec. 3).
+ * Ordered queries for results and range queries give what the machine gives
+ * and find it in a box tree (the bounding boxes of subtrees) that every build
+ * makes beside the level-order tree.
  *
  * Conventions shared by every entry point:
  *   - Pointers prefixed d_ are DEVICE pointers on the current CUDA device,
@@ -58,7 +62,8 @@ extern "C" {
 #define KDT_LEARNED    0x4 /* seed each query's cull radius with the trained radius model
                               and re-run the queries that find fewer than k points with
                               the caller's radius (not in the paper; results unchanged) */
-#define KDT_NO_STAGE   0x8 /* do not stage the top tree levels in shared memory */
+#define KDT_NO_STAGE   0x8 /* do not stage the top tree levels in shared memory (the state
+                              machine's kernels; ordered results never do) */
 #define KDT_COST_ORDER 0x20 /* with KDT_MORTON, single trees with D <= 3: run the queries in cost
                               classes, most expensive first (judged by how far the greedy
                               descent ends from its leaf point, relative to the mean point
@@ -108,7 +113,11 @@ int64_t kdt_launch_count(void);
  * builder produces (Sec. 4).
  *   d_points: float32 [N][D], read only during the call's stream work.
  *   N in [1, 2^30), D in [1, 8].
- *   *out receives a library-owned tree; release it with kdt_free.
+ *   *out receives a library-owned tree; release it with kdt_free.  With its box
+ *   tree it takes 35 to 38 bytes of device memory a point for D <= 3, 44 to 48 for
+ *   D = 4 and 80 to 88 above (the level-order arrays alone: 16, 20 and 36); the
+ *   build's scratch, returned to the stream-ordered pool, is about 4 (D + 5) bytes
+ *   a point more.
  * Synchronises `stream` once to report KDT_ENONFINITE. */
 int kdt_build(const float *d_points, int64_t N, int D, void *stream, kdt_tree **out);
 
@@ -165,7 +174,7 @@ int kdt_knn_visits(const kdt_tree *tree, const float *d_queries, int64_t Q, int 
  * Every point within a radius of a query point (ball, inclusive, the same FP32
  * squared distance as kdt_knn: d2 <= fl(radius * radius)) or inside an
  * axis-aligned box (inclusive bounds; lo > hi in any dimension gives none),
- * found with the unordered stack-free traversal and a fixed range (Sec. 3:
+ * with a fixed range, in the order of the unordered stack-free traversal (Sec. 3:
  * other query primitives change only the range test and processNode).
  * Queries float [Q][D] (ball centres, box lower / upper corners), device.
  * Two passes: *_count writes d_counts int32 [Q]; kdt_offsets turns counts into
@@ -246,7 +255,7 @@ int kdt_knn_host(const float *h_points, int64_t N, int D, const float *h_queries
  * (an application whose own pool owns all device memory, a real-time loop
  * that cannot afford the synchronisation of cudaMalloc / cudaFree, a plugin
  * host that forbids library allocations).  Scratch lives in one fixed device
- * array inside the library (about 4.3 MB per GPU that loads it, held until the
+ * array inside the library (about 6.3 MB per GPU that loads it, held until the
  * process exits), so Q is limited to KDT_STATIC_MAX_Q per call; larger Q gives
  * KDT_EINVAL.  KDT_LEARNED is not accepted.  Same arguments, results and
  * flags as kdt_knn otherwise.
@@ -390,8 +399,8 @@ int kdt_build_batched(const float *d_points, const int64_t *h_offsets, int T, in
  * same arguments come a second time, and replayed from the third on while they are
  * unchanged).  In a capture of the caller's the call takes its offsets by value, so
  * that h_qoffsets need not outlive it; the first call of a forest, and one that needs
- * more scratch than those before, allocates and cannot be captured.  With KDT_PER_TREE the same kernel is launched once per tree
- * instead (for comparison). */
+ * more scratch than those before, allocates and cannot be captured.  With
+ * KDT_PER_TREE the same kernel is launched once per tree instead (for comparison). */
 #define KDT_PER_TREE 0x10
 int kdt_knn_batched(kdt_forest *forest, const float *d_queries, const int64_t *h_qoffsets,
                     int k, float max_radius, int flags, int32_t *d_ids, float *d_d2, void *stream);

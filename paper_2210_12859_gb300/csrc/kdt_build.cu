@@ -41,7 +41,7 @@ enum : uint8_t { SIDE_LEFT = 0, SIDE_NODE = 1, SIDE_RIGHT = 2 };
 
 // Largest subtree that one block builds in shared memory.  Large builds take
 // the largest that leaves two blocks on an SM, since every level above costs a
-// pass over all lists (2^24 points: 0.42 ms a level); small ones, which fill few
+// pass over all lists (2^24 points: 0.31 ms a level); small ones, which fill few
 // SMs either way and whose blocks are bound by instruction issue, a smaller one.
 constexpr int SUB_LOG2_LARGE = 12, SUB_LOG2_SMALL = 10;
 constexpr int64_t SUB_SMALL_TOTAL = (int64_t)1 << 18;

@@ -278,7 +278,7 @@ int check_learned_tree(const kdt_tree *t)
 }
 
 // queries of the last learned call that took the proposal (counted: the far
-// queries the Morton pass counted, for KDT_GATE_FAR)
+// queries that the query order counted, for KDT_GATE_FAR)
 int64_t learned_gated(const kdt_tree *t, int64_t counted)
 {
     switch (t->last_learned_gate) {
@@ -321,8 +321,8 @@ int run_learned_query(kdt_tree *t, const float *d_q, int64_t Q, int k, float r2,
     if (gate == KDT_GATE_NONE)  // the proposal pays on none of these queries: the plain traversal
         return run_query(t, d_q, Q, k, r2, flags & ~KDT_LEARNED, d_ids ? MODE_RESULTS : MODE_VISITS, d_ids, d_d2,
                          d_visits, s);
-    // far queries only: their cost classes come first in the traversal order,
-    // and the Morton pass counts them
+    // far queries only: their cost classes come first in the query order, whose
+    // keys count them
     if (gate == KDT_GATE_FAR)
         flags |= KDT_MORTON | KDT_COST_ORDER;
     const bool morton = flags & KDT_MORTON;

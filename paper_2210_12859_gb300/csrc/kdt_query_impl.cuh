@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(K <= MAX_REG_K ? REG_THREADS : SMEM_THREADS, K
         // the proposed radius is farther than all k held) or when the proposal
         // did not shrink the caller's radius; the others restart at once in the
         // same lane with the caller's radius (the plain traversal): no second
-        // launch, and the re-run stays next to its Morton neighbours
+        // launch, and the re-run stays next to its neighbours in the query order
         const bool fallback = MODE == MODE_BOUNDED && !(full || r2 == a.r2);
         if (fallback) {
             atomicAdd(a.fb_count, 1ull);

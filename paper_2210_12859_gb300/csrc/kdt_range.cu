@@ -12,9 +12,9 @@
 //     ACT_COUNT   count the hits;
 //     ACT_FILL    write the hits to the query's slice [offsets[q], offsets[q+1])
 //                 in traversal order (count and fill walk the same nodes in
-//                 the same order, so no atomics are needed); hits from the
-//                 first 16-byte boundary of the slice on are collected four at
-//                 a time in registers and written as 16-byte stores, the
+//                 the same order, so no atomics are needed); hits wait in a
+//                 ring in shared memory, and from the slice's first 16-byte
+//                 boundary on are written four at a time as 16-byte stores, the
 //                 slice's unaligned head and its last partial group one word
 //                 at a time;
 //     ACT_REDUCE  sum a per-point payload over the hits in traversal order

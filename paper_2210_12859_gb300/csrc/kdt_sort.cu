@@ -145,7 +145,7 @@ int exclusive_scan_t(T *data, int64_t n, T *scratch, cudaStream_t s)
 // Bound: memory, 16 bytes a pair and pass, for large sorts; the latency of a
 // pass's chain (load, rank, look-back, write) for small ones.  Against the
 // passes it replaced (a histogram kernel, three scan kernels and a scatter
-// that wrote every pair by itself, 20 launches a sort), the Morton order of
+// that wrote every pair by itself, 20 launches a sort), the order of
 // 10^7 queries takes 0.54 ms instead of 0.85 and that of 2^14 queries 43 us
 // instead of 115.
 

@@ -6,7 +6,7 @@
 // the implicit synchronisation of cudaMalloc / cudaFree would stall other
 // work; a plugin whose host forbids device allocations from inside a frame.
 // For them this entry point keeps its scratch (the warp work counter and the
-// Morton keys, permutation and radix-sort temporaries) in one file-scope
+// order keys, permutation and radix-sort temporaries) in one file-scope
 // device array of fixed size instead of allocating it per call.  The array
 // lives in every GPU that loads the library until the process exits.
 //
@@ -24,7 +24,7 @@ namespace {
 
 constexpr int64_t STATIC_MAX_Q = KDT_STATIC_MAX_Q;
 constexpr size_t STATIC_COUNTER_BYTES = 256;
-// the work counter block, then the Morton keys, permutation and radix-sort
+// the work counter block, then the order keys, permutation and radix-sort
 // temporaries of the largest call (the same formula run_query sizes its
 // scratch with, evaluated at compile time)
 constexpr size_t STATIC_BYTES = STATIC_COUNTER_BYTES + morton_scratch_bytes_of(STATIC_MAX_Q);
